@@ -378,8 +378,8 @@ def run_steady(args, wl):
         return
     secs = ms / 1e3
     value = faces_cycle * ncyc * args.steps * world / secs
-    fo_face = sum(gks.face_op_count(2, False, False)[:3])
-    so_face = sum(gks.face_op_count(2, False, True)[:3])
+    fo_face = sum(gks.face_op_count(2, False, False, closed_form=True)[:3])
+    so_face = sum(gks.face_op_count(2, False, True, closed_form=True)[:3])
     per_cell = CELL_OPS + sum(gks.cell_op_count(2)[:3])
     ops_cycle = sum(e * (f * (so_face if l == 0 else fo_face) + c * per_cell) for l, (f, c, e) in enumerate(per_level))
     if transport:  # the k-omega update of the finest grid
@@ -568,10 +568,12 @@ def run_ours(args):
         return
     secs = ms / 1e3
     value = faces_per_step * nsteps * args.steps * world / secs
-    # roofline of the fused step kernel (ALU bound): algorithmic operations per launch
+    # roofline of the fused step kernel (ALU bound): operations per launch of the closed-form flux that the
+    # kernel evaluates (the moment-table form of the same flux is reported beside it)
     multid = wl["kw"].get("expand") == "multid" and D > 1
-    counts = gks.face_op_count(D, multid, args.reconstruction == "muscl2")
-    per_face = sum(counts[:3]) + sum(gks.recon_op_count(D, args.reconstruction)[:3])
+    recon_ops = sum(gks.recon_op_count(D, args.reconstruction)[:3])
+    per_face, table_ops = (sum(gks.face_op_count(D, multid, args.reconstruction == "muscl2", closed_form=c)[:3])
+                           + recon_ops for c in (True, False))
     per_cell = CELL_OPS + sum(gks.cell_op_count(D)[:3]) + (KOMEGA_CELL_OPS[D] if transport else 0)
     ops_per_launch = faces_per_step * per_face + cells * per_cell
     avg_launch_s = kms / 1e3 / max(klaunch, 1)
@@ -626,6 +628,7 @@ def run_ours(args):
                                                                          if transport else "")),
                      "avg_launch_us": avg_launch_s * 1e6,
                      "ops_per_face": per_face, "ops_per_cell": per_cell,
+                     "moment_table_ops_per_face": table_ops,
                      "peak_basis": "152 SMs x %d %s lanes x 2 (FMA) x 2070 MHz (derived)" % (lanes, "FP64" if fp64
                                                                                             else "FP32")},
         # per bench step: state_in + rate kernels, one step kernel per time step (plus, with k-omega

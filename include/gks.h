@@ -359,10 +359,12 @@ gks_status gks_face_flux(int dim, int precision, int expand, int abar_mode, int 
                          double mu, double C_a, double dt, const double* faces, long nfaces, double* F_out,
                          double* tau_out, void* cuda_stream);
 
-/* Operation count of one interface flux (Eq. fluxesf) as the device code is written (no GPU needed): counts[0..5]
+/* Operation count of one interface flux (Eq. fluxesf; no GPU needed): counts[0..5]
  * = additions/subtractions, multiplications, divisions, square roots, exponentials, erfc.
- * with_recon adds the face values of the MUSCL reconstruction from the cell slopes.  Operations on
- * literal 0 or 1 are not counted.  Used to state the algorithmic FLOPs behind the roofline figures. */
+ * with_recon: bit 0 adds the face values of the MUSCL reconstruction from the cell slopes; bit 1 counts
+ * the closed form that the device code evaluates, otherwise the moment-table form of the same flux (a
+ * fixed unit of work that throughput can be compared in).  Operations on literal 0 or 1 are not
+ * counted.  Used to state the FLOPs behind the roofline figures. */
 int gks_face_op_count(int dim, int expand, int with_recon, long long* counts);
 /* The same count for the per-cell part of the reconstruction (Section 4): the limited (van Leer) slope of every
  * variable along every axis, computed once per cell and step. */

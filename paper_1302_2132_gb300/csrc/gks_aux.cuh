@@ -104,10 +104,10 @@ __global__ void __launch_bounds__(kThreads) rate_kernel(const __grid_constant__ 
     pos[0] = (int)(c % g.n[0]);
     pos[1] = (int)((c / g.n[0]) % g.n[1]);
     pos[2] = (int)(c / ((long)g.n[0] * g.n[1]));
-    R h[D];
-    for (int d = 0; d < D; ++d) h[d] = (R)g.w[d][pos[d] + kWG];
+    R ih[D];
+    for (int d = 0; d < D; ++d) ih[d] = g_rcp((R)g.w[d][pos[d] + kWG]);
     if (!(w[0] > R(0)) || !(pressure_of<R>(D, kc.gamma, w) > R(0))) bad = 1;
-    rmax = fmax(rmax, cell_rate<D, R>(w, kc.gamma, h));
+    rmax = fmax(rmax, cell_rate_inv<D, R>(w, kc.gamma, ih));
   }
   const double m = block_max<double>((double)rmax, red);
   if (threadIdx.x == 0) atomic_max_nonneg(&A.ctrl->rate[A.slot], m);

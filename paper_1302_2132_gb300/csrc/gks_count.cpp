@@ -1,5 +1,5 @@
-// Static operation count of the interface flux: the device flux code of gks_flux.cuh is compiled
-// for the host with a scalar type that counts every arithmetic operation it performs.  Operations
+// Static operation count of the interface flux: the device flux code of gks_flux.cuh (and the
+// moment-table form of the same flux, gks_flux_tables.h) is compiled for the host with a scalar type that counts every arithmetic operation it performs.  Operations
 // whose operand is a literal 0 or 1 are not counted (the compiler removes them), so the count is
 // that of the algorithm as written.  Used for the algorithmic FLOP figure of the roofline.
 #define GKS_HOST_COUNT 1
@@ -11,6 +11,7 @@ namespace gks {
 struct Cnt;
 }
 #include "gks_flux.cuh"
+#include "gks_flux_tables.h"
 
 namespace gks {
 
@@ -83,7 +84,7 @@ template <> inline Cnt g_erfc<Cnt>(Cnt x) {
 }
 
 template <int D, bool M>
-static void count_face(int with_recon, Ops* out) {
+static void count_face(bool with_recon, bool closed_form, Ops* out) {
   constexpr int nv = D + 2;
   g_ops = Ops{0, 0, 0, 0, 0, 0};
   // a representative face: distinct positive states, dt/tau > 1 (the closed-form time branch)
@@ -117,8 +118,13 @@ static void count_face(int with_recon, Ops* out) {
   gas.mu = Cnt::run(1e-5);
   gas.C_a = Cnt::run(0.0);
   Cnt F[nv], tau;
-  face_flux<D, Cnt, M>(wl, wr, cl, cr, sl, sr, tl, tr, Cnt::run(0.005), Cnt::run(0.005), Cnt::run(1e-5),
-                       Cnt::run(1e-3), gas, 0, F, &tau);
+  const FaceArrays<D, Cnt> in{sl, sr, cl, cr, tl, tr};
+  if (closed_form)
+    face_flux_in<D, Cnt, M>(wl, wr, in, Cnt::run(200.0), Cnt::run(200.0), Cnt::run(1e-5), Cnt::run(1e-3), gas, 0, F,
+                            &tau);
+  else
+    tables::face_flux_in<D, Cnt, M>(wl, wr, in, Cnt::run(0.005), Cnt::run(0.005), Cnt::run(1e-5), Cnt::run(1e-3), gas,
+                                    0, F, &tau);
   *out = g_ops;
 }
 
@@ -207,15 +213,15 @@ extern "C" int gks_cell_op_count(int dim, long long* counts) {
 extern "C" int gks_face_op_count(int dim, int expand, int with_recon, long long* counts) {
   gks::Ops o{0, 0, 0, 0, 0, 0};
   if (dim == 1)
-    gks::count_face<1, false>(with_recon, &o);
+    gks::count_face<1, false>(with_recon & 1, with_recon & 2, &o);
   else if (dim == 2 && expand)
-    gks::count_face<2, true>(with_recon, &o);
+    gks::count_face<2, true>(with_recon & 1, with_recon & 2, &o);
   else if (dim == 2)
-    gks::count_face<2, false>(with_recon, &o);
+    gks::count_face<2, false>(with_recon & 1, with_recon & 2, &o);
   else if (dim == 3 && expand)
-    gks::count_face<3, true>(with_recon, &o);
+    gks::count_face<3, true>(with_recon & 1, with_recon & 2, &o);
   else if (dim == 3)
-    gks::count_face<3, false>(with_recon, &o);
+    gks::count_face<3, false>(with_recon & 1, with_recon & 2, &o);
   else
     return 1;
   counts[0] = o.add;

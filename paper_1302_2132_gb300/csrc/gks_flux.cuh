@@ -5,9 +5,16 @@
 // 1..D-1 the tangential directions (v, w).  Moments <.> are normalised by rho.  The Maxwellian of a
 // state has lambda = rho/(2p) and K = bK - D internal degrees of freedom (bK = 2/(gamma-1)).
 //
-// The moment algebra is hand-expanded: half-line moments of u from erfc/exp (Eq. intermediatestate),
-// tangential moments from the Gaussian recursion, slope coefficients from the closed-form
-// inverse of the moment matrix, and the time integral of Eq. resultingf via T0..T5.
+// The moments are taken in closed form.  A slope a . psi of a Maxwellian is the derivative of its
+// logarithm, r + c.U'/theta + theta'/(2 theta^2) (c^2 + xi^2 - bK theta), with the peculiar velocity c, theta =
+// 1/(2 lambda) = p/rho and the gradients (r = rho'/rho, U', theta') of the macroscopic variables.  The time slope A is
+// then the Euler equations' time derivative, the full-line moments are the Navier-Stokes fluxes of those
+// gradients, and the transverse velocities average out of a half-line moment before it is taken: what
+// is left on a half line are one cubic and one quadratic polynomial in the normal velocity.  889
+// operations per 2D multi-dimensional face and 1192 in 3D (moment tables: 1674 and 2767).  The kernels are bound
+// by their instruction count, in single precision (issue and FP32 pipe about 58% busy) and in double (FP64 pipe 88%
+// busy), so the step times follow: 1024^2 with the double state 122 -> 98 us, 512^2 in FP64 1.88 -> 1.33 ms, 160^3
+// 1.59 -> 1.11 ms.
 #pragma once
 #ifndef GKS_HOST_COUNT
 #include <cuda_runtime.h>
@@ -59,6 +66,20 @@ template <class T> GKS_FN T g_abs(T x) { return x < T(0) ? -x : x; }
 #ifndef GKS_HOST_COUNT
 template <> GKS_FN float g_abs<float>(float x) { return fabsf(x); }
 template <> GKS_FN double g_abs<double>(double x) { return fabs(x); }
+#endif
+
+// Products, sums and fused multiply-adds that are rounded as written (never contracted with their
+// neighbours), for values that two kernels have to agree on to the last bit.
+template <class T> GKS_FN T g_mul_rn(T a, T b) { return a * b; }
+template <class T> GKS_FN T g_add_rn(T a, T b) { return a + b; }
+template <class T> GKS_FN T g_fma_rn(T a, T b, T c) { return a * b + c; }
+#ifndef GKS_HOST_COUNT
+template <> GKS_FN float g_mul_rn<float>(float a, float b) { return __fmul_rn(a, b); }
+template <> GKS_FN double g_mul_rn<double>(double a, double b) { return __dmul_rn(a, b); }
+template <> GKS_FN float g_add_rn<float>(float a, float b) { return __fadd_rn(a, b); }
+template <> GKS_FN double g_add_rn<double>(double a, double b) { return __dadd_rn(a, b); }
+template <> GKS_FN float g_fma_rn<float>(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+template <> GKS_FN double g_fma_rn<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
 #endif
 
 // Quotient and reciprocal: IEEE in double precision (the FP64 path matches the oracle to 1e-12);
@@ -127,8 +148,8 @@ template <int D> struct Dims {
 
 // Macroscopic description of one Maxwellian.
 template <int D, class T> struct Maxw {
-  T rho, ir, U[D], lam, il;  // ir = 1/rho, il = 1/(2 lambda)
-  T c, f4;               // |U|^2 + bK il and 4 lambda^2 / bK (used by every slope solve)
+  T rho, ir, U[D];  // ir = 1/rho
+  T th, it;         // theta = 1/(2 lambda) = p/rho, and 1/theta
 };
 
 // Gas constants used by every face.
@@ -140,11 +161,10 @@ template <class T> struct Gas {
   T C_a;  // artificial-dissipation coefficient (Eq. taua)
 };
 
-// (rho, U, lambda) of the Maxwellian carrying the conservative state w (Section 2: E = (u^2 + xi^2)/2,
-// so rho E = rho |U|^2 / 2 + bK rho / (4 lambda)).  Two reciprocals: 1/rho, and 1/(2 lambda) =
-// (2 rho E - rho |U|^2) / (bK rho) is a product, lambda its reciprocal; ibK = 1/bK.
+// (rho, U, theta) of the Maxwellian carrying the conservative state w (Section 2: E = (u^2 + xi^2)/2,
+// so rho E = rho (|U|^2 + bK theta) / 2).  Two reciprocals: 1/rho and 1/theta; ibK = 1/bK.
 template <int D, class T>
-GKS_FN Maxw<D, T> maxwellian(const T* w, T bK, T ibK) {
+GKS_FN Maxw<D, T> maxwellian(const T* w, T ibK) {
   Maxw<D, T> g;
   g.rho = w[0];
   g.ir = g_rcp(w[0]);
@@ -154,197 +174,75 @@ GKS_FN Maxw<D, T> maxwellian(const T* w, T bK, T ibK) {
     g.U[i] = w[1 + i] * g.ir;
     q += g.U[i] * g.U[i];
   }
-  g.il = (T(2) * w[D + 1] - w[0] * q) * g.ir * ibK;
-  g.lam = T(0.5) * g_rcp(g.il);
-  g.c = q + bK * g.il;
-  g.f4 = T(4) * g.lam * g.lam * ibK;
+  g.th = (T(2) * w[D + 1] - w[0] * q) * g.ir * ibK;
+  g.it = g_rcp(g.th);
   return g;
 }
 
-// Moments of one Maxwellian, split into the normal velocity u and the transverse part.
-//
-// Every polynomial the flux needs is linear in the transverse basis {1, v_s, Et}, with
-// Et = (sum_s v_s^2 + xi^2)/2 (so psi_E = u^2/2 + Et), and has polynomial coefficients in u.  Under
-// the Maxwellian u, the v_s and xi are independent, so a moment factors into a moment of u over the
-// chosen half line and a transverse moment over the full space.  The transverse moments of products
-// of up to three basis functions are tabulated once per Maxwellian.
-template <int D> struct Basis {
-  static constexpr int NB = D + 1;  // 0: 1, 1..D-1: v_s, D: Et
+// n eta_n = n <(u - U)^k>, k = 0..6, over u > 0 (sgn = +1) or u < 0 (sgn = -1), from the textbook half-line
+// Gaussian integrals: <1> = erfc(-sgn U/sqrt(2 theta))/2, <u - U> = sgn sqrt(theta/(2 pi)) exp(-U^2/(2 theta)) =: b,
+// and by parts <(u - U)^(k+2)> = (k + 1) theta <(u - U)^k> + (-U)^(k+1) b.
+template <int D, class T>
+GKS_FN void half_moments(const Maxw<D, T>& g, T sgn, T n, T* e) {
+  const T s2 = g_sqrt(T(2) * g.th);
+  const T z = T(0.5) * g.U[0] * s2 * g.it;
+  e[0] = T(0.5) * n * g_erfc(-sgn * z);
+  e[1] = sgn * T(0.5 * kInvSqrtPi) * n * s2 * g_exp(-z * z);
+  T b = e[1];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    b = -g.U[0] * b;
+    e[k + 2] = T(k + 1) * g.th * e[k] + b;
+  }
+}
+
+// Gradients of the macroscopic variables along one direction.
+template <int D, class T> struct Grad {
+  T r, U[D], th;  // rho'/rho, U', theta'
 };
-
-template <int D, class T> struct Trans {
-  T m1[D + 1];                     // <beta>
-  T m2[D + 1][D + 1];              // <alpha beta>
-  T m3[Dims<D>::nt][D + 1][D + 1];  // <v_s alpha beta>
-};
-
-// Gaussian moments <x^n>, n = 0..N-1, of mean U and variance il: x^{n+2} = U x^{n+1} + (n+1) il x^n.
-template <int N, class T>
-GKS_FN void recur(T U, T il, T* m) {
-#pragma unroll
-  for (int n = 0; n + 2 < N; ++n) m[n + 2] = U * m[n + 1] + T(n + 1) * il * m[n];
-}
-
+// ... from r = W'/rho: W_E' = (rho (|U|^2 + bK theta)/2)'.
 template <int D, class T>
-GKS_FN void transverse(const Maxw<D, T>& g, T K, Trans<D, T>& t) {
-  const T X1 = K * g.il;                        // <xi^2>
-  const T X2 = K * (K + T(2)) * g.il * g.il;    // <xi^4>
-  T V[Dims<D>::nt][6];
+GKS_FN void gradient(const Maxw<D, T>& g, T bK, T ibK, const T* r, Grad<D, T>& o) {
+  T c = bK * g.th, UU = T(0);
 #pragma unroll
-  for (int s = 0; s < D - 1; ++s) {
-    V[s][0] = T(1);
-    V[s][1] = g.U[1 + s];
-    recur<6>(g.U[1 + s], g.il, V[s]);
+  for (int i = 0; i < D; ++i) {
+    c += g.U[i] * g.U[i];
+    o.U[i] = r[1 + i] - g.U[i] * r[0];
+    UU += g.U[i] * o.U[i];
   }
-  t.m1[0] = T(1);
+  o.r = r[0];
+  o.th = (T(2) * (r[D + 1] - UU) - c * r[0]) * ibK;
+}
+
+// Minus the Euler time derivatives of (r, U, theta) from the gradients along the normal (gx) and the
+// tangential axes (gs, multi-dimensional expansion only): convection, dilatation and pressure.  This is
+// -A of the compatibility condition <(a u + b v + A) psi> = 0 (Eq. initialf0).
+template <int D, class T, bool MULTID>
+GKS_FN void euler_rate(const Maxw<D, T>& g, T ibK, const Grad<D, T>& gx, const Grad<D, T>* gs, T& S, T& div,
+                       Grad<D, T>& N) {
+  S = T(0);  // sum of the tangential dilatations
+  div = gx.U[0];
+  if (MULTID) {
 #pragma unroll
-  for (int b = 0; b <= D; ++b) t.m2[0][b] = T(0);
-  if (D == 1) {
-    // basis {1, Et}, Et = xi^2 / 2
-    t.m1[1] = T(0.5) * X1;
-    t.m2[0][0] = T(1);
-    t.m2[0][1] = t.m2[1][0] = t.m1[1];
-    t.m2[1][1] = T(0.25) * X2;
-  } else if (D == 2) {
-    // basis {1, v, Et}, Et = (v^2 + xi^2)/2
-    const T* v = V[0];
-    const T e1 = v[2] + X1;                          // <2 Et>
-    const T ve = v[3] + v[1] * X1;                   // <v 2 Et>
-    const T vve = v[4] + v[2] * X1;                  // <v^2 2 Et>
-    const T ee = v[4] + T(2) * v[2] * X1 + X2;       // <(2 Et)^2>
-    const T vee = v[5] + T(2) * v[3] * X1 + v[1] * X2;  // <v (2 Et)^2>
-    t.m1[1] = v[1];
-    t.m1[2] = T(0.5) * e1;
-    t.m2[0][0] = T(1);
-    t.m2[0][1] = t.m2[1][0] = v[1];
-    t.m2[0][2] = t.m2[2][0] = t.m1[2];
-    t.m2[1][1] = v[2];
-    t.m2[1][2] = t.m2[2][1] = T(0.5) * ve;
-    t.m2[2][2] = T(0.25) * ee;
-    // <v alpha beta>
-    t.m3[0][0][0] = v[1];
-    t.m3[0][0][1] = t.m3[0][1][0] = v[2];
-    t.m3[0][0][2] = t.m3[0][2][0] = t.m2[1][2];
-    t.m3[0][1][1] = v[3];
-    t.m3[0][1][2] = t.m3[0][2][1] = T(0.5) * vve;
-    t.m3[0][2][2] = T(0.25) * vee;
-  } else {
-    // basis {1, v, w, Et}, Et = (v^2 + w^2 + xi^2)/2
-    const T* v = V[0];
-    const T* w = V[Dims<D>::nt - 1];
-    const T rv1 = w[2] + X1, rv2 = w[4] + T(2) * w[2] * X1 + X2;  // moments of 2Et - v^2
-    const T rw1 = v[2] + X1, rw2 = v[4] + T(2) * v[2] * X1 + X2;  // moments of 2Et - w^2
-    const T e1 = v[2] + rv1;
-    const T ee = v[4] + T(2) * v[2] * rv1 + rv2;
-    t.m1[1] = v[1];
-    t.m1[2] = w[1];
-    t.m1[3] = T(0.5) * e1;
-    t.m2[0][0] = T(1);
-#pragma unroll
-    for (int b = 1; b <= 3; ++b) t.m2[0][b] = t.m2[b][0] = t.m1[b];
-    t.m2[1][1] = v[2];
-    t.m2[1][2] = t.m2[2][1] = v[1] * w[1];
-    t.m2[2][2] = w[2];
-    t.m2[1][3] = t.m2[3][1] = T(0.5) * (v[3] + v[1] * rv1);
-    t.m2[2][3] = t.m2[3][2] = T(0.5) * (w[3] + w[1] * rw1);
-    t.m2[3][3] = T(0.25) * ee;
-    const T vwe = T(0.5) * (v[3] * w[1] + v[1] * w[3] + v[1] * w[1] * X1);  // <v w Et>
-    // gamma = v
-    t.m3[0][0][0] = v[1];
-    t.m3[0][0][1] = t.m3[0][1][0] = v[2];
-    t.m3[0][0][2] = t.m3[0][2][0] = t.m2[1][2];
-    t.m3[0][0][3] = t.m3[0][3][0] = t.m2[1][3];
-    t.m3[0][1][1] = v[3];
-    t.m3[0][1][2] = t.m3[0][2][1] = v[2] * w[1];
-    t.m3[0][2][2] = v[1] * w[2];
-    t.m3[0][1][3] = t.m3[0][3][1] = T(0.5) * (v[4] + v[2] * rv1);
-    t.m3[0][2][3] = t.m3[0][3][2] = vwe;
-    t.m3[0][3][3] = T(0.25) * (v[5] + T(2) * v[3] * rv1 + v[1] * rv2);
-    // gamma = w
-    t.m3[1][0][0] = w[1];
-    t.m3[1][0][1] = t.m3[1][1][0] = t.m2[1][2];
-    t.m3[1][0][2] = t.m3[1][2][0] = w[2];
-    t.m3[1][0][3] = t.m3[1][3][0] = t.m2[2][3];
-    t.m3[1][1][1] = v[2] * w[1];
-    t.m3[1][1][2] = t.m3[1][2][1] = v[1] * w[2];
-    t.m3[1][2][2] = w[3];
-    t.m3[1][1][3] = t.m3[1][3][1] = vwe;
-    t.m3[1][2][3] = t.m3[1][3][2] = T(0.5) * (w[4] + w[2] * rw1);
-    t.m3[1][3][3] = T(0.25) * (w[5] + T(2) * w[3] * rw1 + w[1] * rw2);
+    for (int q = 0; q < D - 1; ++q) S += gs[q].U[1 + q];
+    div = gx.U[0] + S;
   }
-}
-
-// <beta> for the transverse basis {1, v_s, Et} (the first row of the transverse table).
-template <int D, class T>
-GKS_FN void trans_mean(const Maxw<D, T>& g, T K, T* m1) {
-  T e = K * g.il;  // <xi^2>
+  N.r = g.U[0] * gx.r + div;
+  N.U[0] = g.U[0] * gx.U[0] + (g.th * gx.r + gx.th);
+  N.th = g.U[0] * gx.th + T(2) * ibK * (g.th * div);
 #pragma unroll
-  for (int s = 0; s < D - 1; ++s) {
-    m1[1 + s] = g.U[1 + s];
-    e += g.U[1 + s] * g.U[1 + s] + g.il;  // <v_s^2>
+  for (int i = 1; i < D; ++i) N.U[i] = g.U[0] * gx.U[i];
+  if (MULTID) {
+#pragma unroll
+    for (int q = 0; q < D - 1; ++q) {
+      const T V = g.U[1 + q];
+      N.r += V * gs[q].r;
+      N.th += V * gs[q].th;
+#pragma unroll
+      for (int i = 0; i < D; ++i) N.U[i] += V * gs[q].U[i];
+      N.U[1 + q] += g.th * gs[q].r + gs[q].th;
+    }
   }
-  m1[0] = T(1);
-  m1[D] = T(0.5) * e;
-}
-
-// <u^n>, n = 0..6, over the full line.
-template <int D, class T>
-GKS_FN void u_full(const Maxw<D, T>& g, T* u) {
-  u[0] = T(1);
-  u[1] = g.U[0];
-  recur<7>(g.U[0], g.il, u);
-}
-
-// <u^n> over u > 0 (sgn = +1) or u < 0 (sgn = -1), from the textbook half-line Gaussian integrals
-//   <1>_{u>0} = erfc(-sqrt(lam) U)/2,  <u>_{u>0} = U <1>_{u>0} + exp(-lam U^2)/(2 sqrt(pi lam)).
-template <int D, class T>
-GKS_FN void u_half(const Maxw<D, T>& g, T sgn, T* u) {
-  const T rs = g_rsqrt(g.lam);  // 1/sqrt(lambda); sqrt(lambda) = lambda / sqrt(lambda)
-  const T z = g.lam * rs * g.U[0];
-  u[0] = T(0.5) * g_erfc(-sgn * z);
-  u[1] = g.U[0] * u[0] + sgn * T(0.5) * g_exp(-z * z) * T(kInvSqrtPi) * rs;
-  recur<7>(g.U[0], g.il, u);
-}
-
-// <psi_m> over the region of table u, m1 the transverse means.
-template <int D, class T>
-GKS_FN void psi_mean(const T* u, const T* m1, T* out) {
-  out[0] = u[0];
-  out[1] = u[1];
-#pragma unroll
-  for (int s = 0; s < D - 1; ++s) out[2 + s] = u[0] * m1[1 + s];
-  out[D + 1] = T(0.5) * u[2] + u[0] * m1[D];
-}
-
-// acc[m] += s * <u^k gamma (a . psi) psi_m>, gamma = 1 (tg = -1) or v_tg.
-// With a . psi = A(u) + sum_beta a_beta beta, A(u) = a0 + a1 u + aE u^2 / 2, and
-// psi_m = P_m(u) + (transverse part), the moment is a sum of (u moment) x (transverse moment).
-template <int D, class T>
-GKS_FN void amom(const T* u, const Trans<D, T>& t, int k, int tg, const T* a, T s, T* acc) {
-  constexpr int NB = D + 1;
-  const T hE = T(0.5) * a[D + 1];
-  const T SA0 = a[0] * u[k] + a[1] * u[k + 1] + hE * u[k + 2];
-  const T SA1 = a[0] * u[k + 1] + a[1] * u[k + 2] + hE * u[k + 3];
-  const T SA2 = a[0] * u[k + 2] + a[1] * u[k + 3] + hE * u[k + 4];
-  // transverse factors: <gamma beta> and <gamma beta tau>
-  T g1[NB], c2[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b) g1[b] = tg < 0 ? t.m1[b] : t.m2[1 + tg][b];
-  T c1 = T(0);
-#pragma unroll
-  for (int b = 1; b < NB; ++b) c1 += a[b == D ? D + 1 : 1 + b] * g1[b];
-#pragma unroll
-  for (int tau = 1; tau < NB; ++tau) {
-    T q = T(0);
-#pragma unroll
-    for (int b = 1; b < NB; ++b) q += a[b == D ? D + 1 : 1 + b] * (tg < 0 ? t.m2[b][tau] : t.m3[tg][b][tau]);
-    c2[tau] = q;
-  }
-  acc[0] += s * (SA0 * g1[0] + u[k] * c1);
-  acc[1] += s * (SA1 * g1[0] + u[k + 1] * c1);
-#pragma unroll
-  for (int v = 0; v < D - 1; ++v) acc[2 + v] += s * (SA0 * g1[1 + v] + u[k] * c2[1 + v]);
-  acc[D + 1] += s * (T(0.5) * (SA2 * g1[0] + u[k + 2] * c1) + SA0 * g1[D] + u[k] * c2[D]);
 }
 
 enum { LIM_MINMOD = 0, LIM_VANLEER = 1 };
@@ -410,77 +308,17 @@ GKS_FN void muscl(int lim, R s0, R s1, R s2, R s3, R h0, R h1, R h2, R h3, R& wl
   wr = s2 - R(0.5) * h2 * sr;
 }
 
-// The pair <u^k gamma (a . psi) psi_m> and <u^(k+1) gamma (a . psi) psi_m>, which share the u-moments
-// of A(u) and the transverse sums: acc_lo += s_lo * first, acc_hi += s_hi * second (k <= 1).
-template <int D, class T>
-GKS_FN void amom2(const T* u, const Trans<D, T>& t, int k, int tg, const T* a, T s_lo, T* acc_lo, T s_hi,
-                  T* acc_hi) {
-  constexpr int NB = D + 1;
-  const T hE = T(0.5) * a[D + 1];
-  T SA[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) SA[j] = a[0] * u[k + j] + a[1] * u[k + j + 1] + hE * u[k + j + 2];
-  T g1[NB], c2[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b) g1[b] = tg < 0 ? t.m1[b] : t.m2[1 + tg][b];
-  T c1 = T(0);
-#pragma unroll
-  for (int b = 1; b < NB; ++b) c1 += a[b == D ? D + 1 : 1 + b] * g1[b];
-#pragma unroll
-  for (int tau = 1; tau < NB; ++tau) {
-    T q = T(0);
-#pragma unroll
-    for (int b = 1; b < NB; ++b) q += a[b == D ? D + 1 : 1 + b] * (tg < 0 ? t.m2[b][tau] : t.m3[tg][b][tau]);
-    c2[tau] = q;
-  }
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const T s = h ? s_hi : s_lo;
-    T* acc = h ? acc_hi : acc_lo;
-    const int kk = k + h;
-    acc[0] += s * (SA[h] * g1[0] + u[kk] * c1);
-    acc[1] += s * (SA[h + 1] * g1[0] + u[kk + 1] * c1);
-#pragma unroll
-    for (int v = 0; v < D - 1; ++v) acc[2 + v] += s * (SA[h] * g1[1 + v] + u[kk] * c2[1 + v]);
-    acc[D + 1] += s * (T(0.5) * (SA[h + 2] * g1[0] + u[kk + 2] * c1) + SA[h] * g1[D] + u[kk] * c2[D]);
-  }
-}
-
-// Coefficients a of a . psi with <(a . psi) psi> = rhs (already divided by rho): closed-form inverse
-// of the Maxwellian moment matrix.
-template <int D, class T>
-GKS_FN void slope(const Maxw<D, T>& g, T bK, const T* rhs, T* a) {
-  T R[D], UR = T(0);
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    R[i] = rhs[1 + i] - g.U[i] * rhs[0];
-    UR += g.U[i] * R[i];
-  }
-  const T RE = T(2) * rhs[D + 1] - g.c * rhs[0];
-  const T aE = g.f4 * (RE - T(2) * UR);
-  const T l2 = T(2) * g.lam;
-  T a0 = rhs[0] - T(0.5) * aE * g.c;
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    a[1 + i] = l2 * R[i] - g.U[i] * aE;
-    a0 -= g.U[i] * a[1 + i];
-  }
-  a[0] = a0;
-  a[D + 1] = aE;
-}
-
-// Time integrals over [0, dt] of Eq. resultingf and the ratios used for Abar:
+// Time integrals over [0, dt] of Eq. resultingf, e = exp(-t/tau):
 //   T0 = int (1 - e), T1 = int ((tau + t) e - tau), T2 = int (t - tau + tau e), T3 = int e,
-//   T4 = -int (tau + t) e, T5 = -tau int e  (e = exp(-t/tau));  Dn = dt^2/2 - T2;
-//   r1 = T1/Dn, r4 = T4/Dn, r5 = T5/Dn.
-// With x = dt/tau and phi_k(x) = sum_m (-x)^m/(m+k)!: T0 = dt x phi2, T1 = -dt^2 x (phi2 - 2 phi3),
-// T2 = dt^2 x phi3, T3 = dt phi1, T4 = tau dt (e - 2 phi1), T5 = -tau dt phi1, Dn = dt^2 phi2.
+//   T4 = -int (tau + t) e, T5 = -tau int e, Dn = dt^2/2 - T2;
+// the flux uses T0, T2, T3, Dn and the ratios r1 = T1/Dn, r4 = T4/Dn, r45 = (T4 - T5)/Dn (finite as
+// tau -> 0).  With x = dt/tau and phi_k(x) = sum_m (-x)^m/(m+k)!: T0 = dt x phi2, T2 = dt^2 x phi3, T3 = dt phi1,
+// Dn = dt^2 phi2, r1 = -x (phi2 - 2 phi3)/phi2, r4 = (e - 2 phi1)/(x phi2), r45 = -(phi1 - phi2)/phi2.
 // For x < 1 phi3 is summed from its series and phi2, phi1, e by the backward recurrence
 // phi_{k-1} = 1/(k-1)! - x phi_k (no cancellation), in the arithmetic type; otherwise the closed
 // forms in e = exp(-x) are used.
-struct TimeCoef {
-  double T[6];
-  double r1, r4, r5;
+template <class T> struct TimeCoef {
+  T T0, T2, T3, Dn, r1, r4, r45;
 };
 
 // phi3 = sum_m (-x)^m / (m+3)! by Horner, then phi2, phi1 and e = exp(-x) by the backward recurrence
@@ -515,339 +353,369 @@ GKS_FN void phi_series(T x, T& p1, T& p2, T& p3, T& e) {
 }
 
 template <class T>
-GKS_FN void time_coeffs(T dt, T tau, T* Tc, T& r1, T& r4, T& r5) {
+GKS_FN void time_coeffs(T dt, T tau, TimeCoef<T>& c) {
   const T x = g_div(dt, tau);
+  const T y = tau * g_rcp(dt);
   if (x < T(1)) {
     // series branch (phi_k summed, no cancellation) in the arithmetic type
     T p1, p2, p3, e;
-    const T xd = x, dtd = dt, taud = tau;
-    phi_series(xd, p1, p2, p3, e);
-    const T Dn = dtd * dtd * p2;
-    const T T1 = -dtd * dtd * xd * (p2 - T(2) * p3);
-    const T T4 = taud * dtd * (e - T(2) * p1);
-    const T T5 = -taud * dtd * p1;
-    Tc[0] = dtd * xd * p2;
-    Tc[1] = T1;
-    Tc[2] = dtd * dtd * xd * p3;
-    Tc[3] = dtd * p1;
-    Tc[4] = T4;
-    Tc[5] = T5;
-    const T iDn = g_rcp(Dn);
-    r1 = T1 * iDn;
-    r4 = T4 * iDn;
-    r5 = T5 * iDn;
+    phi_series<T>(x, p1, p2, p3, e);
+    const T i2 = g_rcp(p2);
+    c.T0 = dt * x * p2;
+    c.T2 = dt * dt * x * p3;
+    c.T3 = dt * p1;
+    c.Dn = dt * dt * p2;
+    c.r1 = -x * (p2 - T(2) * p3) * i2;
+    c.r4 = (e - T(2) * p1) * i2 * y;
+    c.r45 = (p2 - p1) * i2;
   } else {
     const T e = g_exp(-x);
-    const T q = T(1) - e;
-    const T tq = tau * q;
-    Tc[0] = dt - tq;
-    Tc[1] = -tau * dt * (T(1) + e) + T(2) * tau * tq;
-    Tc[2] = T(0.5) * dt * dt - tau * dt + tau * tq;
-    Tc[3] = tq;
-    Tc[4] = tau * dt * e - T(2) * tau * tq;
-    Tc[5] = -tau * tq;
-    const T y = g_div(tau, dt);
-    const T yq = y * q;
-    const T inv = g_rcp(T(1) - yq);
-    r1 = (T(2) * yq - (T(1) + e)) * inv;
-    r4 = (e - T(2) * yq) * inv;
-    r5 = -yq * inv;
+    const T yq = y - y * e;
+    const T P = T(1) - yq;
+    const T inv = g_rcp(P);
+    c.T0 = dt * P;
+    c.Dn = tau * c.T0;
+    c.T2 = T(0.5) * dt * dt - c.Dn;
+    c.T3 = dt * yq;
+    c.r1 = (T(2) * yq - (T(1) + e)) * inv;
+    c.r4 = (e - T(2) * yq) * inv;
+    c.r45 = (e - yq) * inv;
   }
 }
 
 // Two lanes: both branches of time_coeffs, each lane keeping its own (x < 1: the series).
 template <>
-GKS_FN void time_coeffs<F2>(F2 dt, F2 tau, F2* Tc, F2& r1, F2& r4, F2& r5) {
-  const F2 x = g_div(dt, tau);
-  const bool sx = x.v.x < 1.0f, sy = x.v.y < 1.0f;
-  F2 p1, p2, p3, e;
-  phi_series(x, p1, p2, p3, e);
-  const F2 dt2 = F2(dt * dt);
-  const F2 Dn = F2(dt2 * p2);
-  F2 Ts[6];
-  const F2 T1s = F2(-dt2 * x) * (p2 - F2(2.0f) * p3);
-  const F2 T4s = F2(tau * dt) * (e - F2(2.0f) * p1);
-  const F2 T5s = -(F2(tau * dt) * p1);
-  Ts[0] = F2(dt * x) * p2;
-  Ts[1] = T1s;
-  Ts[2] = F2(dt2 * x) * p3;
-  Ts[3] = dt * p1;
-  Ts[4] = T4s;
-  Ts[5] = T5s;
-  const F2 iDn = g_rcp(Dn);
-  const F2 r1s = T1s * iDn, r4s = T4s * iDn, r5s = T5s * iDn;
-  // closed forms in e = exp(-x)
-  const F2 ec = g_exp(-x);
-  const F2 q = F2(1.0f) - ec;
-  const F2 tq = tau * q;
-  F2 Tcl[6];
-  Tcl[0] = dt - tq;
-  Tcl[1] = F2(-(tau * dt)) * (F2(1.0f) + ec) + F2(2.0f) * F2(tau * tq);
-  Tcl[2] = F2(0.5f) * F2(dt * dt) - tau * dt + tau * tq;
-  Tcl[3] = tq;
-  Tcl[4] = F2(tau * dt) * ec - F2(2.0f) * F2(tau * tq);
-  Tcl[5] = -(tau * tq);
-  const F2 y = g_div(tau, dt);
-  const F2 yq = y * q;
-  const F2 inv = g_rcp(F2(1.0f) - yq);
-  const F2 r1c = (F2(2.0f) * yq - (F2(1.0f) + ec)) * inv;
-  const F2 r4c = (ec - F2(2.0f) * yq) * inv;
-  const F2 r5c = -(yq * inv);
-#pragma unroll
-  for (int i = 0; i < 6; ++i) Tc[i] = f2_select(sx, sy, Ts[i], Tcl[i]);
-  r1 = f2_select(sx, sy, r1s, r1c);
-  r4 = f2_select(sx, sy, r4s, r4c);
-  r5 = f2_select(sx, sy, r5s, r5c);
+GKS_FN void time_coeffs<F2>(F2 dt, F2 tau, TimeCoef<F2>& c) {
+  TimeCoef<float> a, b;
+  time_coeffs<float>(dt.v.x, tau.v.x, a);
+  time_coeffs<float>(dt.v.y, tau.v.y, b);
+  c.T0 = F2(a.T0, b.T0);
+  c.T2 = F2(a.T2, b.T2);
+  c.T3 = F2(a.T3, b.T3);
+  c.Dn = F2(a.Dn, b.Dn);
+  c.r1 = F2(a.r1, b.r1);
+  c.r4 = F2(a.r4, b.r4);
+  c.r45 = F2(a.r45, b.r45);
 }
 
 // The time coefficients with the degree of rarefaction eps in place of tau/dt (Eqs. tautautilde,
 // rarefactionkepsilon, epsilonkomega): Eq. fkepsilon with alpha = eps (1 - e^{-1/eps}) and
-// beta = e^{-1/eps} (Eq. alphabetakepsilon with the corrected beta), in the T0..T5 form:
-//   T0 = dt (1 - alpha), T1 = dt tau (2 alpha - 1 - beta), T2 = dt (dt/2 - tau (1 - alpha)),
-//   T3 = dt alpha, T4 = dt tau (beta - 2 alpha), T5 = -dt tau alpha, Dn = dt tau (1 - alpha),
-// so r1 = (2 alpha - 1 - beta)/(1 - alpha), r4 = (beta - 2 alpha)/(1 - alpha), r5 = -alpha/(1 - alpha).
+// beta = e^{-1/eps} (Eq. alphabetakepsilon with the corrected beta):
+//   T0 = dt (1 - alpha), T2 = dt (dt/2 - tau (1 - alpha)), T3 = dt alpha, Dn = dt tau (1 - alpha),
+//   r1 = (2 alpha - 1 - beta)/(1 - alpha), r4 = (beta - 2 alpha)/(1 - alpha), r45 = (beta - alpha)/(1 - alpha).
 // eps = tau/dt gives time_coeffs.  For eps > 1 (x = 1/eps < 1) alpha = phi1(x), 1 - alpha = x phi2,
-// 2 alpha - 1 - beta = -x^2 (phi2 - 2 phi3), from the cancellation-free series.
+// 2 alpha - 1 - beta = -x^2 (phi2 - 2 phi3), beta - alpha = -x (phi1 - phi2), from the cancellation-free series.
 template <class T>
-GKS_FN void time_coeffs_hat(T dt, T tau, T eps, T* Tc, T& r1, T& r4, T& r5) {
-  T a, one_a, c1, c4;
+GKS_FN void time_coeffs_hat(T dt, T tau, T eps, TimeCoef<T>& c) {
+  T a, one_a, c1, c4, c45;
   if (eps > T(1)) {
     const T x = g_rcp(eps);
     T p1, p2, p3, e;
-    phi_series(x, p1, p2, p3, e);
+    phi_series<T>(x, p1, p2, p3, e);
     a = p1;
     one_a = x * p2;
     c1 = -x * x * (p2 - T(2) * p3);
     c4 = e - T(2) * p1;
+    c45 = x * (p2 - p1);
   } else {
     const T beta = eps > T(0) ? g_exp(-g_rcp(eps)) : T(0);
     a = eps * (T(1) - beta);
     one_a = T(1) - a;
     c1 = T(2) * a - T(1) - beta;
     c4 = beta - T(2) * a;
+    c45 = beta - a;
   }
-  const T dtau = dt * tau;
-  Tc[0] = dt * one_a;
-  Tc[1] = dtau * c1;
-  Tc[2] = dt * (T(0.5) * dt - tau * one_a);
-  Tc[3] = dt * a;
-  Tc[4] = dtau * c4;
-  Tc[5] = -dtau * a;
   const T i1 = g_rcp(one_a);
-  r1 = c1 * i1;
-  r4 = c4 * i1;
-  r5 = -a * i1;
+  c.T0 = dt * one_a;
+  c.T2 = dt * (T(0.5) * dt - tau * one_a);
+  c.T3 = dt * a;
+  c.Dn = dt * tau * one_a;
+  c.r1 = c1 * i1;
+  c.r4 = c4 * i1;
+  c.r45 = c45 * i1;
 }
 
-// The density row <u^k gamma (a . psi)> of amom alone.
-template <int D, class T>
-GKS_FN T amom_rho(const T* u, const Trans<D, T>& t, int k, int tg, const T* a) {
-  constexpr int NB = D + 1;
-  const T hE = T(0.5) * a[D + 1];
-  const T SA0 = a[0] * u[k] + a[1] * u[k + 1] + hE * u[k + 2];
-  T g0 = tg < 0 ? t.m1[0] : t.m2[1 + tg][0], c1 = T(0);
+// One side of the initial state (Eq. initialf0): with the slopes sn (normal) and st (tangential) of its
+// conservative variables and the half-line moments rho eta_n in e, the distribution
+// q = r5 A + r4 (u a + v b) of the Abar condition and of the flux is, averaged over the transverse velocities,
+//   <q>       = q0 + q1 c + q2 c^2 + q3 c^3,
+//   <q c_k>   = k0 + k1 c + k2 c^2,                                      c = u - U, k a tangential axis,
+//   <q w/2>   = (bK - 1) theta/2 <q> + e0 + e1 c,                        w = sum c_k^2 + xi^2,
+// with the Euler rates N, the deviatoric strain and the heat-flux gradients as coefficients.  Returned in the
+// frame moving with U0 (that of g0): its moments rhs = <q psi>, and F = Dn <u q psi> + T3 <u psi>.
+template <int D, class T, bool MULTID>
+GKS_FN void side_terms(const Maxw<D, T>& g, const T* e, const T* sn, const T (*st)[D + 2], const T* U0, T bK, T ibK, T T3,
+                       T Dn, T r4, T r45, T* rhs, T* F) {
+  constexpr int nv = D + 2;
+  const T k1d = bK - T(1);
+  Grad<D, T> gx, gs[Dims<D>::nt], N;
+  T r[nv], S, div;
 #pragma unroll
-  for (int b = 1; b < NB; ++b) c1 += a[b == D ? D + 1 : 1 + b] * (tg < 0 ? t.m1[b] : t.m2[1 + tg][b]);
-  return SA0 * g0 + u[k] * c1;
+  for (int m = 0; m < nv; ++m) r[m] = sn[m] * g.ir;
+  gradient<D, T>(g, bK, ibK, r, gx);
+  if (MULTID) {
+#pragma unroll
+    for (int q = 0; q < D - 1; ++q) {
+#pragma unroll
+      for (int m = 0; m < nv; ++m) r[m] = st[q][m] * g.ir;
+      gradient<D, T>(g, bK, ibK, r, gs[q]);
+    }
+  }
+  euler_rate<D, T, MULTID>(g, ibK, gx, gs, S, div, N);
+  const T sg = r4 * (gx.U[0] - ibK * div);  // deviatoric normal strain
+  const T nu = r45 * (T(0.5) * g.it * N.th);
+  const T h = nu + sg;
+  const T ha = T(0.5) * r4 * gx.th, hai = ha * g.it;
+  const T q0 = r45 * N.r - h, q1 = g.it * (r45 * N.U[0]) - T(3) * hai, q2 = g.it * h, q3 = hai * g.it;
+  const T J0 = q0 * e[0] + q1 * e[1] + q2 * e[2] + q3 * e[3];
+  const T J1 = q0 * e[1] + q1 * e[2] + q2 * e[3] + q3 * e[4];
+  const T J2 = q0 * e[2] + q1 * e[3] + q2 * e[4] + q3 * e[5];
+  const T J3 = q0 * e[3] + q1 * e[4] + q2 * e[5] + q3 * e[6];
+  const T e0 = g.th * (k1d * nu - sg), e1 = k1d * ha, hk = T(0.5) * k1d * g.th;
+  // moments of q psi and u q psi in the side's own frame
+  T m[nv], x[nv];
+  m[0] = J0;
+  m[1] = J1;
+  m[D + 1] = T(0.5) * J2 + hk * J0 + e0 * e[0] + e1 * e[1];
+  x[0] = g.U[0] * J0 + J1;
+  x[1] = g.U[0] * J1 + J2;
+  x[D + 1] = g.U[0] * m[D + 1] + (T(0.5) * J3 + hk * J1 + e0 * e[1] + e1 * e[2]);
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) {
+    T k0 = r45 * N.U[1 + k], k1 = r4 * gx.U[1 + k];
+    if (MULTID) {
+      const T hb = T(0.5) * r4 * gs[k].th, k2 = hb * g.it;
+      k0 -= hb;
+      k1 = r4 * (gx.U[1 + k] + gs[k].U[0]);
+      m[2 + k] = k0 * e[0] + k1 * e[1] + k2 * e[2];
+      x[2 + k] = g.U[0] * m[2 + k] + (k0 * e[1] + k1 * e[2] + k2 * e[3]);
+    } else {
+      m[2 + k] = k0 * e[0] + k1 * e[1];
+      x[2 + k] = g.U[0] * m[2 + k] + (k0 * e[1] + k1 * e[2]);
+    }
+  }
+  // free transport <u psi> of the side
+  const T V0 = g.U[0] * e[0] + e[1], VU = g.U[0] * e[1] + e[2];
+  const T VE = T(0.5) * (g.U[0] * e[2] + e[3]) + hk * V0;
+  x[0] = Dn * x[0] + T3 * V0;
+  x[1] = Dn * x[1] + T3 * VU;
+  x[D + 1] = Dn * x[D + 1] + T3 * VE;
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) x[2 + k] = Dn * x[2 + k];
+  // into the frame of g0
+  T hd2 = T(0), sm = m[D + 1], sx = x[D + 1];
+  rhs[0] = m[0];
+  F[0] = x[0];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const T d = g.U[i] - U0[i];
+    hd2 += d * d;
+    sm += d * m[1 + i];
+    sx += d * x[1 + i];
+    rhs[1 + i] = m[1 + i] + d * m[0];
+    F[1 + i] = x[1 + i] + d * x[0];
+  }
+  hd2 = T(0.5) * hd2;
+  rhs[D + 1] = sm + hd2 * m[0];
+  F[D + 1] = sx + hd2 * x[0];
+}
+
+// The equilibrium state (Eq. eqlgform): gradients abar_l, abar_r from W_j -> w0 -> W_{j+1} and the mean
+// tangential slopes.  <(u abar + v bbar) psi> over the full line with abar_r is the Euler rate N; what abar_l adds
+// on u > 0 is the half-line part of d = abar_l - abar_r: rh = <u d psi>, fl = <u^2 d psi> (frame of g0).
+template <int D, class T> struct EqTerms {
+  Grad<D, T> N;
+  T rh[D + 2], fl[D + 2];
+  T sg, ux[Dims<D>::nt], thx;  // U' - div/bK, the shear sums and theta' of the full-line part (abar_r)
+};
+template <int D, class T, bool MULTID, class In>
+GKS_FN void equilibrium_terms(const Maxw<D, T>& g, const T* w0, const In& in, T idxl, T idxr, T bK, T ibK,
+                              EqTerms<D, T>& q) {
+  constexpr int nv = D + 2;
+  const T k1d = bK - T(1);
+  Grad<D, T> gr, gd, gs[Dims<D>::nt];
+  const T fl = g.ir * idxl, fr = g.ir * idxr;
+  T r[nv], d[nv], S, div;
+#pragma unroll
+  for (int m = 0; m < nv; ++m) {
+    r[m] = (in.c(1, m) - w0[m]) * fr;
+    d[m] = (w0[m] - in.c(0, m)) * fl - r[m];
+  }
+  gradient<D, T>(g, bK, ibK, r, gr);
+  gradient<D, T>(g, bK, ibK, d, gd);
+  if (MULTID) {
+    const T hi = T(0.5) * g.ir;
+#pragma unroll
+    for (int s = 0; s < D - 1; ++s) {
+#pragma unroll
+      for (int m = 0; m < nv; ++m) r[m] = (in.t(0, s, m) + in.t(1, s, m)) * hi;
+      gradient<D, T>(g, bK, ibK, r, gs[s]);
+    }
+  }
+  euler_rate<D, T, MULTID>(g, ibK, gr, gs, S, div, q.N);
+  q.sg = gr.U[0] - ibK * div;
+  q.thx = gr.th;
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) q.ux[k] = MULTID ? gr.U[1 + k] + gs[k].U[0] : gr.U[1 + k];
+  // half line u > 0 of u d: <d> = b0 + b1 c + b2 c^2 over the transverse velocities
+  T e[7];
+  half_moments<D, T>(g, T(1), T(1), e);
+  const T hg = T(0.5) * gd.th * g.it;
+  const T b0 = gd.r - hg, b1 = gd.U[0] * g.it, b2 = hg * g.it;
+  T L[5], M[4];
+#pragma unroll
+  for (int n = 0; n < 5; ++n) L[n] = b0 * e[n] + b1 * e[n + 1] + b2 * e[n + 2];
+#pragma unroll
+  for (int n = 0; n < 4; ++n) M[n] = g.U[0] * L[n] + L[n + 1];
+  const T V0 = g.U[0] * e[0] + e[1], W2 = g.U[0] * V0 + (g.U[0] * e[1] + e[2]);
+  const T hk = T(0.5) * k1d * g.th, dk = T(0.5) * k1d * gd.th;
+  q.rh[0] = M[0];
+  q.rh[1] = M[1];
+  q.rh[D + 1] = T(0.5) * M[2] + hk * M[0] + dk * V0;
+  q.fl[0] = g.U[0] * M[0] + M[1];
+  q.fl[1] = g.U[0] * M[1] + M[2];
+  q.fl[D + 1] = T(0.5) * (g.U[0] * M[2] + M[3]) + hk * q.fl[0] + dk * W2;
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) {
+    q.rh[2 + k] = gd.U[1 + k] * V0;
+    q.fl[2 + k] = gd.U[1 + k] * W2;
+  }
 }
 
 // |D rho| = |d_t rho + U_n d_n rho| at the face for the rarefaction option (Eqs. tautautilde,
 // tautilde): d_t rho = -rho0 (<abar_l . psi u>_{u>0} + <abar_r . psi u>_{u<0} + <bbar . psi v>) from
 // the t = 0 compatibility condition of the equilibrium part, d_n rho the mean of the density slopes
-// (w0 - W_j)/dxl and (W_{j+1} - w0)/dxr.  Slopes and moments of g0 as in face_flux.
-template <int D, class T, bool MULTID, class In>
-GKS_FN T face_drho(const Maxw<D, T>& g0, const T* w0, const In& in, T dxl, T dxr, T i0, T bK, T K) {
-  constexpr int nv = D + 2;
-  const T dn = T(0.5) * (g_div(w0[0] - in.c(0, 0), dxl) + g_div(in.c(1, 0) - w0[0], dxr));
-  Trans<D, T> t0;
-  transverse<D, T>(g0, K, t0);
-  T oF[7], oP[7], half[7], r[nv], ab[nv];
-  u_full<D, T>(g0, oF);
-  u_half<D, T>(g0, T(1), oP);
-  const T fl = g_div(i0, dxl), fr = g_div(i0, dxr);
-#pragma unroll
-  for (int m = 0; m < nv; ++m) r[m] = (w0[m] - in.c(0, m)) * fl;
-  slope<D, T>(g0, bK, r, ab);
-  T x1 = amom_rho<D, T>(oP, t0, 1, -1, ab);
-#pragma unroll
-  for (int m = 0; m < nv; ++m) r[m] = (in.c(1, m) - w0[m]) * fr;
-  slope<D, T>(g0, bK, r, ab);
-#pragma unroll
-  for (int n = 0; n < 7; ++n) half[n] = oF[n] - oP[n];
-  x1 += amom_rho<D, T>(half, t0, 1, -1, ab);
-  if (MULTID) {
-#pragma unroll
-    for (int q = 0; q < D - 1; ++q) {
-#pragma unroll
-      for (int m = 0; m < nv; ++m) r[m] = T(0.5) * (in.t(0, q, m) + in.t(1, q, m)) * i0;
-      slope<D, T>(g0, bK, r, ab);
-      x1 += amom_rho<D, T>(oF, t0, 0, q, ab);
-    }
+// (w0 - W_j)/dxl and (W_{j+1} - w0)/dxr.
+template <int D, class T, class In>
+GKS_FN T face_drho(const Maxw<D, T>& g0, const EqTerms<D, T>& q, const T* w0, const In& in, T idxl, T idxr) {
+  const T dn = T(0.5) * ((w0[0] - in.c(0, 0)) * idxl + (in.c(1, 0) - w0[0]) * idxr);
+  return g_abs(g0.U[0] * dn - g0.rho * (q.N.r + q.rh[0]));
+}
+
+// Abar and the flux: rhs, F in the frame of g0 hold the two sides' parts (rho-weighted); on return F is
+// the time-integrated flux in the frame of the face.
+template <int D, class T>
+GKS_FN void close_flux(const Maxw<D, T>& g, const EqTerms<D, T>& q, const TimeCoef<T>& c, int abar_t0, T bK, T ibK,
+                       const T* rhs, T* F) {
+  // Abar from the compatibility condition integrated over [0, dt] (or at t = 0), as gradients of
+  // (r, U, theta); the full-line part enters as such
+  T r1 = c.r1, ws = g.ir;
+  if (abar_t0) {
+    r1 = T(-1);
+    ws = T(0);
   }
-  return g_abs(-g0.rho * x1 + g0.U[0] * dn);
+  const T e1 = c.Dn * c.r1;
+  const T m0 = r1 * q.rh[0] + ws * rhs[0], mE = r1 * q.rh[D + 1] + ws * rhs[D + 1];
+  // Z = T2 Abar + T1 N
+  const T n1 = c.T2 * r1 + e1;
+  const T Zr = c.T2 * m0 + n1 * q.N.r;
+  const T Zt = c.T2 * (T(2) * ibK * mE - g.th * m0) + n1 * q.N.th;
+  T Z[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) Z[i] = c.T2 * (r1 * q.rh[1 + i] + ws * rhs[1 + i]) + n1 * q.N.U[i];
+  // rho0 <u (T0 + T2 Abar + T1 (u abar + v bbar)) psi>: Euler flux of the increments, stress and heat flux
+  const T P = g.th * (Zr + c.T0) + Zt, hb = T(0.5) * bK, et = e1 * g.th;
+  T f[D + 2];
+  f[0] = g.U[0] * (Zr + c.T0) + Z[0] + e1 * q.fl[0];
+  f[1] = g.U[0] * Z[0] + P + T(2) * et * q.sg + e1 * q.fl[1];
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) f[2 + k] = g.U[0] * Z[1 + k] + et * q.ux[k] + e1 * q.fl[2 + k];
+  f[D + 1] = hb * (g.U[0] * P) + (hb + T(1)) * (g.th * Z[0] + et * q.thx) + e1 * q.fl[D + 1];
+  // with the sides, and out of the moving frame
+#pragma unroll
+  for (int m = 0; m < D + 2; ++m) f[m] = g.rho * f[m] + F[m];
+  T q2 = T(0), s = f[D + 1];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    q2 += g.U[i] * g.U[i];
+    s += g.U[i] * f[1 + i];
+    F[1 + i] = f[1 + i] + g.U[i] * f[0];
+  }
+  F[0] = f[0];
+  F[D + 1] = s + T(0.5) * q2 * f[0];
+}
+
+// w0 = sum over the sides of <psi> over their half lines (Eq. intermediatestate), the side's part: e the
+// rho-weighted half-line moments.
+template <int D, class T>
+GKS_FN void side_state(const Maxw<D, T>& g, const T* e, T bK, T* w) {
+  T c = (bK - T(1)) * g.th;
+  w[0] = e[0];
+  w[1] = g.U[0] * e[0] + e[1];
+#pragma unroll
+  for (int i = 0; i < D; ++i) c += g.U[i] * g.U[i];
+#pragma unroll
+  for (int k = 0; k < D - 1; ++k) w[2 + k] = g.U[1 + k] * e[0];
+  w[D + 1] = T(0.5) * (e[2] + c * e[0]) + g.U[0] * e[1];
 }
 
 // One face.  Inputs in the face frame:
 //   wl, wr   reconstructed states; cl, cr cell averages of the two cells; sl, sr normal slopes;
-//   tl, tr   tangential slopes (multi-dimensional expansion only); dxl, dxr centre-to-face distances;
-//   tau_t    turbulent relaxation time at the face; dt the time step.
+//   tl, tr   tangential slopes (multi-dimensional expansion only); idxl, idxr inverse centre-to-face
+//            distances; tau_t turbulent relaxation time at the face; dt the time step.
 // Output: F, the flux integrated over [0, dt] (Eq. fluxesf); tau_out the total relaxation time.
-//
-// The work is ordered so that each velocity region (u > 0 of the left Maxwellian, u < 0 of the
-// right one, and the two halves and the full line of the equilibrium g0) is visited once, adding
-// both its part of the right-hand side of the Abar equation and its part of the flux; only the
-// Abar term of the flux waits for Abar.
 // RAR: the rarefaction option -- the degree of rarefaction eps = tau/tauhat, tauhat = rho0/|D rho|
 // (capped at 1e30), replaces tau/dt inside the time coefficients (Eq. epsilonkomega).
 //
-// The inputs other than wl, wr come through an accessor `in` (FaceArrays below, or a view of a
-// shared-memory tile): in.s(sd, m) the normal slope, in.c(sd, m) the cell average and in.t(sd, q, m)
-// the q-th tangential slope of component m on side sd (0 left, 1 right), each read where it is used.
+// The inputs other than wl, wr come through an accessor `in` (FaceArrays below): in.s(sd, m) the normal slope,
+// in.c(sd, m) the cell average and in.t(sd, q, m) the q-th tangential slope of component m on side sd (0 left, 1
+// right), each read where it is used.
 template <int D, class T, bool MULTID, bool RAR = false, class In>
-GKS_FN void face_flux_in(const T* wl, const T* wr, const In& in, T dxl, T dxr, T tau_t, T dt, const Gas<T>& gas,
+GKS_FN void face_flux_in(const T* wl, const T* wr, const In& in, T idxl, T idxr, T tau_t, T dt, const Gas<T>& gas,
                          int abar_t0, T* F, T* tau_out) {
   constexpr int nv = D + 2;
-  const T bK = gas.bK, K = gas.K, ibK = gas.ibK;
-  const Maxw<D, T> gl = maxwellian<D, T>(wl, bK, ibK);
-  const Maxw<D, T> gr = maxwellian<D, T>(wr, bK, ibK);
-
-  // Eq. intermediatestate: w0 = rho_l <psi>_{l,u>0} + rho_r <psi>_{r,u<0}
-  T w0[nv];
-  T lP[7], rN[7];
-  u_half<D, T>(gl, T(1), lP);
-  u_half<D, T>(gr, T(-1), rN);
-  {
-    T a[nv], b[nv], ml[D + 1], mr[D + 1];
-    trans_mean<D, T>(gl, K, ml);
-    trans_mean<D, T>(gr, K, mr);
-    psi_mean<D, T>(lP, ml, a);
-    psi_mean<D, T>(rN, mr, b);
+  const T bK = gas.bK, ibK = gas.ibK;
+  const Maxw<D, T> gl = maxwellian<D, T>(wl, ibK);
+  const Maxw<D, T> gr = maxwellian<D, T>(wr, ibK);
+  T w0[nv], w1[nv], el[7], er[7];
+  half_moments<D, T>(gl, T(1), gl.rho, el);
+  half_moments<D, T>(gr, T(-1), gr.rho, er);
+  side_state<D, T>(gl, el, bK, w0);
+  side_state<D, T>(gr, er, bK, w1);
 #pragma unroll
-    for (int m = 0; m < nv; ++m) w0[m] = gl.rho * a[m] + gr.rho * b[m];
-  }
-  const Maxw<D, T> g0 = maxwellian<D, T>(w0, bK, ibK);
-
+  for (int m = 0; m < nv; ++m) w0[m] += w1[m];
+  const Maxw<D, T> g0 = maxwellian<D, T>(w0, ibK);
   // Eqs. relaxation time and taua: tau = mu/p0 + tau_t + C_a |p_r - p_l| / (p_r + p_l) dt
-  const T p0 = g0.rho * g0.il, pl = gl.rho * gl.il, pr = gr.rho * gr.il;
-  const T tau = g_div(gas.mu, p0) + tau_t + g_div(gas.C_a * g_abs(pr - pl), pr + pl) * dt;
+  const T pl = gl.rho * gl.th, pr = gr.rho * gr.th;
+  const T tau = gas.mu * g0.ir * g0.it + tau_t + g_div(gas.C_a * g_abs(pr - pl), pr + pl) * dt;
   *tau_out = tau;
-  T Tc[6], r1, r4, r5;
+  TimeCoef<T> c;
+  EqTerms<D, T> q;
   if constexpr (RAR) {
-    const T drho = face_drho<D, T, MULTID>(g0, w0, in, dxl, dxr, g0.ir, bK, K);
+    equilibrium_terms<D, T, MULTID>(g0, w0, in, idxl, idxr, bK, ibK, q);
+    const T drho = face_drho<D, T>(g0, q, w0, in, idxl, idxr);
     const T eps = drho > T(1e-30) * g0.rho ? g_div(tau * drho, g0.rho) : tau * T(1e-30);
-    time_coeffs_hat<T>(dt, tau, eps, Tc, r1, r4, r5);
+    time_coeffs_hat<T>(dt, tau, eps, c);
   } else {
-    time_coeffs<T>(dt, tau, Tc, r1, r4, r5);
+    time_coeffs<T>(dt, tau, c);
   }
-  if (abar_t0) {
-    r1 = T(-1);
-    r4 = r5 = T(0);
-  }
-  const T i0 = g0.ir;
-
-  // Abar right-hand side (per unit rho0) and flux, accumulated region by region
   T rhs[nv];
 #pragma unroll
-  for (int m = 0; m < nv; ++m) {
-    rhs[m] = T(0);
-    F[m] = T(0);
-  }
-
-  // The two sides of the initial state, one loop body (sd = 0: left Maxwellian on u > 0, sd = 1:
-  // right Maxwellian on u < 0): Eq. initialf0 slopes a (normal), b (tangential), A; their parts of
-  // the Abar right-hand side and of the flux.
+  for (int m = 0; m < nv; ++m) rhs[m] = F[m] = T(0);
+  // the two sides in one loop body
 #pragma unroll 1
   for (int sd = 0; sd < 2; ++sd) {
     const Maxw<D, T> g = sd ? gr : gl;
-    Trans<D, T> ts;
-    transverse<D, T>(g, K, ts);
-    T half[7], a[nv], b[Dims<D>::nt][nv], A[nv], r[nv];
+    T e[7], sn[nv], st[Dims<D>::nt][nv], rs[nv], Fs[nv];
 #pragma unroll
-    for (int n = 0; n < 7; ++n) half[n] = sd ? rN[n] : lP[n];
-    const T ir = g.ir;
+    for (int n = 0; n < 7; ++n) e[n] = sd ? er[n] : el[n];
 #pragma unroll
-    for (int m = 0; m < nv; ++m) r[m] = in.s(sd, m) * ir;
-    slope<D, T>(g, bK, r, a);
+    for (int m = 0; m < nv; ++m) sn[m] = in.s(sd, m);
     if (MULTID) {
 #pragma unroll
-      for (int q = 0; q < D - 1; ++q) {
+      for (int s = 0; s < D - 1; ++s)
 #pragma unroll
-        for (int m = 0; m < nv; ++m) r[m] = in.t(sd, q, m) * ir;
-        slope<D, T>(g, bK, r, b[q]);
-      }
+        for (int m = 0; m < nv; ++m) st[s][m] = in.t(sd, s, m);
     }
-    // A from the compatibility condition at t = 0: <(a u + b v + A) psi> = 0 (full line)
-    {
-      T uf[7];
-      u_full<D, T>(g, uf);
+    side_terms<D, T, MULTID>(g, e, sn, st, g0.U, bK, ibK, c.T3, c.Dn, c.r4, c.r45, rs, Fs);
 #pragma unroll
-      for (int m = 0; m < nv; ++m) r[m] = T(0);
-      amom<D, T>(uf, ts, 1, -1, a, T(-1), r);
-      if (MULTID) {
-#pragma unroll
-        for (int q = 0; q < D - 1; ++q) amom<D, T>(uf, ts, 0, q, b[q], T(-1), r);
-      }
-      slope<D, T>(g, bK, r, A);
-    }
-    // Abar rhs: r4 rho/rho0 <(a u + b v) psi> + r5 rho/rho0 <A psi> over the half line, and the
-    // flux rho [T3 <u psi> + T5 <u A psi> + T4 (<u^2 a psi> + <u v b psi>)]: each polynomial once,
-    // at u^k for the rhs and u^(k+1) for the flux
-    const T s4 = r4 * g.rho * i0, s5 = r5 * g.rho * i0, s4f = Tc[4] * g.rho;
-    amom2<D, T>(half, ts, 1, -1, a, s4, rhs, s4f, F);
-    amom2<D, T>(half, ts, 0, -1, A, s5, rhs, Tc[5] * g.rho, F);
-    {
-      T m[nv];
-      psi_mean<D, T>(half + 1, ts.m1, m);  // <u psi> over the half line
-      const T s3 = Tc[3] * g.rho;
-#pragma unroll
-      for (int q = 0; q < nv; ++q) F[q] += s3 * m[q];
-    }
-    if (MULTID) {
-#pragma unroll
-      for (int q = 0; q < D - 1; ++q) amom2<D, T>(half, ts, 0, q, b[q], s4, rhs, s4f, F);
+    for (int m = 0; m < nv; ++m) {
+      rhs[m] += rs[m];
+      F[m] += Fs[m];
     }
   }
-
-  // equilibrium g0: Eq. eqlgform slopes from W_j -> w0 -> W_{j+1} (and the mean tangential slope)
-  Trans<D, T> tr0;
-  transverse<D, T>(g0, K, tr0);
-  T oF[7], oP[7];
-  u_full<D, T>(g0, oF);
-  u_half<D, T>(g0, T(1), oP);
-  {
-    const T fl = g_div(i0, dxl), fr = g_div(i0, dxr);
-    const T s1f = Tc[1] * g0.rho;
-#pragma unroll 1
-    for (int sd = 0; sd < 2; ++sd) {
-      // sd = 0: abar_l on u > 0; sd = 1: abar_r on u < 0 (table = full line minus u > 0)
-      T r[nv], ab[nv], half[7];
-#pragma unroll
-      for (int m = 0; m < nv; ++m) r[m] = sd ? (in.c(1, m) - w0[m]) * fr : (w0[m] - in.c(0, m)) * fl;
-#pragma unroll
-      for (int n = 0; n < 7; ++n) half[n] = sd ? oF[n] - oP[n] : oP[n];
-      slope<D, T>(g0, bK, r, ab);
-      amom2<D, T>(half, tr0, 1, -1, ab, r1, rhs, s1f, F);
-    }
-    if (MULTID) {
-      T r[nv], ab[nv];
-#pragma unroll
-      for (int q = 0; q < D - 1; ++q) {
-#pragma unroll
-        for (int m = 0; m < nv; ++m) r[m] = T(0.5) * (in.t(0, q, m) + in.t(1, q, m)) * i0;
-        slope<D, T>(g0, bK, r, ab);
-        amom2<D, T>(oF, tr0, 0, q, ab, r1, rhs, s1f, F);
-      }
-    }
-  }
-  // Abar from the compatibility condition integrated over [0, dt]; flux rho0 <u (T0 + T2 Abar) psi>
-  {
-    T Ab[nv];
-    slope<D, T>(g0, bK, rhs, Ab);
-#pragma unroll
-    for (int m = 0; m < nv; ++m) Ab[m] *= Tc[2];
-    Ab[0] += Tc[0];
-    amom<D, T>(oF, tr0, 1, -1, Ab, g0.rho, F);
-  }
+  if constexpr (!RAR) equilibrium_terms<D, T, MULTID>(g0, w0, in, idxl, idxr, bK, ibK, q);
+  close_flux<D, T>(g0, q, c, abar_t0, bK, ibK, rhs, F);
 }
 
 // Face inputs held in the caller's arrays (registers): sl, sr normal slopes, cl, cr cell averages,
@@ -861,209 +729,108 @@ template <int D, class T> struct FaceArrays {
   GKS_FN T t(int sd, int q, int m) const { return sd ? tr[q][m] : tl[q][m]; }
 };
 
-// face_flux_in with the inputs in arrays.
+// face_flux_in with the inputs in arrays and the inverse centre-to-face distances given.
+template <int D, class T, bool MULTID, bool RAR = false>
+GKS_FN void face_flux_inv(const T* wl, const T* wr, const T* cl, const T* cr, const T* sl, const T* sr,
+                          const T (*tl)[D + 2], const T (*tr)[D + 2], T idxl, T idxr, T tau_t, T dt,
+                          const Gas<T>& gas, int abar_t0, T* F, T* tau_out) {
+  const FaceArrays<D, T> in{sl, sr, cl, cr, tl, tr};
+  face_flux_in<D, T, MULTID, RAR>(wl, wr, in, idxl, idxr, tau_t, dt, gas, abar_t0, F, tau_out);
+}
+
+// face_flux with the inputs in arrays and the centre-to-face distances.
 template <int D, class T, bool MULTID, bool RAR = false>
 GKS_FN void face_flux(const T* wl, const T* wr, const T* cl, const T* cr, const T* sl, const T* sr,
                       const T (*tl)[D + 2], const T (*tr)[D + 2], T dxl, T dxr, T tau_t, T dt, const Gas<T>& gas,
                       int abar_t0, T* F, T* tau_out) {
-  const FaceArrays<D, T> in{sl, sr, cl, cr, tl, tr};
-  face_flux_in<D, T, MULTID, RAR>(wl, wr, in, dxl, dxr, tau_t, dt, gas, abar_t0, F, tau_out);
+  face_flux_inv<D, T, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, g_rcp(dxl), g_rcp(dxr), tau_t, dt, gas, abar_t0, F,
+                                   tau_out);
 }
 
 // face_flux_in in single precision with the two sides of the face evaluated together on the paired
 // FP32 instructions: lane x carries the left Maxwellian on u > 0, lane y the right one on u < 0, for
-// the intermediate state, the slopes a, b, A and their parts of the Abar right-hand side and of the
-// flux; the two one-sided equilibrium slopes abar_l (u > 0) and abar_r (u < 0) are paired the same
-// way.  The paired sums are added lane x + lane y at the end of each part.  Same terms as
-// face_flux_in; the order of the final additions differs, mu/p0 is taken as 2 mu lambda0 / rho0, the
-// artificial part of tau is skipped when C_a = 0, and idxl, idxr are the reciprocals of dxl, dxr.
+// the intermediate state and the sides' parts of the Abar right-hand side and of the flux.  The paired sums
+// are added lane x + lane y at the end of each part.  Same terms as face_flux_in; the artificial part of tau is
+// skipped when C_a = 0.
 template <int D, bool MULTID, bool RAR = false, class In>
-GKS_FN void face_flux_ps(const float* wl, const float* wr, const In& in, float dxl, float dxr, float idxl,
-                         float idxr, float tau_t, float dt, const Gas<float>& gas, int abar_t0, float* F,
-                         float* tau_out) {
+GKS_FN void face_flux_ps(const float* wl, const float* wr, const In& in, float idxl, float idxr, float tau_t, float dt,
+                         const Gas<float>& gas, int abar_t0, float* F, float* tau_out) {
   using T = float;
   constexpr int nv = D + 2;
-  const T bK = gas.bK, K = gas.K, ibK = gas.ibK;
+  const T bK = gas.bK, ibK = gas.ibK;
   F2 w2[nv];
 #pragma unroll
   for (int m = 0; m < nv; ++m) w2[m] = F2(wl[m], wr[m]);
-  const Maxw<D, F2> gs = maxwellian<D, F2>(w2, F2(bK), F2(ibK));
-  F2 hs[7];  // <u^n> over u > 0 (left) and u < 0 (right)
-  u_half<D, F2>(gs, F2(1.0f, -1.0f), hs);
-
-  // Eq. intermediatestate: w0 = rho_l <psi>_{l,u>0} + rho_r <psi>_{r,u<0}
+  const Maxw<D, F2> gs = maxwellian<D, F2>(w2, F2(ibK));
+  F2 e[7];  // rho eta_n over u > 0 (left) and u < 0 (right)
+  half_moments<D, F2>(gs, F2(1.0f, -1.0f), gs.rho, e);
   T w0[nv];
   {
-    F2 ab[nv], m1[D + 1];
-    trans_mean<D, F2>(gs, F2(K), m1);
-    psi_mean<D, F2>(hs, m1, ab);
+    F2 q[nv];
+    side_state<D, F2>(gs, e, F2(bK), q);
 #pragma unroll
-    for (int m = 0; m < nv; ++m) {
-      const F2 q = F2(gs.rho * ab[m]);
-      w0[m] = q.v.x + q.v.y;
-    }
+    for (int m = 0; m < nv; ++m) w0[m] = q[m].v.x + q[m].v.y;
   }
-  const Maxw<D, T> g0 = maxwellian<D, T>(w0, bK, ibK);
-
-  // Eqs. relaxation time and taua: mu/p0 = 2 mu lambda0 / rho0; the artificial part only with C_a > 0
-  T tau = T(2) * gas.mu * g0.lam * g0.ir + tau_t;
+  const Maxw<D, T> g0 = maxwellian<D, T>(w0, ibK);
+  // Eqs. relaxation time and taua; the artificial part only with C_a > 0
+  T tau = gas.mu * g0.it * g0.ir + tau_t;
   if (gas.C_a != T(0)) {
-    const F2 plr = F2(gs.rho * gs.il);
+    const F2 plr = F2(gs.rho * gs.th);
     const T pl = plr.v.x, pr = plr.v.y;
     tau += g_div(gas.C_a * g_abs(pr - pl), pr + pl) * dt;
   }
   *tau_out = tau;
-  T Tc[6], r1, r4, r5;
+  TimeCoef<T> c;
+  EqTerms<D, T> q;
   if constexpr (RAR) {
-    const T drho = face_drho<D, T, MULTID>(g0, w0, in, dxl, dxr, g0.ir, bK, K);
+    equilibrium_terms<D, T, MULTID>(g0, w0, in, idxl, idxr, bK, ibK, q);
+    const T drho = face_drho<D, T>(g0, q, w0, in, idxl, idxr);
     const T eps = drho > T(1e-30) * g0.rho ? g_div(tau * drho, g0.rho) : tau * T(1e-30);
-    time_coeffs_hat<T>(dt, tau, eps, Tc, r1, r4, r5);
+    time_coeffs_hat<T>(dt, tau, eps, c);
   } else {
-    time_coeffs<T>(dt, tau, Tc, r1, r4, r5);
+    time_coeffs<T>(dt, tau, c);
   }
-  if (abar_t0) {
-    r1 = T(-1);
-    r4 = r5 = T(0);
-  }
-  const T i0 = g0.ir;
-
   T rhs[nv];
-  // the two sides of the initial state: slopes a (normal), b (tangential), A (Eq. initialf0)
   {
-    Trans<D, F2> ts;
-    transverse<D, F2>(gs, F2(K), ts);
-    F2 a[nv], b[Dims<D>::nt][nv], A[nv], r[nv];
-    const F2 ir = gs.ir;
+    F2 sn[nv], st[Dims<D>::nt][nv], U0[D], rs[nv], Fs[nv];
 #pragma unroll
-    for (int m = 0; m < nv; ++m) r[m] = F2(F2(in.s(0, m), in.s(1, m)) * ir);
-    slope<D, F2>(gs, F2(bK), r, a);
+    for (int m = 0; m < nv; ++m) sn[m] = F2(in.s(0, m), in.s(1, m));
     if (MULTID) {
 #pragma unroll
-      for (int q = 0; q < D - 1; ++q) {
+      for (int s = 0; s < D - 1; ++s)
 #pragma unroll
-        for (int m = 0; m < nv; ++m) r[m] = F2(F2(in.t(0, q, m), in.t(1, q, m)) * ir);
-        slope<D, F2>(gs, F2(bK), r, b[q]);
-      }
+        for (int m = 0; m < nv; ++m) st[s][m] = F2(in.t(0, s, m), in.t(1, s, m));
     }
-    // A from the compatibility condition at t = 0: <(a u + b v + A) psi> = 0 (full line)
-    {
-      F2 uf[7];
-      u_full<D, F2>(gs, uf);
 #pragma unroll
-      for (int m = 0; m < nv; ++m) r[m] = F2(0.0f);
-      amom<D, F2>(uf, ts, 1, -1, a, F2(-1.0f), r);
-      if (MULTID) {
-#pragma unroll
-        for (int q = 0; q < D - 1; ++q) amom<D, F2>(uf, ts, 0, q, b[q], F2(-1.0f), r);
-      }
-      slope<D, F2>(gs, F2(bK), r, A);
-    }
-    // Abar rhs r4 rho/rho0 <(a u + b v) psi> + r5 rho/rho0 <A psi> and the flux
-    // rho [T3 <u psi> + T5 <u A psi> + T4 (<u^2 a psi> + <u v b psi>)], over each side's half line
-    const F2 s4 = F2(F2(r4 * i0) * gs.rho), s5 = F2(F2(r5 * i0) * gs.rho), s4f = F2(F2(Tc[4]) * gs.rho);
-    F2 rh2[nv], F2s[nv];
-#pragma unroll
-    for (int m = 0; m < nv; ++m) rh2[m] = F2s[m] = F2(0.0f);
-    amom2<D, F2>(hs, ts, 1, -1, a, s4, rh2, s4f, F2s);
-    amom2<D, F2>(hs, ts, 0, -1, A, s5, rh2, F2(F2(Tc[5]) * gs.rho), F2s);
-    {
-      F2 m[nv];
-      psi_mean<D, F2>(hs + 1, ts.m1, m);  // <u psi> over the half line
-      const F2 s3 = F2(F2(Tc[3]) * gs.rho);
-#pragma unroll
-      for (int q = 0; q < nv; ++q) F2s[q] += s3 * m[q];
-    }
-    if (MULTID) {
-#pragma unroll
-      for (int q = 0; q < D - 1; ++q) amom2<D, F2>(hs, ts, 0, q, b[q], s4, rh2, s4f, F2s);
-    }
+    for (int i = 0; i < D; ++i) U0[i] = F2(g0.U[i]);
+    side_terms<D, F2, MULTID>(gs, e, sn, st, U0, F2(bK), F2(ibK), F2(c.T3), F2(c.Dn), F2(c.r4), F2(c.r45), rs, Fs);
 #pragma unroll
     for (int m = 0; m < nv; ++m) {
-      rhs[m] = rh2[m].v.x + rh2[m].v.y;
-      F[m] = F2s[m].v.x + F2s[m].v.y;
+      rhs[m] = rs[m].v.x + rs[m].v.y;
+      F[m] = Fs[m].v.x + Fs[m].v.y;
     }
   }
-
-  // equilibrium g0: Eq. eqlgform slopes from W_j -> w0 -> W_{j+1} (and the mean tangential slope)
-  Trans<D, T> tr0;
-  transverse<D, T>(g0, K, tr0);
-  T oF[7], oP[7];
-  u_full<D, T>(g0, oF);
-  u_half<D, T>(g0, T(1), oP);
-  {
-    // lane x: abar_l on u > 0; lane y: abar_r on u < 0 (table = full line minus u > 0)
-    const T fl = i0 * idxl, fr = i0 * idxr;
-    Maxw<D, F2> g02;
-    g02.rho = F2(g0.rho);
-    g02.ir = F2(g0.ir);
-#pragma unroll
-    for (int i = 0; i < D; ++i) g02.U[i] = F2(g0.U[i]);
-    g02.lam = F2(g0.lam);
-    g02.il = F2(g0.il);
-    g02.c = F2(g0.c);
-    g02.f4 = F2(g0.f4);
-    Trans<D, F2> t02;
-#pragma unroll
-    for (int b = 0; b <= D; ++b) {
-      t02.m1[b] = F2(tr0.m1[b]);
-#pragma unroll
-      for (int c = 0; c <= D; ++c) t02.m2[b][c] = F2(tr0.m2[b][c]);
-    }
-    F2 r[nv], ab[nv], half[7];
-#pragma unroll
-    for (int m = 0; m < nv; ++m) r[m] = F2(F2(w0[m] - in.c(0, m), in.c(1, m) - w0[m]) * F2(fl, fr));
-#pragma unroll
-    for (int n = 0; n < 7; ++n) half[n] = F2(oP[n], oF[n] - oP[n]);
-    slope<D, F2>(g02, F2(bK), r, ab);
-    F2 rh2[nv], F2s[nv];
-#pragma unroll
-    for (int m = 0; m < nv; ++m) rh2[m] = F2s[m] = F2(0.0f);
-    amom2<D, F2>(half, t02, 1, -1, ab, F2(r1), rh2, F2(Tc[1] * g0.rho), F2s);
-#pragma unroll
-    for (int m = 0; m < nv; ++m) {
-      rhs[m] += rh2[m].v.x + rh2[m].v.y;
-      F[m] += F2s[m].v.x + F2s[m].v.y;
-    }
-    if (MULTID) {
-      const T s1f = Tc[1] * g0.rho;
-      T rr[nv], abt[nv];
-#pragma unroll
-      for (int q = 0; q < D - 1; ++q) {
-#pragma unroll
-        for (int m = 0; m < nv; ++m) rr[m] = T(0.5) * (in.t(0, q, m) + in.t(1, q, m)) * i0;
-        slope<D, T>(g0, bK, rr, abt);
-        amom2<D, T>(oF, tr0, 0, q, abt, r1, rhs, s1f, F);
-      }
-    }
-  }
-  // Abar from the compatibility condition integrated over [0, dt]; flux rho0 <u (T0 + T2 Abar) psi>
-  {
-    T Ab[nv];
-    slope<D, T>(g0, bK, rhs, Ab);
-#pragma unroll
-    for (int m = 0; m < nv; ++m) Ab[m] *= Tc[2];
-    Ab[0] += Tc[0];
-    amom<D, T>(oF, tr0, 1, -1, Ab, g0.rho, F);
-  }
+  if constexpr (!RAR) equilibrium_terms<D, T, MULTID>(g0, w0, in, idxl, idxr, bK, ibK, q);
+  close_flux<D, T>(g0, q, c, abar_t0, bK, ibK, rhs, F);
 }
 
 // face_flux_ps with the inputs in arrays, the inverse centre-to-face distances given.
 template <int D, bool MULTID, bool RAR = false>
-GKS_FN void face_flux_ps(const float* wl, const float* wr, const float* cl, const float* cr, const float* sl,
-                         const float* sr, const float (*tl)[D + 2], const float (*tr)[D + 2], float dxl, float dxr,
-                         float idxl, float idxr, float tau_t, float dt, const Gas<float>& gas, int abar_t0, float* F,
-                         float* tau_out) {
+GKS_FN void face_flux_ps_inv(const float* wl, const float* wr, const float* cl, const float* cr, const float* sl,
+                             const float* sr, const float (*tl)[D + 2], const float (*tr)[D + 2], float idxl,
+                             float idxr, float tau_t, float dt, const Gas<float>& gas, int abar_t0, float* F,
+                             float* tau_out) {
   const FaceArrays<D, float> in{sl, sr, cl, cr, tl, tr};
-  face_flux_ps<D, MULTID, RAR>(wl, wr, in, dxl, dxr, idxl, idxr, tau_t, dt, gas, abar_t0, F, tau_out);
+  face_flux_ps<D, MULTID, RAR>(wl, wr, in, idxl, idxr, tau_t, dt, gas, abar_t0, F, tau_out);
 }
 
-// face_flux_ps with the inputs in arrays.
+// face_flux_ps with the inputs in arrays and the centre-to-face distances.
 template <int D, bool MULTID, bool RAR = false>
 GKS_FN void face_flux_ps(const float* wl, const float* wr, const float* cl, const float* cr, const float* sl,
                          const float* sr, const float (*tl)[D + 2], const float (*tr)[D + 2], float dxl, float dxr,
                          float tau_t, float dt, const Gas<float>& gas, int abar_t0, float* F, float* tau_out) {
-  face_flux_ps<D, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, dxl, dxr, g_rcp(dxl), g_rcp(dxr), tau_t, dt, gas,
-                               abar_t0, F, tau_out);
+  face_flux_ps_inv<D, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, g_rcp(dxl), g_rcp(dxr), tau_t, dt, gas, abar_t0, F,
+                                   tau_out);
 }
 
 }  // namespace gks

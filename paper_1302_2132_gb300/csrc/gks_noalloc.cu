@@ -56,7 +56,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreadsNA) rate_partials(const double* W, long ncell, double gamma, double h0,
                                                             double h1, double h2, double* scratch) {
   __shared__ double red[gks::kMaxWarps];
-  const double h[3] = {h0, h1, h2};
+  const double ih[3] = {1.0 / h0, 1.0 / h1, 1.0 / h2};
   double rmax = 0.0;
   int bad = 0;
   for (long c = (long)blockIdx.x * kThreadsNA + threadIdx.x; c < ncell; c += (long)gridDim.x * kThreadsNA) {
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kThreadsNA) rate_partials(const double* W, lon
       bad = 1;
       continue;
     }
-    rmax = fmax(rmax, gks::cell_rate<D, double>(w, gamma, h));
+    rmax = fmax(rmax, gks::cell_rate_inv<D, double>(w, gamma, ih));
   }
   const double m = gks::block_max<double>(rmax, red);
   const int any_bad = __syncthreads_or(bad);

@@ -601,25 +601,21 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return v;
 }
 
-// CFL rate of one cell: sum_d (|U_d| + c) / dx_d, c = sqrt(gamma p / rho).
-template <int D, class R>
-__device__ __forceinline__ R cell_rate(const R* w, R gamma, const R* h) {
-  const R p = pressure_of<R>(D, gamma, w);
-  const R cs = g_sqrt(g_div(gamma * p, w[0]));
-  R r = R(0);
-#pragma unroll
-  for (int d = 0; d < D; ++d) r += g_div(g_abs(g_div(w[1 + d], w[0])) + cs, h[d]);
-  return r;
-}
-
-// The same rate from the inverse cell widths, with one reciprocal of the density and one square root.
+// CFL rate of one cell, sum_d (|U_d| + c) / dx_d, c = sqrt(gamma p / rho), from the inverse cell widths, with one
+// reciprocal of the density and one square root.  The step kernel (for its successor) and the rate kernel
+// (for a state that was copied in) take it, every operation rounded as written, so that a run restarted
+// from a copied-out state takes the same time steps to the last bit.
 template <int D, class R>
 __device__ __forceinline__ R cell_rate_inv(const R* w, R gamma, const R* ih) {
   const R ir = g_rcp(w[0]);
-  const R cs = g_sqrt(gamma * pressure_of<R>(D, gamma, w) * ir);
+  R q = g_mul_rn<R>(w[1], w[1]);
+#pragma unroll
+  for (int d = 1; d < D; ++d) q = g_fma_rn<R>(w[1 + d], w[1 + d], q);
+  const R p = g_mul_rn<R>(gamma - R(1), g_fma_rn<R>(R(-0.5), g_mul_rn<R>(q, ir), w[D + 1]));
+  const R cs = g_sqrt(g_mul_rn<R>(g_mul_rn<R>(gamma, p), ir));
   R r = R(0);
 #pragma unroll
-  for (int d = 0; d < D; ++d) r += (g_abs(w[1 + d] * ir) + cs) * ih[d];
+  for (int d = 0; d < D; ++d) r = g_fma_rn<R>(g_add_rn<R>(g_abs(g_mul_rn<R>(w[1 + d], ir)), cs), ih[d], r);
   return r;
 }
 
@@ -1049,7 +1045,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     // Inputs of one face in its frame (velocity order: normal first, then tangential axes).
     struct FaceIn {
       R wl[nv], wr[nv], cl[nv], cr[nv], sl[nv], sr[nv], tl[Dims<D>::nt][nv], tr[Dims<D>::nt][nv];
-      R dxl, dxr, idxl, idxr, tau_t;
+      R idxl, idxr, tau_t;  // inverse centre-to-face distances
       int ax, ci, cj, ck, perm[3];
     };
     // AX: the face's axis when the caller knows it at compile time (the frame permutation, strides
@@ -1186,8 +1182,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
           }
         }
       }
-      in.dxl = R(0.5) * h1;
-      in.dxr = R(0.5) * h2;
       {
         const R* iwn = ax == 0 ? iwx : (ax == 1 ? iwy : iwz);
         in.idxl = R(2) * iwn[pn - 1];
@@ -1250,8 +1244,8 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
             }
           }
           F2 F[nv], tau;
-          face_flux<D, F2, MULTID, false>(wl, wr, cl, cr, sl, sr, tl, tr, F2(a.dxl, b.dxl), F2(a.dxr, b.dxr),
-                                          F2(a.tau_t, b.tau_t), F2(dt), gas2, g.abar_t0, F, &tau);
+          face_flux_inv<D, F2, MULTID, false>(wl, wr, cl, cr, sl, sr, tl, tr, F2(a.idxl, b.idxl), F2(a.idxr, b.idxr),
+                                              F2(a.tau_t, b.tau_t), F2(dt), gas2, g.abar_t0, F, &tau);
           R Fa[nv], Fb[nv];
 #pragma unroll
           for (int v = 0; v < nv; ++v) {
@@ -1282,11 +1276,11 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
           if constexpr (std::is_same<R, float>::value && D <= 2) {
             // single precision: the two sides of the face on the paired FP32 instructions (in 3D the
             // paired body does not fit the register budget of two CTAs per SM)
-            face_flux_ps<D, MULTID, RAR>(in.wl, in.wr, in.cl, in.cr, in.sl, in.sr, in.tl, in.tr, in.dxl, in.dxr,
-                                         in.idxl, in.idxr, in.tau_t, dt, gas, g.abar_t0, F, &tau);
+            face_flux_ps_inv<D, MULTID, RAR>(in.wl, in.wr, in.cl, in.cr, in.sl, in.sr, in.tl, in.tr, in.idxl, in.idxr,
+                                             in.tau_t, dt, gas, g.abar_t0, F, &tau);
           } else {
-            face_flux<D, R, MULTID, RAR>(in.wl, in.wr, in.cl, in.cr, in.sl, in.sr, in.tl, in.tr, in.dxl, in.dxr,
-                                         in.tau_t, dt, gas, g.abar_t0, F, &tau);
+            face_flux_inv<D, R, MULTID, RAR>(in.wl, in.wr, in.cl, in.cr, in.sl, in.sr, in.tl, in.tr, in.idxl, in.idxr,
+                                             in.tau_t, dt, gas, g.abar_t0, F, &tau);
           }
           if (f < G::NFX)
             store(f, in, F, std::integral_constant<int, 0>{});

@@ -398,10 +398,11 @@ def probe_cvt():
     return a.value, b.value
 
 
-def face_op_count(dim, expand=True, with_recon=True):
-    """Static per-face operation count of the flux code: (add, mul, div, sqrt, exp, erfc)."""
+def face_op_count(dim, expand=True, with_recon=True, closed_form=False):
+    """Static per-face operation count of the flux in moment tables, or of the closed form that the
+    kernels evaluate: (add, mul, div, sqrt, exp, erfc)."""
     c = (ctypes.c_longlong * 6)()
-    load().gks_face_op_count(dim, int(expand), int(with_recon), c)
+    load().gks_face_op_count(dim, int(expand), int(with_recon) + 2 * int(closed_form), c)
     return tuple(c)
 
 
