@@ -114,6 +114,93 @@ __global__ void __launch_bounds__(kThreads) rate_kernel(const __grid_constant__ 
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&A.ctrl->status, 1u);
 }
 
+// Residual norms of the step that took Win to Wout: l2 += (dW/dt)^2, linf = max |dW|/dt, total += W volume (area: per
+// cell, body-fitted grids; null: the product of the widths).  It runs after the last step of a call only, so the
+// step kernels carry none of it.  Doubles run at 1/64 of the FP32 rate on this part and bound it: three double
+// operations per value, dt divided out once per CTA, and a reduction in shared memory in which one warp
+// adds up one quantity (T/32 + 5 additions a lane, against five per quantity in every warp).
+// Accumulated inside the step kernel the norms took 115 us of that step at 1024^2 with the double state, and
+// their code 5% of every other step (the 49-step call 4.82 -> 4.53 ms, 160^3 x 7 steps 7.65 -> 6.67 ms).
+template <int D, int PREC>
+__global__ void __launch_bounds__(kThreads) residual_kernel(const __grid_constant__ StepArgs A, const double* area) {
+  using S = typename PrecT<PREC>::S;
+  constexpr int NV = D + 2, T = kThreads, NW = T / 32;
+  using M = S;
+  __shared__ double sums[2 * NV * T];
+  __shared__ M maxs[NV * T];
+  const DevGrid& g = A.g;
+  const double dt = A.ctrl->last_dt;
+  if (dt == 0.0) return;  // past t_end: the state was carried over
+  const int tid = threadIdx.x;
+  double s2[NV], tot[NV];
+  M mx[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    s2[v] = tot[v] = 0.0;
+    mx[v] = M(0);
+  }
+  const S* W0 = (const S*)A.Win;
+  const S* W1 = (const S*)A.Wout;
+  for (long c = (long)blockIdx.x * T + tid; c < g.ncell; c += (long)gridDim.x * T) {
+    double vol;
+    if (area) {
+      vol = area[c];
+    } else {
+      vol = g.w[0][(int)(c % g.n[0]) + kWG];
+      if (D >= 2) vol *= g.w[1][(int)((c / g.n[0]) % g.n[1]) + kWG];
+      if (D >= 3) vol *= g.w[2][(int)(c / ((long)g.n[0] * g.n[1])) + kWG];
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const long i = (long)v * g.ncell + c;
+      double w, r;
+      if constexpr (PREC == PREC_F32) {  // float pairs: the difference of the high words is exact up to rounding
+        const float h1 = W1[i], l1 = A.Wout_lo[i];
+        const float d = (h1 - W0[i]) + (l1 - A.Win_lo[i]);
+        w = f2d(h1) + f2d(l1);
+        r = f2d(d);
+        mx[v] = fmaxf(mx[v], fabsf(d));
+      } else {
+        w = W1[i];
+        r = w - W0[i];
+        mx[v] = fmax(mx[v], fabs(r));
+      }
+      s2[v] += r * r;
+      tot[v] += w * vol;
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    sums[v * T + tid] = s2[v];
+    sums[(NV + v) * T + tid] = tot[v];
+    maxs[v * T + tid] = mx[v];
+  }
+  __syncthreads();
+  const int lane = tid & 31;
+  for (int q = tid >> 5; q < 3 * NV; q += NW) {
+    if (q < 2 * NV) {
+      double s = sums[q * T + lane];
+#pragma unroll
+      for (int k = 1; k < NW; ++k) s += sums[q * T + lane + 32 * k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) {
+        if (q < NV)
+          atomicAdd(&A.ctrl->l2[q], s / dt / dt);
+        else
+          atomicAdd(&A.ctrl->total[q - NV], s);
+      }
+    } else {
+      M m = maxs[(q - 2 * NV) * T + lane];
+#pragma unroll
+      for (int k = 1; k < NW; ++k) m = fmax(m, maxs[(q - 2 * NV) * T + lane + 32 * k]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) atomic_max_nonneg(&A.ctrl->linf[q - 2 * NV], (double)m / dt);
+    }
+  }
+}
+
 template <int unused = 0>
 __global__ void set_params_kernel(Ctrl* c, double dt_fixed, double cfl, double t_end) {
   c->dt_fixed = dt_fixed;

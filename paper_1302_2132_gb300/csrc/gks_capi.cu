@@ -272,7 +272,7 @@ void launch_step(gks_handle* h, const StepArgs& A) {
 }
 
 // Arguments of the step that starts at absolute step index s.
-StepArgs step_args(const gks_handle* h, long long s, int resid) {
+StepArgs step_args(const gks_handle* h, long long s) {
   StepArgs A = h->base;
   const int cur = (int)(s & 1);
   A.Win = h->W[cur];
@@ -281,7 +281,6 @@ StepArgs step_args(const gks_handle* h, long long s, int resid) {
   A.Wout_lo = h->Wlo[cur ^ 1];
   A.slot = (int)(s % 3);
   A.tslot = cur;
-  A.resid = resid;
   if (h->transport) {
     A.f1 = h->RK[cur];
     A.f2 = h->RW[cur];
@@ -322,7 +321,7 @@ void launch_rate_d(gks_handle* h, const StepArgs& A, unsigned blocks) {
 }
 
 gks_status launch_rate(gks_handle* h) {
-  StepArgs A = step_args(h, h->step, 0);
+  StepArgs A = step_args(h, h->step);
   if (h->curv) {
     launch_curv_rate(h->prec, A, h->cg, h->stream);
     GKS_CK(h, cudaGetLastError());
@@ -337,6 +336,27 @@ gks_status launch_rate(gks_handle* h) {
     launch_rate_d<3>(h, A, blocks);
   GKS_CK(h, cudaGetLastError());
   return GKS_OK;
+}
+
+template <int D>
+void launch_residual_d(gks_handle* h, const StepArgs& A, unsigned blocks) {
+  const double* area = h->curv ? h->cg.area : nullptr;
+  if (h->prec == PREC_F64)
+    residual_kernel<D, PREC_F64><<<blocks, kThreads, 0, h->stream>>>(A, area);
+  else if (h->prec == PREC_F32)
+    residual_kernel<D, PREC_F32><<<blocks, kThreads, 0, h->stream>>>(A, area);
+  else
+    residual_kernel<D, PREC_F32D><<<blocks, kThreads, 0, h->stream>>>(A, area);
+}
+
+void launch_residual(gks_handle* h, const StepArgs& A) {
+  const unsigned blocks = std::min<unsigned>(grid_for(h->ncell, kThreads), 152u * 4u);
+  if (h->D == 1)
+    launch_residual_d<1>(h, A, blocks);
+  else if (h->D == 2)
+    launch_residual_d<2>(h, A, blocks);
+  else
+    launch_residual_d<3>(h, A, blocks);
 }
 
 template <int D>
@@ -491,7 +511,7 @@ gks_status autotune(gks_handle* h) {
   cudaEvent_t e0, e1;
   GKS_CK(h, cudaEventCreate(&e0));
   GKS_CK(h, cudaEventCreate(&e1));
-  const StepArgs A = step_args(h, h->step, 0);
+  const StepArgs A = step_args(h, h->step);
   const std::vector<int> cand = tile_candidates(h);
   std::vector<float> fastest(cand.size(), 1e30f);
   for (int v : cand) launch_step_variant(h, A, v);  // warm-up
@@ -1000,7 +1020,7 @@ gks_status gks_step(gks_handle* h, double dt, double cfl, int nsteps, double t_e
       if (it == h->graphs.end()) {
         cudaGraph_t graph;
         GKS_CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        for (int k = 0; k < kGraphChunk; ++k) launch_step(h, step_args(h, k, 0));
+        for (int k = 0; k < kGraphChunk; ++k) launch_step(h, step_args(h, k));
         cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
         if (e != cudaSuccess) return cuda_fail(h, e, "graph capture");
         cudaGraphExec_t exec;
@@ -1014,7 +1034,7 @@ gks_status gks_step(gks_handle* h, double dt, double cfl, int nsteps, double t_e
       remaining -= kGraphChunk;
       continue;
     }
-    const StepArgs A = step_args(h, h->step, remaining == 1);
+    const StepArgs A = step_args(h, h->step);
     if (h->timing) {
       cudaEvent_t e0, e1;
       GKS_CK(h, cudaEventCreate(&e0));
@@ -1028,6 +1048,10 @@ gks_status gks_step(gks_handle* h, double dt, double cfl, int nsteps, double t_e
       launch_step(h, A);
     }
     GKS_CK(h, cudaGetLastError());
+    if (remaining == 1) {  // residual norms of the call's last step
+      launch_residual(h, A);
+      GKS_CK(h, cudaGetLastError());
+    }
     h->step += 1;
     remaining -= 1;
   }
@@ -1093,7 +1117,7 @@ static gks_status get_diag(gks_handle* h, int what, void* out, int memspace, int
     if (s) return s;
     dst = h->staging;
   }
-  const StepArgs A = step_args(h, h->step, 0);
+  const StepArgs A = step_args(h, h->step);
   if (h->curv) {
     if (what == 0 && h->base.g.turb_model == GKS_TURB_NONE) {
       GKS_CK(h, cudaMemsetAsync(dst, 0, bytes, h->stream));

@@ -174,7 +174,7 @@ struct CurvTileGeom {
   static constexpr int HX = X + 2 * H, HY = Y + 2 * H, NH = HX * HY;
   static constexpr int NFX = (X + 1) * Y, NFY = X * (Y + 1), NF = NFX + NFY;
   static constexpr int TX = X + 2, TY = Y + 2, NT = TX * TY;  // tile and first ring (tau)
-  template <class R, bool TR = false> static constexpr size_t smem_bytes() {
+  template <class R, bool TR = false> __host__ __device__ static constexpr size_t smem_bytes() {
     return sizeof(R) * (4 * (size_t)NH + 8 * (size_t)NF + 4 * (size_t)NF + NT + (TR ? 4 * (size_t)NH + 2 * (size_t)NF : 0)) +
            sizeof(float) * 4 * X * Y;
   }
@@ -578,12 +578,9 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
 
   // the next step may start its launch (it waits for this kernel's completion before its reads)
   if (MODE == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // ---- update, next CFL rate, physical check, residual norms ---------------------------------
+  // ---- update, next CFL rate, physical check ------------------------------------------------
   R rmax = R(0);
   unsigned bad = 0u;
-  double racc[12];
-#pragma unroll
-  for (int q = 0; q < 12; ++q) racc[q] = 0.0;
   for (int l = tid; l < X * Y; l += T) {
     const int li = l % X, lj = l / X;
     const int gi = ox + li, gj = oy + lj;
@@ -597,18 +594,11 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
     for (int v = 0; v < 4; ++v) {
       const R net = Fs[v * NF + fa + 1] - Fs[v * NF + fa] + Fs[v * NF + fc + X] - Fs[v * NF + fc];
       const long gidx = (long)v * g.ncell + c;
-      double wd;
       if (PREC == PREC_F64) {
         const double w_old = (double)Ws[v * NH + hidx];
         const double w = w_old - (double)net / G.area[c];
         ((double*)A.Wout)[gidx] = w;
         wn[v] = (R)w;
-        wd = w;
-        if (A.resid) {
-          const double r = (w - w_old) / dt_d;
-          racc[v] += r * r;
-          racc[4 + v] = fmax(racc[4 + v], fabs(r));
-        }
       } else {
         const R inc = -net * ia;
         if (PREC == PREC_F32) {
@@ -622,20 +612,12 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
           ((float*)A.Wout)[gidx] = nhi;
           A.Wout_lo[gidx] = nlo;
           wn[v] = nhi;
-          wd = (double)nhi + (double)nlo;
         } else {
-          const double w = ((const double*)A.Win)[gidx] + (double)inc;
+          const double w = ((const double*)A.Win)[gidx] + f2d(inc);
           ((double*)A.Wout)[gidx] = w;
           wn[v] = (R)w;
-          wd = w;
-        }
-        if (A.resid) {
-          const double r = (double)inc / dt_d;
-          racc[v] += r * r;
-          racc[4 + v] = fmax(racc[4 + v], fabs(r));
         }
       }
-      if (A.resid) racc[8 + v] += wd * G.area[c];
     }
     if (!physical<2, R>(kc.gamma, wn)) bad = 1u;
     if (TR) {  // rho k, rho omega (the transport kernel's arithmetic)
@@ -683,16 +665,6 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
   const unsigned long long bmax = block_max_rate<R>(rmax, red);
   if (tid == 0) atomicMax(&A.ctrl->rate[(A.slot + 1) % 3], bmax);
   if (__syncthreads_or(bad) && tid == 0) atomicOr(&A.ctrl->status, 1u);
-  if (A.resid) {
-    for (int v = 0; v < 4; ++v) {
-      double s_ = block_sum(racc[v], red);
-      if (tid == 0) atomicAdd(&A.ctrl->l2[v], s_);
-      s_ = block_sum(racc[8 + v], red);
-      if (tid == 0) atomicAdd(&A.ctrl->total[v], s_);
-      const double m = block_max<double>(racc[4 + v], red);
-      if (tid == 0) atomic_max_nonneg(&A.ctrl->linf[v], m);
-    }
-  }
 }
 
 template <int PREC, int V, int MODE = 0, bool MD = false, int RC = 0, bool TR = false, bool RAR = false>

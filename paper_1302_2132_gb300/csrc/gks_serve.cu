@@ -244,7 +244,6 @@ bool admit(gks_server* s, Req* r) {
     A.Wout_lo = Wlo[c ^ 1];
     A.slot = ph % 3;
     A.tslot = c;
-    A.resid = 0;
     S.args[ph] = A;
   }
   S.stop_at = s->step + q.nsteps;

@@ -172,7 +172,6 @@ struct StepArgs {
                    // for j = 0 .. n_d (x fastest), in the arithmetic type (k-omega transport input)
   int slot;    // rate slot read by this step (step index mod 3)
   int tslot;   // time slot read by this step (step index mod 2)
-  int resid;   // accumulate residual norms in this step
   // k-omega transport fused into the body-fitted step (f1, f2 are then rho k, rho omega): outputs
   // and the closure coefficients (double, and float for the single-precision kernels)
   void* RKout;
@@ -818,7 +817,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
   const Consts<R> kc = make_consts<R>(g);
   __shared__ R s_dtr;   // the time step in the arithmetic type, converted once per CTA
   __shared__ int s_end;  // the time step is zero (t_end reached)
-  __shared__ double s_dt;
 
   // ---- stage the tile with two halo layers, the ring's turbulence fields and the low words ------
   // In-grid cells are copied asynchronously; ghost cells are resolved by the boundary rules.  A tile
@@ -984,7 +982,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     if (c_tend > 0.0) dtv = (c_t >= c_tend) ? 0.0 : fmin(dtv, c_tend - c_t);
     s_dtr = (R)dtv;
     s_end = dtv == 0.0;
-    s_dt = dtv;
     if (b == 0) {
       Ctrl* c = A.ctrl;
       c->t[A.tslot ^ 1] = c_t + dtv;
@@ -1012,7 +1009,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     }
   }
   __syncthreads();
-  const double dt_d = s_dt;
   if (s_end) {  // t_end reached: carry the state over
     for (int l = tid; l < G::NC; l += kThreads) {
       const int li = l % X, lj = (l / X) % Y, lk = l / (X * Y);
@@ -1310,11 +1306,8 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
   }
   __syncthreads();
 
-  // ---- conservative update, CFL rate of the new state, residual norms --------------------------
+  // ---- conservative update, CFL rate of the new state ------------------------------------------
   R rmax = R(0);
-  double racc[3 * 5];
-#pragma unroll
-  for (int q = 0; q < 15; ++q) racc[q] = 0.0;
   unsigned int bad = 0;
 #pragma unroll
   for (int qc = 0; qc < NCI; ++qc) {
@@ -1343,11 +1336,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
 #pragma unroll
     for (int d = 0; d < D; ++d) ih[d] = (d == 0 ? iwx[li + H] : (d == 1 ? iwy[lj + H] : iwz[lk + H]));
     R wn[nv];
-    double vol = 1.0;
-    if (A.resid) {  // cell volume from the double-precision widths
-      const int gc[3] = {gi, gj, gk};
-      for (int d = 0; d < D; ++d) vol *= g.w[d][gc[d] + kWG];
-    }
     // the cell's old state: staged in shared memory (FP64, float pair), else loaded into wold above
     const int hidx = ((lk + (D >= 3 ? H : 0)) * HY + (lj + (D >= 2 ? H : 0))) * HX + (li + H);
 #pragma unroll
@@ -1355,22 +1343,14 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       const long gidx = (long)v * g.ncell + c;
       if constexpr (PREC == PREC_F64) {
         double w = (double)Ws[v * G::NH + hidx];
-        const double w_old = w;
 #pragma unroll
         for (int d = 0; d < D; ++d) w -= ((double)Fs[v * G::NF + fp[d]] - (double)Fs[v * G::NF + fm[d]]) / (double)h[d];
         ((double*)A.Wout)[gidx] = w;
         wn[v] = (R)w;
-        if (A.resid) {
-          const double r = (w - w_old) / dt_d;
-          racc[v] += r * r;
-          racc[5 + v] = fmax(racc[5 + v], fabs(r));
-          racc[10 + v] += w * vol;
-        }
       } else {
         R inc = R(0);
 #pragma unroll
         for (int d = 0; d < D; ++d) inc -= (Fs[v * G::NF + fp[d]] - Fs[v * G::NF + fm[d]]) * ih[d];
-        double wd = 0.0;
         if constexpr (PREC == PREC_F32) {
           // (hi, lo) += inc with an error-free sum, then renormalise
           const float hi = (float)Ws[v * G::NH + hidx], lo = Lo[v * G::NC + l];
@@ -1383,18 +1363,10 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
           ((float*)A.Wout)[gidx] = nhi;
           A.Wout_lo[gidx] = nlo;
           wn[v] = nhi;
-          if (A.resid) wd = (double)nhi + (double)nlo;
         } else {
           const double w = wold[qc][v] + f2d(inc);
           ((double*)A.Wout)[gidx] = w;
           wn[v] = (float)Ws[v * G::NH + hidx] + inc;  // the new state in float, for the rate and status
-          wd = w;
-        }
-        if (A.resid) {
-          const double r = (double)inc / dt_d;
-          racc[v] += r * r;
-          racc[5 + v] = fmax(racc[5 + v], fabs(r));
-          racc[10 + v] += wd * vol;
         }
       }
     }
@@ -1405,16 +1377,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
   const unsigned long long bmax = block_max_rate<R>(rmax, red);
   if (tid == 0) atomicMax(&A.ctrl->rate[(A.slot + 1) % 3], bmax);
   if (__syncthreads_or(bad) && tid == 0) atomicOr(&A.ctrl->status, 1u);
-  if (A.resid) {
-    for (int v = 0; v < nv; ++v) {
-      double s = block_sum(racc[v], red);
-      if (tid == 0) atomicAdd(&A.ctrl->l2[v], s);
-      s = block_sum(racc[10 + v], red);
-      if (tid == 0) atomicAdd(&A.ctrl->total[v], s);
-      const double m = block_max<double>(racc[5 + v], red);
-      if (tid == 0) atomic_max_nonneg(&A.ctrl->linf[v], m);
-    }
-  }
 }
 
 template <int D, int V = 0> constexpr int min_blocks(int prec) {
