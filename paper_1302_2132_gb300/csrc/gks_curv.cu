@@ -235,24 +235,6 @@ __global__ void __launch_bounds__(kCurvThreads) curv_tau_kernel(const __grid_con
   ((R*)out)[c] = (g_div(kc.mu, p) + tau_t) * g_abs(div);
 }
 
-// CFL rate of a cell on the curvilinear grid: sum over its faces of (|U.n| + c) L / (2 A).
-template <class R>
-__device__ __forceinline__ R curv_rate(const R* w, R gamma, const CurvGeom& G, int n0, int i, int j, long c) {
-  const FaceView<R> fi{(const R*)G.face[0], G.nf[0]}, fj{(const R*)G.face[1], G.nf[1]};
-  const R ir = g_rcp(w[0]);
-  const R u = w[1] * ir, v = w[2] * ir;
-  const R p = pressure_of<R>(2, gamma, w);
-  const R cs = g_sqrt(g_div(gamma * p, w[0]));
-  const long fa = (long)j * (n0 + 1) + i, fc = (long)j * n0 + i;
-  R r = R(0);
-#pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    r += (g_abs(u * fi(0, fa + s) + v * fi(1, fa + s)) + cs) * fi(2, fa + s);
-    r += (g_abs(u * fj(0, fc + s * n0) + v * fj(1, fc + s * n0)) + cs) * fj(2, fc + s * n0);
-  }
-  return R(0.5) * r * ((const R*)G.iarea)[c];
-}
-
 // CFL rate of the stored state into ctrl->rate[slot].
 template <int PREC>
 __global__ void __launch_bounds__(kCurvThreads) curv_rate_kernel(const __grid_constant__ StepArgs A,
@@ -593,20 +575,6 @@ __global__ void __launch_bounds__(KwTile::T) steady_komega_kernel(const __grid_c
   RW[c] = fmax(rw0 - rw / dw, rho * omega_floor);
 }
 
-// Local explicit step (CFL 1) of every cell: 2 A / sum_faces (|U.n| + c) L.
-template <int PREC>
-__global__ void __launch_bounds__(kCurvThreads) lts_kernel(const __grid_constant__ StepArgs A,
-                                                           const __grid_constant__ CurvGeom G, void* s_out) {
-  using R = typename PrecT<PREC>::R;
-  const DevGrid& g = A.g;
-  const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= g.ncell) return;
-  const Consts<R> kc = make_consts<R>(g);
-  R w[4];
-  load_stored<2, PREC>(g, A.Win, c, w);
-  ((R*)s_out)[c] = g_rcp(curv_rate<R>(w, kc.gamma, G, g.n[0], (int)(c % g.n[0]), (int)(c / g.n[0]), c));
-}
-
 inline unsigned blocks_for(long n) { return (unsigned)((n + kCurvThreads - 1) / kCurvThreads); }
 
 inline unsigned kw_tiles(const DevGrid& g) {
@@ -652,7 +620,11 @@ cudaError_t curv_metrics(const double* nodes, int n0, int n1, const bool periodi
 
 cudaError_t prepare_curv() {
   cudaError_t e = cudaSuccess;
-  const cudaError_t r[13] = {prepare_fused<PREC_F64, 0>(),   prepare_fused<PREC_F64, 1>(),
+  const cudaError_t r[17] = {prepare_one<PREC_F64, 0, 1, false, 0, false, false, true>(),
+                            prepare_one<PREC_F32, 0, 1, false, 0, false, false, true>(),
+                            prepare_one<PREC_F64, 3, 1, false, 0, false, false, true>(),
+                            prepare_one<PREC_F32, 3, 1, false, 0, false, false, true>(),
+                            prepare_fused<PREC_F64, 0>(),   prepare_fused<PREC_F64, 1>(),
                             prepare_fused<PREC_F32, 0>(),    prepare_fused<PREC_F32, 1>(),
                             prepare_fused<PREC_F32D, 0>(),   prepare_fused<PREC_F32D, 1>(),
                             prepare_fused<PREC_F64, 2>(),    prepare_fused<PREC_F32, 2>(),
@@ -697,28 +669,31 @@ void launch_curv_rate(int prec, const StepArgs& A, const CurvGeom& G, cudaStream
     curv_rate_kernel<PREC_F32D><<<blocks, kCurvThreads, 0, s>>>(A, G);
 }
 
-void launch_curv_residual(int prec, const StepArgs& A, const CurvGeom& G, const SteadyArgs& SA, cudaStream_t s) {
+namespace {
+template <int PREC>
+void residual_prec(const StepArgs& A, const CurvGeom& G, const SteadyArgs& SA, cudaStream_t s) {
   // 32 x 15 tiles on grids of two or more waves of them, 16 x 11 tiles (one wave of four CTAs per SM
-  // covers 107k cells) on the smaller grids and coarse multigrid levels
+  // covers 107k cells) on the smaller grids; first-order residuals (coarse multigrid levels) on 8 x 6 tiles
+  // while those make up no more than two waves of eight CTAs per SM (about 100k cells)
   const bool big = A.g.ncell >= 300000;
-  if (SA.multid) {
-    if (prec == PREC_F64)
-      big ? launch_fused<PREC_F64, 0, 1, true>(A, G, s, SA) : launch_fused<PREC_F64, 2, 1, true>(A, G, s, SA);
+  if (SA.first_order) {
+    if (A.g.ncell < 100000)
+      launch_fused<PREC, 3, 1, false, 0, false, false, true>(A, G, s, SA);
     else
-      big ? launch_fused<PREC_F32, 0, 1, true>(A, G, s, SA) : launch_fused<PREC_F32, 2, 1, true>(A, G, s, SA);
+      launch_fused<PREC, 0, 1, false, 0, false, false, true>(A, G, s, SA);
+  } else if (SA.multid) {
+    big ? launch_fused<PREC, 0, 1, true>(A, G, s, SA) : launch_fused<PREC, 2, 1, true>(A, G, s, SA);
   } else {
-    if (prec == PREC_F64)
-      big ? launch_fused<PREC_F64, 0, 1>(A, G, s, SA) : launch_fused<PREC_F64, 2, 1>(A, G, s, SA);
-    else
-      big ? launch_fused<PREC_F32, 0, 1>(A, G, s, SA) : launch_fused<PREC_F32, 2, 1>(A, G, s, SA);
+    big ? launch_fused<PREC, 0, 1>(A, G, s, SA) : launch_fused<PREC, 2, 1>(A, G, s, SA);
   }
 }
+}  // namespace
 
-void launch_curv_lts(int prec, const StepArgs& A, const CurvGeom& G, void* s_out, cudaStream_t s) {
+void launch_curv_residual(int prec, const StepArgs& A, const CurvGeom& G, const SteadyArgs& SA, cudaStream_t s) {
   if (prec == PREC_F64)
-    lts_kernel<PREC_F64><<<blocks_for(A.g.ncell), kCurvThreads, 0, s>>>(A, G, s_out);
+    residual_prec<PREC_F64>(A, G, SA, s);
   else
-    lts_kernel<PREC_F32><<<blocks_for(A.g.ncell), kCurvThreads, 0, s>>>(A, G, s_out);
+    residual_prec<PREC_F32>(A, G, SA, s);
 }
 
 void launch_curv_komega(int prec, const KOmegaArgs& K, const CurvGeom& G, cudaStream_t s) {

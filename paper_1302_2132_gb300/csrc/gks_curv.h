@@ -24,12 +24,14 @@ struct CurvGeom {
 
 // Steady-residual mode of the fused tile kernel (arithmetic-type arrays of the level).
 struct SteadyArgs {
-  const void* s_loc;      // local explicit steps (CFL 1) per cell
+  void* s_loc;            // out: local explicit steps (CFL 1) per cell
   double cfl_flux;        // face window = cfl_flux min(s_l, s_r)
   int first_order;        // no slopes
   void* R;                // out: [4][ncell] sum over faces of the flux rate times L, outward (+ forcing)
   const void* forcing;    // [4][ncell] or null
-  void* tau;              // out: tau_t per cell
+  void* hl[2];            // out if set: half spectral radius times length of every face, per axis
+  void* forcing_io;       // if set: the FAS forcing, [4][ncell], forcing_io -= residual in place of R, and the state
+  void* W_start;          // is copied to W_start
   double* res_acc;        // if set: += sum over cells of (R_rho / A)^2
   int multid;             // multi-dimensional expansion (second-order levels only)
   int recon;              // GKS_RECON_* of the second-order level (MUSCL-3, WENO-5: launch_curv_residual_recon)
@@ -65,9 +67,8 @@ void curv_tile_shape(int variant, int* x, int* y);
 constexpr int kCurvVariants = 3;
 void launch_curv_rate(int prec, const StepArgs& A, const CurvGeom& G, cudaStream_t s);
 void launch_curv_tau(int prec, const StepArgs& A, const CurvGeom& G, void* out, cudaStream_t s, int what = 0);
-// steady solver pieces (FP64 and FP32 state): the residual of A.Win, the local explicit steps
+// steady solver (FP64 and FP32 state): the residual of A.Win
 void launch_curv_residual(int prec, const StepArgs& A, const CurvGeom& G, const SteadyArgs& SA, cudaStream_t s);
-void launch_curv_lts(int prec, const StepArgs& A, const CurvGeom& G, void* s_out, cudaStream_t s);
 // k-omega transport after a flow step on the grid (K.mflux: the step's face mass fluxes times length)
 void launch_curv_komega(int prec, const KOmegaArgs& K, const CurvGeom& G, cudaStream_t s);
 // Steady k-omega update on the finest grid of the steady solver, in place (K.mflux: the residual's

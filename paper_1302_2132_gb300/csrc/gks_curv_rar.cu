@@ -9,7 +9,8 @@
 namespace gks {
 
 cudaError_t prepare_curv_rar() {
-  const cudaError_t r[12] = {
+  const cudaError_t r[14] = {
+      prepare_one<PREC_F64, 2, 1, false, 0, false, true, true>(), prepare_one<PREC_F32, 2, 1, false, 0, false, true, true>(),
       prepare_one<PREC_F64, 2, 0, false, 0, false, true>(), prepare_one<PREC_F64, 2, 0, true, 0, false, true>(),
       prepare_one<PREC_F32, 2, 0, false, 0, false, true>(), prepare_one<PREC_F32, 2, 0, true, 0, false, true>(),
       prepare_one<PREC_F64, 0, 1, false, 0, false, true>(), prepare_one<PREC_F64, 0, 1, true, 0, false, true>(),
@@ -33,7 +34,12 @@ void launch_curv_step_rar(int prec, const StepArgs& A, const CurvGeom& G, bool m
 
 void launch_curv_residual_rar(int prec, const StepArgs& A, const CurvGeom& G, const SteadyArgs& SA, cudaStream_t s) {
   const bool big = A.g.ncell >= 300000;
-  if (SA.multid) {
+  if (SA.first_order) {
+    if (prec == PREC_F64)
+      launch_fused<PREC_F64, 2, 1, false, 0, false, true, true>(A, G, s, SA);
+    else
+      launch_fused<PREC_F32, 2, 1, false, 0, false, true, true>(A, G, s, SA);
+  } else if (SA.multid) {
     if (prec == PREC_F64)
       big ? launch_fused<PREC_F64, 0, 1, true, 0, false, true>(A, G, s, SA)
           : launch_fused<PREC_F64, 2, 1, true, 0, false, true>(A, G, s, SA);

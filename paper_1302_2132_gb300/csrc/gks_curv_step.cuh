@@ -17,6 +17,24 @@ struct FaceView {
   __device__ __forceinline__ R operator()(int q, long f) const { return p[(long)q * nf + f]; }
 };
 
+// CFL rate of a cell on the curvilinear grid: sum over its faces of (|U.n| + c) L / (2 A).
+template <class R>
+__device__ __forceinline__ R curv_rate(const R* w, R gamma, const CurvGeom& G, int n0, int i, int j, long c) {
+  const FaceView<R> fi{(const R*)G.face[0], G.nf[0]}, fj{(const R*)G.face[1], G.nf[1]};
+  const R ir = g_rcp(w[0]);
+  const R u = w[1] * ir, v = w[2] * ir;
+  const R p = pressure_of<R>(2, gamma, w);
+  const R cs = g_sqrt(g_div(gamma * p, w[0]));
+  const long fa = (long)j * (n0 + 1) + i, fc = (long)j * n0 + i;
+  R r = R(0);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    r += (g_abs(u * fi(0, fa + s) + v * fi(1, fa + s)) + cs) * fi(2, fa + s);
+    r += (g_abs(u * fj(0, fc + s * n0) + v * fj(1, fc + s * n0)) + cs) * fj(2, fc + s * n0);
+  }
+  return R(0.5) * r * ((const R*)G.iarea)[c];
+}
+
 // Turbulent relaxation time of interior cell (gi, gj) from Green-Gauss gradients; st(q, v) gives
 // the state of the cell (q = 4) and of its neighbours i-1, i+1, j-1, j+1 (q = 0..3).
 // CONS = false: a caller whose fields are never rho k, rho omega (g.turb_cons unset) skips that test.
@@ -166,6 +184,9 @@ template <> struct CurvTile<1> { static constexpr int X = 16, Y = 7, T = 128; };
 // 16 x 11: 379 faces fill three rounds of 128 threads; one wave of 4 CTAs per SM covers the paper's
 // fine aerofoil grid (608 x 160: 570 tiles)
 template <> struct CurvTile<2> { static constexpr int X = 16, Y = 11, T = 128; };
+// 8 x 6 (first-order residual): 110 faces in one round of 128 threads, for the coarse multigrid levels, whose
+// 16 x 11 tiles leave most of the chip idle (66 x 17 cells: 10 CTAs of three rounds, 27 of one)
+template <> struct CurvTile<3> { static constexpr int X = 8, Y = 6, T = 128; };
 
 // H: halo layers (two for the four-cell MUSCL stencils, three for WENO-5's six cells)
 template <int V, int H_ = 2>
@@ -174,15 +195,22 @@ struct CurvTileGeom {
   static constexpr int HX = X + 2 * H, HY = Y + 2 * H, NH = HX * HY;
   static constexpr int NFX = (X + 1) * Y, NFY = X * (Y + 1), NF = NFX + NFY;
   static constexpr int TX = X + 2, TY = Y + 2, NT = TX * TY;  // tile and first ring (tau)
-  template <class R, bool TR = false> __host__ __device__ static constexpr size_t smem_bytes() {
-    return sizeof(R) * (4 * (size_t)NH + 8 * (size_t)NF + 4 * (size_t)NF + NT + (TR ? 4 * (size_t)NH + 2 * (size_t)NF : 0)) +
+  // (local: the local steps of the tile and its first ring, of the steady residual)
+  template <class R, bool TR = false, bool LOCAL = false> __host__ __device__ static constexpr size_t smem_bytes() {
+    return sizeof(R) * (4 * (size_t)NH + 8 * (size_t)NF + 4 * (size_t)NF + NT + (LOCAL ? NT : 0) +
+                        (TR ? 4 * (size_t)NH + 2 * (size_t)NF : 0)) +
            sizeof(float) * 4 * X * Y;
   }
 };
 
 // MODE 0: one time step (A.Win -> A.Wout, control block as the rectilinear step).  MODE 1: the
-// steady residual of A.Win (SteadyArgs): face windows cfl_flux min(s_l, s_r) from the local steps s,
-// flux rates times L summed per cell (plus the forcing) into R, tau_t of the tile cells stored.
+// steady residual of A.Win (SteadyArgs): the local steps s of the tile and its first ring (the ghost ring
+// takes its source cell's; stored for the tile cells), face windows cfl_flux min(s_l, s_r), flux rates times
+// L summed per cell (plus the forcing) into R, and if asked for the half spectral radii of the faces or the
+// forcing of a coarse level.  Everything a level's smoother needs comes out of this one launch: the local steps
+// and spectral radii as kernels of their own, and the forcing as a third, cost 80 of the 340 us of a four-level
+// cycle at 528 x 136 (with the coarse levels on 16 x 11 tiles).
+// FO (MODE 1): first-order faces.
 // MD: the multi-dimensional expansion (tangential slopes of the two cells in the face frame).
 // RC: the face reconstruction along the grid line (0 MUSCL-2 with limited slopes over the centroid
 // distances; 1 MUSCL-3 and 2 WENO-5 in index space on the rotated states, normal slopes the
@@ -194,7 +222,7 @@ __host__ __device__ constexpr int halo_for(int rc) { return rc == 2 ? 3 : 2; }
 // rho omega with its mass flux, and each cell's update advances them (the transport kernel's
 // arithmetic) into A.RKout, A.RWout.
 // RAR: the rarefaction option (eps = tau/tauhat in the faces' time coefficients).
-template <int PREC, int V, int MODE, bool MD, int RC = 0, bool TR = false, bool RAR = false>
+template <int PREC, int V, int MODE, bool MD, int RC = 0, bool TR = false, bool RAR = false, bool FO = false>
 __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / CurvTile<V>::T)
     curv_step_kernel(const __grid_constant__ StepArgs A, const __grid_constant__ CurvGeom G,
                      const __grid_constant__ SteadyArgs SA) {
@@ -220,6 +248,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
   R* Vs = Us + (TR ? NH : 0);
   R* Gk = Vs + (TR ? NH : 0);
   R* Gw = Gk + (TR ? NF : 0);
+  R* Ls = Ks;  // MODE 1: [TY][TX] local explicit steps of the tile and its first ring (TR is a time step's)
   __shared__ double red[kMaxWarps];
   __shared__ double s_dt;
   const DevGrid& g = A.g;
@@ -346,28 +375,37 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
     if (g.turb_model == TURB_NONE) __syncthreads();  // else the tau phase's barrier follows
   }
   // ---- tau_t of the tile and its first ring (corners unused) ---------------------------------
-  if (g.turb_model != TURB_NONE) {
+  if (MODE == 1 || g.turb_model != TURB_NONE) {
+    const bool turb = g.turb_model != TURB_NONE;
     for (int l = tid; l < NT; l += T) {
       const int ti = l % TX - 1, tj = l / TX - 1;
       if ((ti < 0 || ti >= X) && (tj < 0 || tj >= Y)) continue;
       const int gi = ox + ti, gj = oy + tj;
-      R t;
+      R t = R(0), sl = R(0);
       if (gi >= 0 && gi < n0 && gj >= 0 && gj < n1) {
         const int h0 = (tj + H) * HX + (ti + H);
         const int off[5] = {-1, 1, -HX, HX, 0};
-        t = tau_gg<R, CONS>(g, kc, G, A.f1, A.f2, gi, gj, [&](int q, int v) { return Ws[v * NH + h0 + off[q]]; });
-      } else {  // a ghost cell takes its source cell's value
+        if (turb)
+          t = tau_gg<R, CONS>(g, kc, G, A.f1, A.f2, gi, gj, [&](int q, int v) { return Ws[v * NH + h0 + off[q]]; });
+        if (MODE == 1) {
+          const R w[4] = {Ws[h0], Ws[NH + h0], Ws[2 * NH + h0], Ws[3 * NH + h0]};
+          sl = g_rcp(curv_rate<R>(w, kc.gamma, G, n0, gi, gj, (long)gj * n0 + gi));
+        }
+      } else if (gi >= -1 && gi <= n0 && gj >= -1 && gj <= n1) {  // a ghost cell takes its source cell's value
         const long sc = field_cell(g, 2, gi, gj, 0);
         const int si = (int)(sc % n0), sj = (int)(sc / n0);
         R nb[5][4];
         const int di[5] = {-1, 1, 0, 0, 0}, dj[5] = {0, 0, -1, 1, 0};
 #pragma unroll
         for (int q = 0; q < 5; ++q) load_cell<2, PREC>(g, A.Win, kc, si + di[q], sj + dj[q], 0, nb[q]);
-        t = tau_gg<R, CONS>(g, kc, G, A.f1, A.f2, si, sj, [&](int q, int v) { return nb[q][v]; });
+        if (turb) t = tau_gg<R, CONS>(g, kc, G, A.f1, A.f2, si, sj, [&](int q, int v) { return nb[q][v]; });
+        if (MODE == 1) sl = g_rcp(curv_rate<R>(nb[4], kc.gamma, G, n0, si, sj, sc));
       }
       Ts[l] = t;
-      if (MODE == 1 && ti >= 0 && ti < X && tj >= 0 && tj < Y && gi < n0 && gj < n1)
-        ((R*)SA.tau)[(long)gj * n0 + gi] = t;
+      if (MODE == 1) {
+        Ls[l] = sl;
+        if (ti >= 0 && ti < X && tj >= 0 && tj < Y && gi < n0 && gj < n1) ((R*)SA.s_loc)[(long)gj * n0 + gi] = sl;
+      }
     }
     __syncthreads();
   }
@@ -415,14 +453,13 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
 #pragma unroll
       for (int s = 0; s < 4; ++s) rotated(base + s * stride, S4[s]);
       R wl[4], wr[4], cl[4], cr[4], sl[4], sr[4];
-      const bool fo = MODE == 1 && SA.first_order;
-      if (RC == 0 || fo) {
+      if (RC == 0) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
           const R dm = (S4[1][v] - S4[0][v]) * i01, dc = (S4[2][v] - S4[1][v]) * i12,
                   dp = (S4[3][v] - S4[2][v]) * i23;
-          sl[v] = fo ? R(0) : limiter<R>(g.limiter, dm, dc);
-          sr[v] = fo ? R(0) : limiter<R>(g.limiter, dc, dp);
+          sl[v] = FO ? R(0) : limiter<R>(g.limiter, dm, dc);
+          sr[v] = FO ? R(0) : limiter<R>(g.limiter, dc, dp);
           wl[v] = S4[1][v] + dl * sl[v];
           wr[v] = S4[2][v] - dr * sr[v];
           cl[v] = S4[1][v];
@@ -468,7 +505,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
         tau_t = R(0.5) * (Ts[tr_ - (a == 0 ? 1 : TX)] + Ts[tr_]);
       }
       R tl[1][4] = {{R(0), R(0), R(0), R(0)}}, trr[1][4] = {{R(0), R(0), R(0), R(0)}};
-      if (MD && !fo) {
+      if (MD && !FO) {
         // tangential slopes: limited differences of the rotated states along the transverse grid
         // line over the projected centroid steps (face records tang)
         const long gf = a == 0 ? (long)(oy + lj) * (n0 + 1) + ox + li : (long)(oy + lj) * n0 + ox + li;
@@ -502,26 +539,32 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
         }
       }
       R F[4], tau;
-      R win = dt, Ls = L;
+      R win = dt, Lw = L;
       if (MODE == 1) {  // window of the face from the local steps of its two cells
-        const int ai = a == 0 ? ox + li - 1 : ox + li, aj = a == 0 ? oy + lj : oy + lj - 1;
-        const R* sloc = (const R*)SA.s_loc;
-        win = (R)SA.cfl_flux * fmin(sloc[field_cell(g, 2, ai, aj, 0)], sloc[field_cell(g, 2, ox + li, oy + lj, 0)]);
-        Ls = L / win;
+        const int tr_ = (lj + 1) * TX + li + 1;
+        win = (R)SA.cfl_flux * fmin(Ls[tr_ - (a == 0 ? 1 : TX)], Ls[tr_]);
+        Lw = L / win;
+        if (SA.hl[a]) {
+          // half spectral radius times length of the face: 1/2 L (max over the two cells of |U.n| + c +
+          // 2 (mu + p tau_t) / (rho d)), rho, p, tau_t face means, d the centroid distance
+          const R pa = pressure_of<R>(2, kc.gamma, S4[1]), pb = pressure_of<R>(2, kc.gamma, S4[2]);
+          const R ra = g_rcp(S4[1][0]), rb = g_rcp(S4[2][0]);
+          const R sa = g_abs(S4[1][1] * ra) + g_sqrt(kc.gamma * pa * ra);
+          const R sb = g_abs(S4[2][1] * rb) + g_sqrt(kc.gamma * pb * rb);
+          const R rho = R(0.5) * (S4[1][0] + S4[2][0]), pm = R(0.5) * (pa + pb);
+          const R lam = fmax(sa, sb) + g_div(R(2) * (kc.mu + pm * tau_t) * i12, rho);
+          const long gfm = a == 0 ? (long)(oy + lj) * (n0 + 1) + ox + li : (long)(oy + lj) * n0 + ox + li;
+          ((R*)SA.hl[a])[gfm] = R(0.5) * L * lam;
+        }
       }
-      if constexpr (std::is_same<R, float>::value) {
-        // single precision: the two sides of the face on the paired FP32 instructions
-        if (MD && !fo)
-          face_flux_ps<2, true, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
-        else
-          face_flux_ps<2, false, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
-      } else {
-        if (MD && !fo)
-          face_flux<2, R, true, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
-        else
-          face_flux<2, R, false, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
-      }
-      const R L_ = Ls;
+      // single precision: the two sides of the face on the paired FP32 instructions
+      if constexpr (FO)
+        face_flux_first_order<2, R, RAR>(cl, cr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
+      else if constexpr (std::is_same<R, float>::value)
+        face_flux_ps<2, MD, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
+      else
+        face_flux<2, R, MD, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
+      const R L_ = Lw;
       Fs[l] = F[0] * L_;
       Fs[NF + l] = (F[1] * nx - F[2] * ny) * L_;
       Fs[2 * NF + l] = (F[1] * ny + F[2] * nx) * L_;
@@ -561,8 +604,14 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         R r = Fs[v * NF + fa + 1] - Fs[v * NF + fa] + Fs[v * NF + fc + X] - Fs[v * NF + fc];
-        if (SA.forcing) r += ((const R*)SA.forcing)[(long)v * g.ncell + c];
-        ((R*)SA.R)[(long)v * g.ncell + c] = r;
+        const long q = (long)v * g.ncell + c;
+        if (SA.forcing) r += ((const R*)SA.forcing)[q];
+        if (SA.forcing_io) {  // FAS forcing of a coarse level; the level's state starts from this one
+          ((R*)SA.forcing_io)[q] -= r;
+          ((S*)SA.W_start)[q] = (S)Ws[v * NH + (lj + H) * HX + li + H];
+        } else {
+          ((R*)SA.R)[q] = r;
+        }
         if (v == 0) {
           const double rr = (double)r / G.area[c];
           s2 += rr * rr;
@@ -667,11 +716,11 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
   if (__syncthreads_or(bad) && tid == 0) atomicOr(&A.ctrl->status, 1u);
 }
 
-template <int PREC, int V, int MODE = 0, bool MD = false, int RC = 0, bool TR = false, bool RAR = false>
+template <int PREC, int V, int MODE = 0, bool MD = false, int RC = 0, bool TR = false, bool RAR = false, bool FO = false>
 void launch_fused(const StepArgs& A, const CurvGeom& G, cudaStream_t s, const SteadyArgs& SA = SteadyArgs{}) {
   using TG = CurvTileGeom<V, halo_for(RC)>;
   const int nt = ((A.g.n[0] + TG::X - 1) / TG::X) * ((A.g.n[1] + TG::Y - 1) / TG::Y);
-  const size_t smem = TG::template smem_bytes<typename PrecT<PREC>::R, TR>();
+  const size_t smem = TG::template smem_bytes<typename PrecT<PREC>::R, TR, MODE == 1>();
   // time steps follow one another: on a grid of one wave of tiles or less a programmatic launch
   // lets a step's prologue (the static face records) overlap the end of the previous step; larger
   // grids (and the steady residual) launch plainly
@@ -680,12 +729,12 @@ void launch_fused(const StepArgs& A, const CurvGeom& G, cudaStream_t s, const St
     int per_sm = 0, nsm = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR>, TG::T,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR, FO>, TG::T,
                                                   smem);
     resident = per_sm * nsm > 0 ? per_sm * nsm : -1;
   }
   if (MODE == 1 || nt > resident) {
-    curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR><<<nt, TG::T, smem, s>>>(A, G, SA);
+    curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR, FO><<<nt, TG::T, smem, s>>>(A, G, SA);
     return;
   }
   cudaLaunchConfig_t cfg = {};
@@ -698,15 +747,15 @@ void launch_fused(const StepArgs& A, const CurvGeom& G, cudaStream_t s, const St
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR>, A, G, SA);
+  cudaLaunchKernelEx(&cfg, curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR, FO>, A, G, SA);
 }
 
-template <int PREC, int V, int MODE, bool MD, int RC = 0, bool TR = false, bool RAR = false>
+template <int PREC, int V, int MODE, bool MD, int RC = 0, bool TR = false, bool RAR = false, bool FO = false>
 cudaError_t prepare_one() {
   using TG = CurvTileGeom<V, halo_for(RC)>;
-  return cudaFuncSetAttribute(curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR>,
+  return cudaFuncSetAttribute(curv_step_kernel<PREC, V, MODE, MD, RC, TR, RAR, FO>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)TG::template smem_bytes<typename PrecT<PREC>::R, TR>());
+                              (int)TG::template smem_bytes<typename PrecT<PREC>::R, TR, MODE == 1>());
 }
 
 template <int PREC, int V, int MODE = 0>

@@ -443,55 +443,60 @@ GKS_FN void time_coeffs_hat(T dt, T tau, T eps, TimeCoef<T>& c) {
 //   <q w/2>   = (bK - 1) theta/2 <q> + e0 + e1 c,                        w = sum c_k^2 + xi^2,
 // with the Euler rates N, the deviatoric strain and the heat-flux gradients as coefficients.  Returned in the
 // frame moving with U0 (that of g0): its moments rhs = <q psi>, and F = Dn <u q psi> + T3 <u psi>.
-template <int D, class T, bool MULTID>
+// FO: a first-order face (no slopes): free transport only, rhs = 0.
+template <int D, class T, bool MULTID, bool FO = false>
 GKS_FN void side_terms(const Maxw<D, T>& g, const T* e, const T* sn, const T (*st)[D + 2], const T* U0, T bK, T ibK, T T3,
                        T Dn, T r4, T r45, T* rhs, T* F) {
   constexpr int nv = D + 2;
-  const T k1d = bK - T(1);
-  Grad<D, T> gx, gs[Dims<D>::nt], N;
-  T r[nv], S, div;
+  const T k1d = bK - T(1), hk = T(0.5) * k1d * g.th;
+  T m[nv], x[nv];  // moments of q psi and u q psi in the side's own frame
+  if constexpr (FO) {
 #pragma unroll
-  for (int m = 0; m < nv; ++m) r[m] = sn[m] * g.ir;
-  gradient<D, T>(g, bK, ibK, r, gx);
-  if (MULTID) {
+    for (int v = 0; v < nv; ++v) m[v] = x[v] = T(0);
+  } else {
+    Grad<D, T> gx, gs[Dims<D>::nt], N;
+    T r[nv], S, div;
 #pragma unroll
-    for (int q = 0; q < D - 1; ++q) {
-#pragma unroll
-      for (int m = 0; m < nv; ++m) r[m] = st[q][m] * g.ir;
-      gradient<D, T>(g, bK, ibK, r, gs[q]);
-    }
-  }
-  euler_rate<D, T, MULTID>(g, ibK, gx, gs, S, div, N);
-  const T sg = r4 * (gx.U[0] - ibK * div);  // deviatoric normal strain
-  const T nu = r45 * (T(0.5) * g.it * N.th);
-  const T h = nu + sg;
-  const T ha = T(0.5) * r4 * gx.th, hai = ha * g.it;
-  const T q0 = r45 * N.r - h, q1 = g.it * (r45 * N.U[0]) - T(3) * hai, q2 = g.it * h, q3 = hai * g.it;
-  const T J0 = q0 * e[0] + q1 * e[1] + q2 * e[2] + q3 * e[3];
-  const T J1 = q0 * e[1] + q1 * e[2] + q2 * e[3] + q3 * e[4];
-  const T J2 = q0 * e[2] + q1 * e[3] + q2 * e[4] + q3 * e[5];
-  const T J3 = q0 * e[3] + q1 * e[4] + q2 * e[5] + q3 * e[6];
-  const T e0 = g.th * (k1d * nu - sg), e1 = k1d * ha, hk = T(0.5) * k1d * g.th;
-  // moments of q psi and u q psi in the side's own frame
-  T m[nv], x[nv];
-  m[0] = J0;
-  m[1] = J1;
-  m[D + 1] = T(0.5) * J2 + hk * J0 + e0 * e[0] + e1 * e[1];
-  x[0] = g.U[0] * J0 + J1;
-  x[1] = g.U[0] * J1 + J2;
-  x[D + 1] = g.U[0] * m[D + 1] + (T(0.5) * J3 + hk * J1 + e0 * e[1] + e1 * e[2]);
-#pragma unroll
-  for (int k = 0; k < D - 1; ++k) {
-    T k0 = r45 * N.U[1 + k], k1 = r4 * gx.U[1 + k];
+    for (int v = 0; v < nv; ++v) r[v] = sn[v] * g.ir;
+    gradient<D, T>(g, bK, ibK, r, gx);
     if (MULTID) {
-      const T hb = T(0.5) * r4 * gs[k].th, k2 = hb * g.it;
-      k0 -= hb;
-      k1 = r4 * (gx.U[1 + k] + gs[k].U[0]);
-      m[2 + k] = k0 * e[0] + k1 * e[1] + k2 * e[2];
-      x[2 + k] = g.U[0] * m[2 + k] + (k0 * e[1] + k1 * e[2] + k2 * e[3]);
-    } else {
-      m[2 + k] = k0 * e[0] + k1 * e[1];
-      x[2 + k] = g.U[0] * m[2 + k] + (k0 * e[1] + k1 * e[2]);
+#pragma unroll
+      for (int q = 0; q < D - 1; ++q) {
+#pragma unroll
+        for (int v = 0; v < nv; ++v) r[v] = st[q][v] * g.ir;
+        gradient<D, T>(g, bK, ibK, r, gs[q]);
+      }
+    }
+    euler_rate<D, T, MULTID>(g, ibK, gx, gs, S, div, N);
+    const T sg = r4 * (gx.U[0] - ibK * div);  // deviatoric normal strain
+    const T nu = r45 * (T(0.5) * g.it * N.th);
+    const T h = nu + sg;
+    const T ha = T(0.5) * r4 * gx.th, hai = ha * g.it;
+    const T q0 = r45 * N.r - h, q1 = g.it * (r45 * N.U[0]) - T(3) * hai, q2 = g.it * h, q3 = hai * g.it;
+    const T J0 = q0 * e[0] + q1 * e[1] + q2 * e[2] + q3 * e[3];
+    const T J1 = q0 * e[1] + q1 * e[2] + q2 * e[3] + q3 * e[4];
+    const T J2 = q0 * e[2] + q1 * e[3] + q2 * e[4] + q3 * e[5];
+    const T J3 = q0 * e[3] + q1 * e[4] + q2 * e[5] + q3 * e[6];
+    const T e0 = g.th * (k1d * nu - sg), e1 = k1d * ha;
+    m[0] = J0;
+    m[1] = J1;
+    m[D + 1] = T(0.5) * J2 + hk * J0 + e0 * e[0] + e1 * e[1];
+    x[0] = g.U[0] * J0 + J1;
+    x[1] = g.U[0] * J1 + J2;
+    x[D + 1] = g.U[0] * m[D + 1] + (T(0.5) * J3 + hk * J1 + e0 * e[1] + e1 * e[2]);
+#pragma unroll
+    for (int k = 0; k < D - 1; ++k) {
+      T k0 = r45 * N.U[1 + k], k1 = r4 * gx.U[1 + k];
+      if (MULTID) {
+        const T hb = T(0.5) * r4 * gs[k].th, k2 = hb * g.it;
+        k0 -= hb;
+        k1 = r4 * (gx.U[1 + k] + gs[k].U[0]);
+        m[2 + k] = k0 * e[0] + k1 * e[1] + k2 * e[2];
+        x[2 + k] = g.U[0] * m[2 + k] + (k0 * e[1] + k1 * e[2] + k2 * e[3]);
+      } else {
+        m[2 + k] = k0 * e[0] + k1 * e[1];
+        x[2 + k] = g.U[0] * m[2 + k] + (k0 * e[1] + k1 * e[2]);
+      }
     }
   }
   // free transport <u psi> of the side
@@ -656,11 +661,12 @@ GKS_FN void side_state(const Maxw<D, T>& g, const T* e, T bK, T* w) {
 // Output: F, the flux integrated over [0, dt] (Eq. fluxesf); tau_out the total relaxation time.
 // RAR: the rarefaction option -- the degree of rarefaction eps = tau/tauhat, tauhat = rho0/|D rho|
 // (capped at 1e30), replaces tau/dt inside the time coefficients (Eq. epsilonkomega).
+// FO: a first-order face (the slopes are taken as zero and not read).
 //
 // The inputs other than wl, wr come through an accessor `in` (FaceArrays below): in.s(sd, m) the normal slope,
 // in.c(sd, m) the cell average and in.t(sd, q, m) the q-th tangential slope of component m on side sd (0 left, 1
 // right), each read where it is used.
-template <int D, class T, bool MULTID, bool RAR = false, class In>
+template <int D, class T, bool MULTID, bool RAR = false, bool FO = false, class In>
 GKS_FN void face_flux_in(const T* wl, const T* wr, const In& in, T idxl, T idxr, T tau_t, T dt, const Gas<T>& gas,
                          int abar_t0, T* F, T* tau_out) {
   constexpr int nv = D + 2;
@@ -700,14 +706,14 @@ GKS_FN void face_flux_in(const T* wl, const T* wr, const In& in, T idxl, T idxr,
 #pragma unroll
     for (int n = 0; n < 7; ++n) e[n] = sd ? er[n] : el[n];
 #pragma unroll
-    for (int m = 0; m < nv; ++m) sn[m] = in.s(sd, m);
+    for (int m = 0; m < nv; ++m) sn[m] = FO ? T(0) : in.s(sd, m);
     if (MULTID) {
 #pragma unroll
       for (int s = 0; s < D - 1; ++s)
 #pragma unroll
         for (int m = 0; m < nv; ++m) st[s][m] = in.t(sd, s, m);
     }
-    side_terms<D, T, MULTID>(g, e, sn, st, g0.U, bK, ibK, c.T3, c.Dn, c.r4, c.r45, rs, Fs);
+    side_terms<D, T, MULTID, FO>(g, e, sn, st, g0.U, bK, ibK, c.T3, c.Dn, c.r4, c.r45, rs, Fs);
 #pragma unroll
     for (int m = 0; m < nv; ++m) {
       rhs[m] += rs[m];
@@ -752,7 +758,7 @@ GKS_FN void face_flux(const T* wl, const T* wr, const T* cl, const T* cr, const 
 // the intermediate state and the sides' parts of the Abar right-hand side and of the flux.  The paired sums
 // are added lane x + lane y at the end of each part.  Same terms as face_flux_in; the artificial part of tau is
 // skipped when C_a = 0.
-template <int D, bool MULTID, bool RAR = false, class In>
+template <int D, bool MULTID, bool RAR = false, bool FO = false, class In>
 GKS_FN void face_flux_ps(const float* wl, const float* wr, const In& in, float idxl, float idxr, float tau_t, float dt,
                          const Gas<float>& gas, int abar_t0, float* F, float* tau_out) {
   using T = float;
@@ -794,7 +800,7 @@ GKS_FN void face_flux_ps(const float* wl, const float* wr, const In& in, float i
   {
     F2 sn[nv], st[Dims<D>::nt][nv], U0[D], rs[nv], Fs[nv];
 #pragma unroll
-    for (int m = 0; m < nv; ++m) sn[m] = F2(in.s(0, m), in.s(1, m));
+    for (int m = 0; m < nv; ++m) sn[m] = FO ? F2(0.0f) : F2(in.s(0, m), in.s(1, m));
     if (MULTID) {
 #pragma unroll
       for (int s = 0; s < D - 1; ++s)
@@ -803,7 +809,7 @@ GKS_FN void face_flux_ps(const float* wl, const float* wr, const In& in, float i
     }
 #pragma unroll
     for (int i = 0; i < D; ++i) U0[i] = F2(g0.U[i]);
-    side_terms<D, F2, MULTID>(gs, e, sn, st, U0, F2(bK), F2(ibK), F2(c.T3), F2(c.Dn), F2(c.r4), F2(c.r45), rs, Fs);
+    side_terms<D, F2, MULTID, FO>(gs, e, sn, st, U0, F2(bK), F2(ibK), F2(c.T3), F2(c.Dn), F2(c.r4), F2(c.r45), rs, Fs);
 #pragma unroll
     for (int m = 0; m < nv; ++m) {
       rhs[m] = rs[m].v.x + rs[m].v.y;
@@ -831,6 +837,17 @@ GKS_FN void face_flux_ps(const float* wl, const float* wr, const float* cl, cons
                          float tau_t, float dt, const Gas<float>& gas, int abar_t0, float* F, float* tau_out) {
   face_flux_ps_inv<D, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, g_rcp(dxl), g_rcp(dxr), tau_t, dt, gas, abar_t0, F,
                                    tau_out);
+}
+
+// A first-order face: the sides are the cells' own states cl, cr (no slopes).
+template <int D, class T, bool RAR = false>
+GKS_FN void face_flux_first_order(const T* cl, const T* cr, T dxl, T dxr, T tau_t, T dt, const Gas<T>& gas, int abar_t0,
+                                  T* F, T* tau_out) {
+  const FaceArrays<D, T> in{nullptr, nullptr, cl, cr, nullptr, nullptr};
+  if constexpr (std::is_same<T, float>::value)
+    face_flux_ps<D, false, RAR, true>(cl, cr, in, g_rcp(dxl), g_rcp(dxr), tau_t, dt, gas, abar_t0, F, tau_out);
+  else
+    face_flux_in<D, T, false, RAR, true>(cl, cr, in, g_rcp(dxl), g_rcp(dxr), tau_t, dt, gas, abar_t0, F, tau_out);
 }
 
 }  // namespace gks

@@ -1,13 +1,13 @@
 // Steady-state solver on body-fitted 2D grids (Section 4: local time stepping, LU-SGS smoothing in
 // the form of Yoon and Jameson, multigrid after Jameson; the readings are stated in gks.h).  One
 // cycle on the device:
-//   per level, down: local explicit steps s (lts_kernel), the residual R of the level's state with
-//   face windows cfl_flux min(s_l, s_r) (the fused tile kernel in its residual mode; first order and
-//   with the FAS forcing on coarse levels), half spectral radius times length of every face
-//   (face_lambda_kernel), one LU-SGS smoothing with pseudo-time steps cfl s (lusgs_kernel: 32 x 32
+//   per level, down: local explicit steps s, the residual R of the level's state with
+//   face windows cfl_flux min(s_l, s_r) and half spectral radius times length of every face (all out of
+//   the fused tile kernel in its residual mode; first order and with the FAS forcing on coarse levels),
+//   one LU-SGS smoothing with pseudo-time steps cfl s (lusgs_kernel: 32 x 32
 //   or 16 x 16 cell tiles, one lane per tile column, hyperplane by hyperplane), then the residual
 //   after smoothing restricted with the state to the next level (restrict_kernel) and the forcing
-//   formed (forcing_kernel);
+//   formed (by the residual kernel of the restricted state);
 //   up: the coarse corrections injected (prolong_kernel).
 // Every launch of a cycle is captured once in a CUDA graph; the fine residual norm of each cycle
 // is appended to a device history by the last node.
@@ -43,42 +43,6 @@ __device__ __forceinline__ void euler_normal(R gamma, const R* w, R nx, R ny, R*
   F[1] = w[1] * un + p * nx;
   F[2] = w[2] * un + p * ny;
   F[3] = (w[3] + p) * un;
-}
-
-// Half spectral radius times length of every face: 1/2 L (max over the two cells of |U.n| + c +
-// 2 (mu + p tau_t) / (rho d)), rho, p, tau_t face means, d the centroid distance.
-template <int PREC>
-__global__ void __launch_bounds__(kST) face_lambda_kernel(const __grid_constant__ StepArgs A,
-                                                          const __grid_constant__ CurvGeom G, const void* tau_cell,
-                                                          void* hli, void* hlj) {
-  using R = typename PrecT<PREC>::R;
-  const DevGrid& g = A.g;
-  const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= G.nf[0] + G.nf[1]) return;
-  const int a = t < G.nf[0] ? 0 : 1;
-  const long f = a == 0 ? t : t - G.nf[0];
-  const long nf = G.nf[a];
-  const int n0 = g.n[0];
-  const int nfa = a == 0 ? n0 + 1 : n0;
-  const int fi = (int)(f % nfa), fj = (int)(f / nfa);
-  const int ia = a == 0 ? fi - 1 : fi, ja = a == 0 ? fj : fj - 1;
-  const Consts<R> kc = make_consts<R>(g);
-  const R* rec = (const R*)G.face[a];
-  const R nx = rec[f], ny = rec[nf + f], L = rec[2 * nf + f], id = rec[4 * nf + f];
-  R wa[4], wb[4];
-  load_cell<2, PREC>(g, A.Win, kc, ia, ja, 0, wa);
-  load_cell<2, PREC>(g, A.Win, kc, fi, fj, 0, wb);
-  const R pa = pressure_of<R>(2, kc.gamma, wa), pb = pressure_of<R>(2, kc.gamma, wb);
-  const R sa = g_abs((wa[1] * nx + wa[2] * ny) / wa[0]) + sqrt(kc.gamma * pa / wa[0]);
-  const R sb = g_abs((wb[1] * nx + wb[2] * ny) / wb[0]) + sqrt(kc.gamma * pb / wb[0]);
-  const R rho = R(0.5) * (wa[0] + wb[0]), p = R(0.5) * (pa + pb);
-  R tau = R(0);
-  if (g.turb_model != TURB_NONE) {
-    const R* tc = (const R*)tau_cell;  // per-cell tau_t of this state
-    tau = R(0.5) * (tc[field_cell(g, 2, ia, ja, 0)] + tc[field_cell(g, 2, fi, fj, 0)]);
-  }
-  const R lam = fmax(sa, sb) + R(2) * (kc.mu + p * tau) / (rho / id);
-  ((R*)(a == 0 ? hli : hlj))[f] = R(0.5) * L * lam;
 }
 
 // dynamic shared memory of lusgs_kernel: dW, state (4 planes each) and the diagonal.  Rows are not
@@ -271,16 +235,6 @@ __global__ void restrict_kernel(int m0, int m1, int k0, long kc_, const S* Wf, c
   }
 }
 
-// FAS forcing P = (restricted residual) - R_c(W_c^0), in place over the restricted residual; the
-// level's state starts from W_c^0.
-template <class S, class R>
-__global__ void forcing_kernel(long n, R* P, const R* Rc, const S* W0, S* W) {
-  const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  P[q] = P[q] - Rc[q];
-  W[q] = W0[q];
-}
-
 // W_f += W_c - W_c^0 on the four children of every coarse cell.
 template <class S>
 __global__ void prolong_kernel(int m0, int m1, int k0, long kc_, S* Wf, const S* Wc, const S* Wc0) {
@@ -431,21 +385,27 @@ StepArgs level_args(const gks_steady* s, int l, const void* Win) {
   return A;
 }
 
-// Residual of level l's state Win into lev.R (forcing on coarse levels), with the local steps.
+// Residual of level l's state Win into lev.R (forcing on coarse levels), with the local steps and, for a
+// smoothing to follow, the faces' spectral radii.  start: Win is the restricted state of a coarse level, whose
+// forcing (restricted residual minus this one) and starting state come out instead.
 void residual(gks_steady* s, int l, const void* Win, const void* forcing, double cfl_flux, double* acc,
-              bool mass_flux = false) {
+              bool mass_flux, bool radii, bool start = false) {
   SteadyLevel& lev = s->L[l];
   StepArgs A = level_args(s, l, Win);
   if (mass_flux)
     for (int a = 0; a < 2; ++a) A.mflux[a] = s->mflux[a];
-  launch_curv_lts(s->prec, A, lev.G, lev.s, s->stream);
   SteadyArgs SA{};
   SA.s_loc = lev.s;
+  if (radii)
+    for (int a = 0; a < 2; ++a) SA.hl[a] = lev.hl[a];
+  if (start) {
+    SA.forcing_io = lev.P;
+    SA.W_start = lev.W;
+  }
   SA.cfl_flux = cfl_flux;
   SA.first_order = l > 0;
   SA.R = lev.R;
   SA.forcing = forcing;
-  SA.tau = lev.G.tau;
   SA.res_acc = acc;
   SA.multid = s->multid;
   SA.recon = l == 0 ? s->recon : GKS_RECON_MUSCL2;
@@ -525,14 +485,12 @@ void cycle_prec(gks_steady* s, double cfl, double cfl_flux) {
   for (int l = 0; l < nl; ++l) {
     SteadyLevel& lev = s->L[l];
     const void* forcing = l > 0 ? lev.P : nullptr;
-    residual(s, l, lev.W, forcing, cfl_flux, l == 0 ? s->acc : nullptr, l == 0 && s->transport);
+    residual(s, l, lev.W, forcing, cfl_flux, l == 0 ? s->acc : nullptr, l == 0 && s->transport, true);
     if (l == 0 && s->transport) {  // the k-omega update from the same state, fields and residual
       const KOmegaArgs K = kw_args(s);
       launch_steady_komega(s->prec, K, lev.G, lev.f1, lev.f2, s->RK, s->RW, lev.s, cfl, s->stream);
     }
     const StepArgs A = level_args(s, l, lev.W);
-    face_lambda_kernel<PREC><<<nblk(lev.G.nf[0] + lev.G.nf[1]), kST, 0, s->stream>>>(A, lev.G, lev.G.tau, lev.hl[0],
-                                                                                      lev.hl[1]);
     LusgsArgs LA;
     LA.s_loc = lev.s;
     LA.cfl = cfl;
@@ -548,13 +506,11 @@ void cycle_prec(gks_steady* s, double cfl, double cfl_flux) {
       lusgs_kernel<PREC, 32><<<tiles, 32, lusgs_smem<R, 32>(), s->stream>>>(A, lev.G, LA);
     if (l + 1 == nl) break;
     // residual after smoothing, restricted with the state; coarse residual of W_c^0; forcing
-    residual(s, l, lev.W, forcing, cfl_flux, nullptr);
+    residual(s, l, lev.W, forcing, cfl_flux, nullptr, false, false);
     SteadyLevel& c = s->L[l + 1];
     restrict_kernel<S, R><<<nblk(c.ncell), kST, 0, s->stream>>>(c.n0, c.n1, lev.n0, lev.ncell, (const S*)lev.W,
                                                                  (const R*)lev.R, lev.G.area, (S*)c.W0, (R*)c.P);
-    residual(s, l + 1, c.W0, nullptr, cfl_flux, nullptr);
-    forcing_kernel<S, R><<<nblk(4 * c.ncell), kST, 0, s->stream>>>(4 * c.ncell, (R*)c.P, (const R*)c.R,
-                                                                    (const S*)c.W0, (S*)c.W);
+    residual(s, l + 1, c.W0, nullptr, cfl_flux, nullptr, false, false, true);
   }
   for (int l = nl - 1; l >= 1; --l) {
     SteadyLevel& c = s->L[l];
@@ -984,7 +940,6 @@ gks_status gks_steady_residual(gks_steady* s, double cfl_flux, int first_order, 
   if (s->L[0].g.turb_model != GKS_TURB_NONE && !s->has_turb) return sfail(s, GKS_EINVAL, "turbulence fields not set");
   SteadyLevel& f = s->L[0];
   const StepArgs A = level_args(s, 0, f.W);
-  launch_curv_lts(s->prec, A, f.G, f.s, s->stream);
   SteadyArgs SA{};
   SA.s_loc = f.s;
   SA.cfl_flux = cfl_flux;
@@ -992,7 +947,6 @@ gks_status gks_steady_residual(gks_steady* s, double cfl_flux, int first_order, 
   SA.multid = s->multid;
   SA.recon = first_order ? GKS_RECON_MUSCL2 : s->recon;
   SA.R = f.R;
-  SA.tau = f.G.tau;
   if (SA.recon != GKS_RECON_MUSCL2)
     launch_curv_residual_recon(s->prec, A, f.G, SA, s->stream);
   else if (A.g.rar)
