@@ -34,25 +34,6 @@ constexpr int kST = 128;
 
 inline unsigned nblk(long n, int t = kST) { return (unsigned)((n + t - 1) / t); }
 
-// (single precision divides with the fast reciprocal, double precision exactly)
-template <class R>
-__device__ __forceinline__ void euler_normal(R gamma, const R* w, R nx, R ny, R* F) {
-  const R un = g_div(w[1] * nx + w[2] * ny, w[0]);
-  const R p = pressure_of<R>(2, gamma, w);
-  F[0] = w[0] * un;
-  F[1] = w[1] * un + p * nx;
-  F[2] = w[2] * un + p * ny;
-  F[3] = (w[3] + p) * un;
-}
-
-// dynamic shared memory of lusgs_kernel: dW, state (4 planes each) and the diagonal.  Rows are not
-// padded: the lanes of a sweep step touch one anti-diagonal of a plane, (k - l) TL + l, which with a
-// row pitch of TL falls into TL different banks (a pitch of TL + 1 would put them all in one).
-template <class R, int TL>
-constexpr size_t lusgs_smem() {
-  return sizeof(R) * 9 * TL * TL;
-}
-
 struct LusgsArgs {
   const void* s_loc;  // local explicit steps; pseudo step = cfl s
   double cfl;
@@ -61,153 +42,188 @@ struct LusgsArgs {
   void* W;            // state, advanced by the increment
 };
 
-// Contribution 1/2 (dF - lambda dX) L of neighbour state w with increment X through normal (nx, ny).
+// Shared memory of lusgs_kernel: per cell the state (rho, u, v, |U|^2/2, enthalpy rho H), the inverse diagonal and
+// the increment, per face half its normal times length and its spectral radius.  The lanes of a sweep step touch one
+// anti-diagonal, (k - l) pitch + l, which falls into different banks when the pitch is even: rows of TL, and of
+// TL + 2 for the TL + 1 i-faces.
+template <int TL> struct LusgsTile {
+  static constexpr int NC = TL * TL, PI = TL + 2, NI = TL * PI, NJ = (TL + 1) * TL;
+  template <class R> static constexpr size_t smem() { return sizeof(R) * (10 * NC + 3 * NI + 3 * NJ); }
+};
+constexpr int kLusgsT = 128;
+
+// Contribution 1/2 (F(w + x) - F(w)).n L - 1/2 lambda L x of a neighbour with state q = (rho, u, v, |U|^2/2, rho H) and
+// increment x; (sx, sy) = n L / 2, hl = lambda L / 2.  The difference of the Euler fluxes is written out (du = u' - u, dv,
+// dp), so that the chain from x to the result is one reciprocal and a few multiply-adds long and nothing cancels.
 template <class R>
-__device__ __forceinline__ void offdiag(R gamma, const R* w, const R* X, R nx, R ny, R hl, R L, R* acc) {
-  R wp[4], F0[4], F1[4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) wp[v] = w[v] + X[v];
-  euler_normal<R>(gamma, wp, nx, ny, F1);
-  euler_normal<R>(gamma, w, nx, ny, F0);
-#pragma unroll
-  for (int v = 0; v < 4; ++v) acc[v] += R(0.5) * (F1[v] - F0[v]) * L - hl * X[v];
+__device__ __forceinline__ void offdiag(R gm1, const R* q, const R* x, R sx, R sy, R hl, R* acc) {
+  const R ir = g_rcp(q[0] + x[0]);
+  const R a1 = x[1] - q[1] * x[0], a2 = x[2] - q[2] * x[0];  // rho' du, rho' dv
+  const R du = a1 * ir, dv = a2 * ir;
+  const R dun = du * sx + dv * sy, un = (q[1] * sx + q[2] * sy) + dun, ul = un - hl;
+  const R dp = gm1 * ((x[3] - q[1] * x[1] - q[2] * x[2] + q[3] * x[0]) - R(0.5) * (a1 * du + a2 * dv));
+  const R m = q[0] * dun;
+  acc[0] = x[1] * sx + x[2] * sy - hl * x[0];
+  acc[1] = x[1] * ul + m * q[1] + dp * sx;
+  acc[2] = x[2] * ul + m * q[2] + dp * sy;
+  acc[3] = x[3] * ul + dp * un + q[4] * dun;
 }
 
-// LU-SGS on one TL x TL tile per group of TL lanes: forward and backward sweeps hyperplane by
-// hyperplane (lane l takes tile column l), neighbours outside the tile left out; then W += dW on the
-// tile.  The tile's
-// state and diagonal are staged in shared memory before the sweeps; each lane loads the residual
-// and face records of its next cell while it works on the current one, so that the sweeps wait
-// on shared memory and arithmetic only.
-template <class R>
-struct SweepIn {  // what a lane needs from global memory for one cell of a sweep
-  R r[4];         // forward: the residual
-  R f[2][4];      // the two faces towards the sweep's neighbours: n_x, n_y, L, 1/2 lambda L
-};
-
+// LU-SGS on one TL x TL tile per CTA: forward and backward sweeps hyperplane by hyperplane (lane l takes tile
+// column l), neighbours outside the tile left out; then W += dW on the tile.  A sweep is 2 TL - 1 dependent
+// steps of one warp, so its latency is the kernel.  All of the tile's inputs are staged in shared memory by the whole
+// CTA and read a step ahead; the increment of the neighbour in the lane's own column is the register of its
+// last step, that of the other neighbour one shuffle away.  (Two lanes per cell, one per neighbour, were slower:
+// the second round of shuffles costs more than the shorter instruction stream gains.) A four-level cycle
+// at 528 x 136 in single precision took 56 us less for it (5.21 -> 4.10 ms per 20 cycles with their copies).
 template <int PREC, int TL>
-__global__ void __launch_bounds__(TL) lusgs_kernel(const __grid_constant__ StepArgs A,
-                                                   const __grid_constant__ CurvGeom G,
-                                                   const __grid_constant__ LusgsArgs LA) {
-  constexpr int kLT = TL;
-  constexpr unsigned kMask = TL == 32 ? 0xffffffffu : (1u << TL) - 1u;  // the lanes of the block
+__global__ void __launch_bounds__(kLusgsT) lusgs_kernel(const __grid_constant__ StepArgs A,
+                                                        const __grid_constant__ CurvGeom G,
+                                                        const __grid_constant__ LusgsArgs LA) {
   using R = typename PrecT<PREC>::R;
   using S = typename PrecT<PREC>::S;
+  using TG = LusgsTile<TL>;
+  constexpr unsigned kMask = TL == 32 ? 0xffffffffu : (1u << TL) - 1u;  // the sweeping lanes
   extern __shared__ __align__(16) unsigned char lu_raw[];
-  using Plane = R[kLT][kLT];
-  Plane* X = (Plane*)lu_raw;  // [4]: dW* in the forward sweep, dW after the backward one
-  Plane* Ws = X + 4;          // [4]: the tile's state
-  Plane& Dg = Ws[4];
+  R* Q = (R*)lu_raw;          // [5][NC] rho, u, v, |U|^2/2, rho H
+  R* ID = Q + 5 * TG::NC;     // [NC] 1 / D
+  R* X = ID + TG::NC;         // [4][NC] -residual / D, then dW*, then dW
+  R* FI = X + 4 * TG::NC;     // [3][NI] i-faces: n_x L / 2, n_y L / 2, lambda L / 2
+  R* FJ = FI + 3 * TG::NI;    // [3][NJ] j-faces
   const DevGrid& g = A.g;
-  const int lane = threadIdx.x;
+  const int tid = threadIdx.x;
   const int n0 = g.n[0], n1 = g.n[1];
-  const int ntx = (n0 + kLT - 1) / kLT;
-  const int ox = (blockIdx.x % ntx) * kLT, oy = (blockIdx.x / ntx) * kLT;
-  const int ex = min(kLT, n0 - ox), ey = min(kLT, n1 - oy);
+  const int ntx = (n0 + TL - 1) / TL;
+  const int ox = (blockIdx.x % ntx) * TL, oy = (blockIdx.x / ntx) * TL;
+  const int ex = min(TL, n0 - ox), ey = min(TL, n1 - oy);
   const Consts<R> kc = make_consts<R>(g);
+  const R gm1 = kc.gamma - R(1);
   const R* hli = (const R*)LA.hl[0];
   const R* hlj = (const R*)LA.hl[1];
-  const R* fi_rec = (const R*)G.face[0];
-  const R* fj_rec = (const R*)G.face[1];
   const long nf0 = G.nf[0], nf1 = G.nf[1];
   const R* Rr = (const R*)LA.R;
   const R* sl = (const R*)LA.s_loc;
   S* Wg = (S*)LA.W;
-  // stage the state and the diagonal D = A / (cfl s) + 1/2 sum lambda L
-  for (int q = lane; q < ex * ey; q += kLT) {
-    const int li = q % ex, lj = q / ex;
+  for (int q = tid; q < TG::NC; q += kLusgsT) {
+    const int li = q % TL, lj = q / TL;
+    if (li >= ex || lj >= ey) continue;
     const int i = ox + li, j = oy + lj;
     const long c = (long)j * n0 + i;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) Ws[v][lj][li] = (R)Wg[(long)v * g.ncell + c];
-    const long fa = (long)j * (n0 + 1) + i, fc = (long)j * n0 + i;
-    const R dt = sl[c] * (R)LA.cfl;
-    Dg[lj][li] = (R)G.area[c] / dt + hli[fa] + hli[fa + 1] + hlj[fc] + hlj[fc + n0];
-  }
-  __syncwarp(kMask);
-  const int nk = ex + ey - 1;
-  // loads of the cell of hyperplane k (forward: lower faces and the residual; backward: upper faces)
-  auto fetch = [&](int k, bool fwd, SweepIn<R>& in) {
-    const int li = lane, lj = k - lane;
-    if (!(k >= 0 && k < nk && li < ex && lj >= 0 && lj < ey)) return;
-    const int i = ox + li, j = oy + lj;
-    const long c = (long)j * n0 + i;
-    const long fi = (long)j * (n0 + 1) + i + (fwd ? 0 : 1), fj = (long)(j + (fwd ? 0 : 1)) * n0 + i;
-    if (fwd) {
-#pragma unroll
-      for (int v = 0; v < 4; ++v) in.r[v] = Rr[(long)v * g.ncell + c];
-    }
-    in.f[0][0] = fi_rec[fi];
-    in.f[0][1] = fi_rec[nf0 + fi];
-    in.f[0][2] = fi_rec[2 * nf0 + fi];
-    in.f[0][3] = hli[fi];
-    in.f[1][0] = fj_rec[fj];
-    in.f[1][1] = fj_rec[nf1 + fj];
-    in.f[1][2] = fj_rec[2 * nf1 + fj];
-    in.f[1][3] = hlj[fj];
-  };
-  auto nbr = [&](int li, int lj, R* w, R* x) {
+    R w[4], r[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      w[v] = Ws[v][lj][li];
-      x[v] = X[v][lj][li];
+      w[v] = (R)Wg[(long)v * g.ncell + c];
+      r[v] = Rr[(long)v * g.ncell + c];
     }
-  };
-  // forward sweep
-  SweepIn<R> cur, nxt;
-  fetch(0, true, cur);
-  for (int k = 0; k < nk; ++k) {
-    fetch(k + 1, true, nxt);
-    const int li = lane, lj = k - lane;
-    if (li < ex && lj >= 0 && lj < ey) {
-      R acc[4] = {R(0), R(0), R(0), R(0)};
-      if (li > 0) {  // face i - 1/2, normal away from the cell: -n
-        R w[4], x[4];
-        nbr(li - 1, lj, w, x);
-        offdiag<R>(kc.gamma, w, x, -cur.f[0][0], -cur.f[0][1], cur.f[0][3], cur.f[0][2], acc);
-      }
-      if (lj > 0) {
-        R w[4], x[4];
-        nbr(li, lj - 1, w, x);
-        offdiag<R>(kc.gamma, w, x, -cur.f[1][0], -cur.f[1][1], cur.f[1][3], cur.f[1][2], acc);
-      }
-      const R D = Dg[lj][li];
+    const R ir = g_rcp(w[0]), u = w[1] * ir, vv = w[2] * ir;
+    Q[q] = w[0];
+    Q[TG::NC + q] = u;
+    Q[2 * TG::NC + q] = vv;
+    Q[3 * TG::NC + q] = R(0.5) * (u * u + vv * vv);
+    Q[4 * TG::NC + q] = w[3] + pressure_of<R>(2, kc.gamma, w);
+    // diagonal D = A / (cfl s) + 1/2 sum lambda L
+    const long fa = (long)j * (n0 + 1) + i, fc = (long)j * n0 + i;
+    const R id = g_rcp(g_div((R)G.area[c], sl[c] * (R)LA.cfl) + hli[fa] + hli[fa + 1] + hlj[fc] + hlj[fc + n0]);
+    ID[q] = id;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) X[v][lj][li] = g_div(-cur.r[v] - acc[v], D);
-    }
-    cur = nxt;
-    __syncwarp(kMask);
+    for (int v = 0; v < 4; ++v) X[v * TG::NC + q] = -r[v] * id;
   }
-  // backward sweep
-  fetch(nk - 1, false, cur);
-  for (int k = nk - 1; k >= 0; --k) {
-    fetch(k - 1, false, nxt);
-    const int li = lane, lj = k - lane;
-    if (li < ex && lj >= 0 && lj < ey) {
-      R acc[4] = {R(0), R(0), R(0), R(0)};
-      if (li + 1 < ex) {
-        R w[4], x[4];
-        nbr(li + 1, lj, w, x);
-        offdiag<R>(kc.gamma, w, x, cur.f[0][0], cur.f[0][1], cur.f[0][3], cur.f[0][2], acc);
+  for (int q = tid; q < TL * (TL + 1); q += kLusgsT) {
+    {
+      const int li = q % (TL + 1), lj = q / (TL + 1);
+      if (li <= ex && lj < ey) {
+        const long f = (long)(oy + lj) * (n0 + 1) + ox + li;
+        const R* rec = (const R*)G.face[0];
+        const R hL = R(0.5) * rec[2 * nf0 + f];
+        FI[lj * TG::PI + li] = rec[f] * hL;
+        FI[TG::NI + lj * TG::PI + li] = rec[nf0 + f] * hL;
+        FI[2 * TG::NI + lj * TG::PI + li] = hli[f];
       }
-      if (lj + 1 < ey) {
-        R w[4], x[4];
-        nbr(li, lj + 1, w, x);
-        offdiag<R>(kc.gamma, w, x, cur.f[1][0], cur.f[1][1], cur.f[1][3], cur.f[1][2], acc);
-      }
-      const R D = Dg[lj][li];
+    }
+    const int li = q % TL, lj = q / TL;
+    if (li < ex && lj <= ey) {
+      const long f = (long)(oy + lj) * n0 + ox + li;
+      const R* rec = (const R*)G.face[1];
+      const R hL = R(0.5) * rec[2 * nf1 + f];
+      FJ[q] = rec[f] * hL;
+      FJ[TG::NJ + q] = rec[nf1 + f] * hL;
+      FJ[2 * TG::NJ + q] = hlj[f];
+    }
+  }
+  __syncthreads();
+  if (tid < TL) {
+    const int nk = ex + ey - 1, li = tid;
+    R x[4] = {R(0), R(0), R(0), R(0)};  // increment of the lane's last cell
+    // what a step reads of its cell, its two neighbours' states and the faces towards them: read a step
+    // ahead, so that shared memory is off the chain from one increment to the next
+    struct Step {
+      R wi[5], wj[5], fi[3], fj[3], id, x0[4];
+      int q;  // the cell, or -1
+      bool ni, nj;
+    };
+    // dir = 0: forward (neighbours i - 1, j - 1 through their faces, normals away from the cell: -n); 1: backward
+#pragma unroll 1
+    for (int dir = 0; dir < 2; ++dir) {
+      const R sgn = dir ? R(1) : R(-1);
+      auto read = [&](int kk, Step& t) {
+        const int lj = (dir ? nk - 1 - kk : kk) - li;
+        // lanes without a cell, and cells without the neighbour, read a cell of the tile and its faces instead;
+        // a neighbour that is not there has a zero increment, whose contribution is exactly zero
+        const int ci = min(li, ex - 1), cj = min(max(lj, 0), ey - 1);
+        const int q = cj * TL + ci;
+        t.q = li < ex && lj >= 0 && lj < ey ? q : -1;
+        t.ni = dir ? ci + 1 < ex : ci > 0;
+        t.nj = dir ? cj + 1 < ey : cj > 0;
+        const int qi = t.ni ? (dir ? q + 1 : q - 1) : q, qj = t.nj ? (dir ? q + TL : q - TL) : q;
+        const int fi = cj * TG::PI + ci + dir, fj = q + dir * TL;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) X[v][lj][li] = X[v][lj][li] - g_div(acc[v], D);
+        for (int v = 0; v < 5; ++v) {
+          t.wi[v] = Q[v * TG::NC + qi];
+          t.wj[v] = Q[v * TG::NC + qj];
+        }
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          t.fi[v] = FI[v * TG::NI + fi];
+          t.fj[v] = FJ[v * TG::NJ + fj];
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) t.x0[v] = X[v * TG::NC + q];
+        t.id = ID[q];
+      };
+      Step cur, nxt;
+      read(0, cur);
+      const int src = dir ? tid + 1 : tid - 1;
+      for (int kk = 0; kk < nk; ++kk) {
+        read(min(kk + 1, nk - 1), nxt);
+        R xi[4], xj[4], ai[4], aj[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const R t = __shfl_sync(kMask, x[v], src & (TL - 1), TL);
+          xi[v] = cur.ni ? t : R(0);
+          xj[v] = cur.nj ? x[v] : R(0);
+        }
+        offdiag<R>(gm1, cur.wi, xi, sgn * cur.fi[0], sgn * cur.fi[1], cur.fi[2], ai);
+        offdiag<R>(gm1, cur.wj, xj, sgn * cur.fj[0], sgn * cur.fj[1], cur.fj[2], aj);
+        // forward: dW* = (-R - acc) / D; backward: dW = dW* - acc / D
+        if (cur.q >= 0) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            x[v] = cur.x0[v] - (ai[v] + aj[v]) * cur.id;
+            X[v * TG::NC + cur.q] = x[v];
+          }
+        }
+        cur = nxt;
+      }
     }
-    cur = nxt;
-    __syncwarp(kMask);
   }
-  // W += dW
-  for (int q = lane; q < ex * ey; q += kLT) {
-    const int li = q % ex, lj = q / ex;
+  __syncthreads();
+  for (int q = tid; q < TG::NC; q += kLusgsT) {
+    const int li = q % TL, lj = q / TL;
+    if (li >= ex || lj >= ey) continue;
     const long c = (long)(oy + lj) * n0 + ox + li;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) Wg[(long)v * g.ncell + c] = (S)(Ws[v][lj][li] + X[v][lj][li]);
+    for (int v = 0; v < 4; ++v)
+      Wg[(long)v * g.ncell + c] = (S)((R)Wg[(long)v * g.ncell + c] + X[v * TG::NC + q]);
   }
 }
 
@@ -501,9 +517,9 @@ void cycle_prec(gks_steady* s, double cfl, double cfl_flux) {
     const int TLs = s->tile;
     const int tiles = ((lev.n0 + TLs - 1) / TLs) * ((lev.n1 + TLs - 1) / TLs);
     if (TLs == 16)
-      lusgs_kernel<PREC, 16><<<tiles, 16, lusgs_smem<R, 16>(), s->stream>>>(A, lev.G, LA);
+      lusgs_kernel<PREC, 16><<<tiles, kLusgsT, LusgsTile<16>::smem<R>(), s->stream>>>(A, lev.G, LA);
     else
-      lusgs_kernel<PREC, 32><<<tiles, 32, lusgs_smem<R, 32>(), s->stream>>>(A, lev.G, LA);
+      lusgs_kernel<PREC, 32><<<tiles, kLusgsT, LusgsTile<32>::smem<R>(), s->stream>>>(A, lev.G, LA);
     if (l + 1 == nl) break;
     // residual after smoothing, restricted with the state; coarse residual of W_c^0; forcing
     residual(s, l, lev.W, forcing, cfl_flux, nullptr, false, false);
@@ -616,9 +632,9 @@ gks_status gks_steady_create(const gks_grid* grid, const gks_gas* gas, const gks
   }
   if (prepare_curv() != cudaSuccess || prepare_curv_recon() != cudaSuccess || prepare_curv_rar() != cudaSuccess ||
       cudaFuncSetAttribute(lusgs_kernel<PREC_F64, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)lusgs_smem<double, 32>()) != cudaSuccess ||
+                           (int)LusgsTile<32>::smem<double>()) != cudaSuccess ||
       cudaFuncSetAttribute(lusgs_kernel<PREC_F32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)lusgs_smem<float, 32>()) != cudaSuccess) {
+                           (int)LusgsTile<32>::smem<float>()) != cudaSuccess) {
     cudaGetLastError();
     return bad(GKS_ECUDA);
   }
