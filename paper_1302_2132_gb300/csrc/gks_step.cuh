@@ -268,21 +268,17 @@ template <class R>
 __device__ __forceinline__ R pressure_of(int D, R gamma, const R* w) {
   R q = R(0);
   for (int i = 0; i < D; ++i) q += w[1 + i] * w[1 + i];
-  return (gamma - R(1)) * (w[D + 1] - R(0.5) * g_div(q, w[0]));
+  return (gamma - R(1)) * (w[D + 1] - R(0.5) * g_quot(q, w[0]));
 }
 
-// rho > 0 and p > 0 for a conservative state.  Single precision tests 2 rho (rho E) > |rho U|^2 (the
-// same condition once rho > 0, without a quotient); double precision evaluates p as the oracle does.
+// rho > 0 and p > 0 for a conservative state: 2 rho (rho E) > |rho U|^2 is the same condition once rho > 0, without
+// a quotient.
 template <int D, class R>
 __device__ __forceinline__ bool physical(R gamma, const R* w) {
-  if constexpr (sizeof(R) == sizeof(float)) {
-    R q = R(0);
+  R q = R(0);
 #pragma unroll
-    for (int i = 0; i < D; ++i) q += w[1 + i] * w[1 + i];
-    return w[0] > R(0) && R(2) * w[0] * w[D + 1] > q;
-  } else {
-    return w[0] > R(0) && pressure_of<R>(D, gamma, w) > R(0);
-  }
+  for (int i = 0; i < D; ++i) q += w[1 + i] * w[1 + i];
+  return w[0] > R(0) && R(2) * w[0] * w[D + 1] > q;
 }
 
 // Isothermal no-slip wall image: velocity reversed, same pressure, T_g = T_w^2 / T_i (T = p/rho).
@@ -1318,19 +1314,15 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     const long c = cell_index(g, gi, gj, gk);
     // faces below/above the cell along each axis
     int fm[3], fp[3];
-    R h[3];
     fm[0] = (lk * Y + lj) * (X + 1) + li;
     fp[0] = fm[0] + 1;
-    h[0] = wsx[li + H];
     if (D >= 2) {
       fm[1] = G::NFX + (lk * (Y + 1) + lj) * X + li;
       fp[1] = fm[1] + X;
-      h[1] = wsy[lj + H];
     }
     if (D >= 3) {
       fm[2] = G::NFX + G::NFY + (lk * Y + lj) * X + li;
       fp[2] = fm[2] + X * Y;
-      h[2] = wsz[lk + H];
     }
     R ih[3];
 #pragma unroll
@@ -1344,7 +1336,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       if constexpr (PREC == PREC_F64) {
         double w = (double)Ws[v * G::NH + hidx];
 #pragma unroll
-        for (int d = 0; d < D; ++d) w -= ((double)Fs[v * G::NF + fp[d]] - (double)Fs[v * G::NF + fm[d]]) / (double)h[d];
+        for (int d = 0; d < D; ++d) w -= ((double)Fs[v * G::NF + fp[d]] - (double)Fs[v * G::NF + fm[d]]) * (double)ih[d];
         ((double*)A.Wout)[gidx] = w;
         wn[v] = (R)w;
       } else {

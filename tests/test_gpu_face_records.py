@@ -45,3 +45,27 @@ def test_counts_and_alignment(D, n, offset, precision):
     if precision == "fp32":
         Fr, _ = gks.face_flux(D, part.float().double(), 1e-3, mu=1e-4, C_a=0.3, precision=precision)
         assert torch.equal(F, Fr)
+
+
+@pytest.mark.parametrize("mach", [0.0, 1e-9, 0.3, 1.0, 3.0, 8.0])
+@pytest.mark.parametrize("sign", [-1.0, 1.0])
+def test_fp64_flux_over_the_range_of_the_half_line_moments(mach, sign):
+    """Both sides at the same normal Mach number, from rest (erfc near 1) to far supersonic (one half line empty):
+    the double flux matches the oracle to the 1e-12 of the parity tests."""
+    import oracle
+    D, nv, n, dt = 2, 4, 20, 1e-3
+    rng = np.random.default_rng(int(10 * mach) + 7)
+    rec = records(D, n, 5)
+    for o in range(4):
+        rho, p = rng.uniform(0.5, 2, n), rng.uniform(0.5, 2, n)
+        u = np.stack([sign * mach * np.sqrt(1.4 * p / rho), rng.uniform(-1, 1, n)], 1)
+        rec[:, o * nv:(o + 1) * nv] = np.concatenate(
+            [rho[:, None], rho[:, None] * u, (p / 0.4 + 0.5 * rho * (u * u).sum(1))[:, None]], 1)
+    F, _ = gks.face_flux(D, torch.tensor(rec, device="cuda"), dt, mu=1e-4, C_a=0.3, precision="fp64")
+    F = F.cpu().numpy()
+    for i in range(n):
+        r = rec[i]
+        f = oracle.make_face(D, r[:4], r[4:8], r[8:12], r[12:16], r[16:20], r[20:24], r[24:28][None], r[28:32][None],
+                             r[32], r[33], r[34])
+        Fo = oracle.face_flux(D, 1.4, 1e-4, 0.3, dt, f, multid=1)
+        assert np.linalg.norm(F[i] - Fo) <= 1e-12 * np.linalg.norm(Fo)
