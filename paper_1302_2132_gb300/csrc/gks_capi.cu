@@ -181,6 +181,15 @@ int tiles_for(const gks_handle* h, int variant) {
   return (int)n;
 }
 
+// The 8 x 8 tile joins the 2D candidates while a grid is too small to fill the chip otherwise: in single
+// precision up to one such tile per SM (152 x 64 cells), in double, where the 32 x 15 tile is the only other shape
+// and a round of its faces takes tens of microseconds, up to one of those per SM.  64^2 in single precision took
+// 10.1 us per step with the shapes above, 4.2 with this one and programmatic launches.
+const int kSmallTile2D = 9;
+bool small_grid_2d(const gks_handle* h) {
+  return h->D == 2 && (h->prec == PREC_F64 ? tiles_for(h, 0) <= 152 : h->ncell <= 152 * 64);
+}
+
 // k-omega transport fused into the body-fitted step (MUSCL-2, FP64 or the FP32 float-pair form);
 // other combinations run the step and the transport kernel one after the other.
 bool fused_transport(const gks_handle* h) {
@@ -214,7 +223,9 @@ void launch_step_variant(gks_handle* h, const StepArgs& A, int variant) {
     launch_step_weno5(h->D, h->prec, h->multid, variant, A, tiles_for(h, variant), h->stream);
     return;
   }
-  if (h->D == 1 && variant > 0)
+  if ((h->D == 1 && variant == 3) || (h->D == 2 && variant == kSmallTile2D))
+    launch_step_small(h->D, h->prec, h->multid, A, tiles_for(h, variant), h->stream);
+  else if (h->D == 1 && variant > 0)
     launch_step_d1_variant(variant, h->prec, A, tiles_for(h, variant), h->stream);
   else if (h->D == 1)
     launch_step_d1(h->prec, false, A, tiles_for(h, 0), h->stream);
@@ -471,30 +482,21 @@ std::vector<int> tile_candidates(const gks_handle* h) {
   const int n = h->D == 1 ? kTileVariants1D
                           : (h->D == 2 && f32 ? kTileVariants2D : (h->D == 3 && f32 ? kTileVariants3D : 1));
   for (int v = 0; v < n; ++v) c.push_back(v);
+  if (small_grid_2d(h)) c.push_back(kSmallTile2D);
   return c;
-}
-
-int n_variants(const gks_handle* h) {
-  if (h->base.g.rar) return 1;
-  if (h->curv) return (h->recon != GKS_RECON_MUSCL2 || fused_transport(h)) ? 2 : kCurvVariants;
-  if (h->recon != GKS_RECON_MUSCL2) return (int)tile_candidates(h).size();
-  if (h->D == 1) return kTileVariants1D;
-  if (h->D == 2 && (h->prec == PREC_F32 || h->prec == PREC_F32D)) return kTileVariants2D;
-  if (h->D == 3 && (h->prec == PREC_F32 || h->prec == PREC_F32D)) return kTileVariants3D;
-  return 1;
 }
 
 gks_status autotune(gks_handle* h) {
   h->tuned = true;
-  const int nvar = n_variants(h);
-  if (nvar == 1) {
-    h->tile_variant = tile_candidates(h)[0];
+  const std::vector<int> cand = tile_candidates(h);
+  if (cand.size() == 1) {
+    h->tile_variant = cand[0];
     return GKS_OK;
   }
   const char* force = std::getenv("GKS_TILE_VARIANT");
   if (force) {
     const int v = std::atoi(force);
-    for (int c : tile_candidates(h))
+    for (int c : cand)
       if (c == v) h->tile_variant = v;
     return GKS_OK;
   }
@@ -512,7 +514,6 @@ gks_status autotune(gks_handle* h) {
   GKS_CK(h, cudaEventCreate(&e0));
   GKS_CK(h, cudaEventCreate(&e1));
   const StepArgs A = step_args(h, h->step);
-  const std::vector<int> cand = tile_candidates(h);
   std::vector<float> fastest(cand.size(), 1e30f);
   for (int v : cand) launch_step_variant(h, A, v);  // warm-up
   // round robin, each launch timed alone, the fastest launch of each shape kept: a clock that is
@@ -640,6 +641,7 @@ gks_status gks_create(const gks_grid* grid, const gks_gas* gas, const gks_turb* 
     if (e == cudaSuccess && D == 3) e = prepare_step_d3_variants();
     if (e == cudaSuccess && D >= 2) e = prepare_step_acc64();
     if (e == cudaSuccess && D >= 2) e = prepare_step_pair();
+    if (e == cudaSuccess && D <= 2) e = prepare_step_small();
     if (e == cudaSuccess) e = prepare_step_rar();
     if (e == cudaSuccess && D == 2) e = prepare_curv_rar();
     if (e == cudaSuccess) e = prepare_komega();

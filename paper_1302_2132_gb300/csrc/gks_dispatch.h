@@ -36,10 +36,13 @@ void launch_step_acc64_variant(int D, int variant, bool multid, const StepArgs& 
 // the rarefaction option (MUSCL-2, default tile of each dimension, every precision)
 cudaError_t prepare_step_rar();
 void launch_step_rar(int D, int prec, bool multid, const StepArgs& A, int nblocks, cudaStream_t s);
+// small grids: 2D variant 9 (8x8 cells) in every precision, 1D variant 3 (30 cells)
+cudaError_t prepare_step_small();
+void launch_step_small(int D, int prec, bool multid, const StepArgs& A, int nblocks, cudaStream_t s);
 // 1D tile variants 1 and 2 (narrow tiles for small grids)
 cudaError_t prepare_step_d1_variants();
 void launch_step_d1_variant(int variant, int prec, const StepArgs& A, int nblocks, cudaStream_t s);
-constexpr int kTileVariants1D = 3;
+constexpr int kTileVariants1D = 4;  // the fourth in gks_step_small.cu
 
 // batches of independent solves (FP64 or FP32 float-pair arithmetic) with a tile variant per group;
 // prepare_* fill the resident CTAs per SM of each variant (1D: [v]; 2D: [2 v + multid])

@@ -36,7 +36,8 @@ void launch_step_d2_variant(int variant, bool multid, const StepArgs& A, int nbl
 
 void tile_shape(int D, int variant, int* x, int* y, int* z) {
   if (D == 1) {
-    *x = variant == 1 ? Tile<1, 1>::X : (variant == 2 ? Tile<1, 2>::X : Tile<1, 0>::X);
+    *x = variant == 1 ? Tile<1, 1>::X
+                      : (variant == 2 ? Tile<1, 2>::X : (variant == 3 ? Tile<1, 3>::X : Tile<1, 0>::X));
     *y = 1;
     *z = 1;
     return;
@@ -56,6 +57,7 @@ void tile_shape(int D, int variant, int* x, int* y, int* z) {
   else if (variant == 6) { *x = Tile<2, 6>::X; *y = Tile<2, 6>::Y; }
   else if (variant == 7) { *x = Tile<2, 7>::X; *y = Tile<2, 7>::Y; }
   else if (variant == 8) { *x = Tile<2, 8>::X; *y = Tile<2, 8>::Y; }
+  else if (variant == 9) { *x = Tile<2, 9>::X; *y = Tile<2, 9>::Y; }
   else { *x = Tile<2, 0>::X; *y = Tile<2, 0>::Y; }
   *z = 1;
 }
