@@ -83,11 +83,11 @@ __device__ __forceinline__ R tau_gg(const DevGrid& g, const Consts<R>& kc, const
   const R S = g_sqrt(R(2) * s2);
   R nu, eta;
   if (g.turb_model == TURB_KEPS) {
-    nu = g_div(kc.C_mu * f1 * f1, f2);
-    eta = g_div(S * f1, f2);
+    nu = g_div_full(kc.C_mu * f1 * f1, f2);
+    eta = g_div_full(S * f1, f2);
   } else {
-    nu = g_div(f1, f2);
-    eta = g_div(S, kc.beta_star * f2);
+    nu = g_div_full(f1, f2);
+    eta = g_div_full(S, kc.beta_star * f2);
   }
   return (f1 > R(0) && f2 > R(0)) ? g_div(w[0] * nu, p * g_sqrt(R(1) + eta * eta)) : R(0);
 }

@@ -471,11 +471,11 @@ __device__ __forceinline__ R tau_turb_cell(int turb_model, bool cons, const Cons
   const R S = g_sqrt(R(2) * s2);
   R nu, eta;
   if (turb_model == TURB_KEPS) {
-    nu = g_div(kc.C_mu * f1 * f1, f2);
-    eta = g_div(S * f1, f2);
+    nu = g_div_full(kc.C_mu * f1 * f1, f2);
+    eta = g_div_full(S * f1, f2);
   } else {
-    nu = g_div(f1, f2);
-    eta = g_div(S, kc.beta_star * f2);
+    nu = g_div_full(f1, f2);
+    eta = g_div_full(S, kc.beta_star * f2);
   }
   return g_div(w[0] * nu, p * g_sqrt(R(1) + eta * eta));
 }
@@ -515,8 +515,8 @@ __device__ __forceinline__ R tau_turb_two_eq(bool keps, bool cons, const Consts<
     }
   const R S = g_sqrt(R(2) * s2);
   // k-epsilon: nu = C_mu k^2/eps, eta = S k/eps; k-omega: nu = k/omega, eta = S/(beta* omega)
-  const R nu = keps ? g_div(kc.C_mu * f1 * f1, f2) : g_div(f1, f2);
-  const R eta = keps ? g_div(S * f1, f2) : g_div(S, kc.beta_star * f2);
+  const R nu = keps ? g_div_full(kc.C_mu * f1 * f1, f2) : g_div_full(f1, f2);
+  const R eta = keps ? g_div_full(S * f1, f2) : g_div_full(S, kc.beta_star * f2);
   const R t = g_div(w[0] * nu, p * g_sqrt(R(1) + eta * eta));
   return (f1 > R(0) && f2 > R(0)) ? t : R(0);
 }
