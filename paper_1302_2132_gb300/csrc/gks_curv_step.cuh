@@ -474,8 +474,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
           if (RC == 2) {
-            wl[v] = weno5<R>(E0[v], S4[0][v], S4[1][v], S4[2][v], S4[3][v]);
-            wr[v] = weno5<R>(E1[v], S4[3][v], S4[2][v], S4[1][v], S4[0][v]);
+            weno5_sides(E0[v], S4[0][v], S4[1][v], S4[2][v], S4[3][v], E1[v], wl[v], wr[v]);
           } else {
             wl[v] = muscl3_right<R>(S4[0][v], S4[1][v], S4[2][v]);
             wr[v] = muscl3_left<R>(S4[1][v], S4[2][v], S4[3][v]);

@@ -381,6 +381,20 @@ GKS_FN R weno5(R a, R b, R c, R d, R e) {
   return g_div(a0 * q0 + a1 * q1 + a2 * q2, a0 + a1 + a2);
 }
 
+// Both sides of the face between c and d of the cells a..f; in single precision on the paired
+// instructions (603 x 501, float pair, 45.8 -> 43.5 us per step against one side after the other).
+template <class R>
+GKS_FN void weno5_sides(R a, R b, R c, R d, R e, R f, R& wl, R& wr) {
+  if constexpr (std::is_same<R, float>::value) {
+    const F2 w = weno5<F2>(F2(a, f), F2(b, e), F2(c, d), F2(d, c), F2(e, b));
+    wl = w.v.x;
+    wr = w.v.y;
+  } else {
+    wl = weno5<R>(a, b, c, d, e);
+    wr = weno5<R>(f, e, d, c, b);
+  }
+}
+
 // MUSCL on one variable at the face between cells 1 and 2 of the stencil s0..s3 with widths
 // h0..h3: limited slopes of cells 1 and 2 and the face values left and right.
 template <class R>

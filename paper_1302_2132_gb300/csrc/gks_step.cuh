@@ -1114,8 +1114,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
           // higher-order face values from the normal stencil (cells pn-3 .. pn+2); the normal
           // slopes are the one-sided differences to them
           if constexpr (RECON == RECON_WENO5) {
-            wl[v] = weno5<R>(p[-3 * sn], p[-2 * sn], s1, s2, p[sn]);
-            wr[v] = weno5<R>(p[2 * sn], p[sn], s2, s1, p[-2 * sn]);
+            weno5_sides(p[-3 * sn], p[-2 * sn], s1, s2, p[sn], p[2 * sn], wl[v], wr[v]);
           } else {
             wl[v] = muscl3_right<R>(p[-2 * sn], s1, s2);
             wr[v] = muscl3_left<R>(s1, s2, p[sn]);
