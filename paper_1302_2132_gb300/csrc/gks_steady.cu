@@ -74,8 +74,9 @@ __device__ __forceinline__ void offdiag(R gm1, const R* q, const R* x, R sx, R s
 // steps of one warp, so its latency is the kernel.  All of the tile's inputs are staged in shared memory by the whole
 // CTA and read a step ahead; the increment of the neighbour in the lane's own column is the register of its
 // last step, that of the other neighbour one shuffle away.  (Two lanes per cell, one per neighbour, were slower:
-// the second round of shuffles costs more than the shorter instruction stream gains.) A four-level cycle
-// at 528 x 136 in single precision took 56 us less for it (5.21 -> 4.10 ms per 20 cycles with their copies).
+// the second round of shuffles costs more than the shorter instruction stream gains.)  In single precision both
+// neighbours go through the paired instructions, and two steps alternate between two sets of registers, with no copies
+// between them: each took about 4 us off a 185 us four-level cycle at 528 x 136.
 template <int PREC, int TL>
 __global__ void __launch_bounds__(kLusgsT) lusgs_kernel(const __grid_constant__ StepArgs A,
                                                         const __grid_constant__ CurvGeom G,
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kLusgsT) lusgs_kernel(const __grid_constant__ 
         // a neighbour that is not there has a zero increment, whose contribution is exactly zero
         const int ci = min(li, ex - 1), cj = min(max(lj, 0), ey - 1);
         const int q = cj * TL + ci;
-        t.q = li < ex && lj >= 0 && lj < ey ? q : -1;
+        t.q = kk < nk && li < ex && lj >= 0 && lj < ey ? q : -1;
         t.ni = dir ? ci + 1 < ex : ci > 0;
         t.nj = dir ? cj + 1 < ey : cj > 0;
         const int qi = t.ni ? (dir ? q + 1 : q - 1) : q, qj = t.nj ? (dir ? q + TL : q - TL) : q;
@@ -190,11 +191,8 @@ __global__ void __launch_bounds__(kLusgsT) lusgs_kernel(const __grid_constant__ 
         for (int v = 0; v < 4; ++v) t.x0[v] = X[v * TG::NC + q];
         t.id = ID[q];
       };
-      Step cur, nxt;
-      read(0, cur);
       const int src = dir ? tid + 1 : tid - 1;
-      for (int kk = 0; kk < nk; ++kk) {
-        read(min(kk + 1, nk - 1), nxt);
+      auto step = [&](const Step& cur) {
         R xi[4], xj[4], ai[4], aj[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
@@ -202,8 +200,23 @@ __global__ void __launch_bounds__(kLusgsT) lusgs_kernel(const __grid_constant__ 
           xi[v] = cur.ni ? t : R(0);
           xj[v] = cur.nj ? x[v] : R(0);
         }
-        offdiag<R>(gm1, cur.wi, xi, sgn * cur.fi[0], sgn * cur.fi[1], cur.fi[2], ai);
-        offdiag<R>(gm1, cur.wj, xj, sgn * cur.fj[0], sgn * cur.fj[1], cur.fj[2], aj);
+        if constexpr (std::is_same<R, float>::value) {  // the two neighbours on the paired FP32 instructions
+          F2 w2[5], x2[4], a2[4];
+#pragma unroll
+          for (int v = 0; v < 5; ++v) w2[v] = F2(cur.wi[v], cur.wj[v]);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) x2[v] = F2(xi[v], xj[v]);
+          offdiag<F2>(F2(gm1), w2, x2, F2(sgn * cur.fi[0], sgn * cur.fj[0]), F2(sgn * cur.fi[1], sgn * cur.fj[1]),
+                      F2(cur.fi[2], cur.fj[2]), a2);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            ai[v] = a2[v].v.x;
+            aj[v] = a2[v].v.y;
+          }
+        } else {
+          offdiag<R>(gm1, cur.wi, xi, sgn * cur.fi[0], sgn * cur.fi[1], cur.fi[2], ai);
+          offdiag<R>(gm1, cur.wj, xj, sgn * cur.fj[0], sgn * cur.fj[1], cur.fj[2], aj);
+        }
         // forward: dW* = (-R - acc) / D; backward: dW = dW* - acc / D
         if (cur.q >= 0) {
 #pragma unroll
@@ -212,7 +225,14 @@ __global__ void __launch_bounds__(kLusgsT) lusgs_kernel(const __grid_constant__ 
             X[v * TG::NC + cur.q] = x[v];
           }
         }
-        cur = nxt;
+      };
+      Step a, b;  // in turn: no copies between them
+      read(0, a);
+      for (int kk = 0; kk < nk; kk += 2) {
+        read(kk + 1, b);
+        step(a);
+        read(kk + 2, a);
+        step(b);
       }
     }
   }
