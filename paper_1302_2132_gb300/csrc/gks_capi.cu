@@ -149,7 +149,9 @@ __global__ void __launch_bounds__(kThreads) diag_kernel(const __grid_constant__ 
     f1 = ((const R*)A.f1)[c];
     if (g.turb_model != TURB_MUT) f2 = ((const R*)A.f2)[c];
   }
-  R val = tau_turb_cell<D, R>(g.turb_model, g.turb_cons != 0, kc, Wn, NN, idx, strides, igrad, pos, f1, f2);
+  const int ims[3] = {idx - strides[0], idx - strides[1], idx - strides[2]};
+  const int ips[3] = {idx + strides[0], idx + strides[1], idx + strides[2]};
+  R val = tau_turb_cell<D, R>(g.turb_model, g.turb_cons != 0, kc, Wn, NN, idx, ims, ips, igrad, pos, f1, f2);
   if (what == 1) {  // rarefaction: (mu/p + tau_t) |div U|
     R w[nv];
     for (int v = 0; v < nv; ++v) w[v] = Wn[v * NN + idx];

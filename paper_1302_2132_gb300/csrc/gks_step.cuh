@@ -427,6 +427,36 @@ __device__ __forceinline__ long field_cell(const DevGrid& g, int D, int i, int j
   return cell_index(g, c[0], c[1], c[2]);
 }
 
+// Shared-memory layout of a tile's states, slopes and fluxes: in 2D single precision the four values of a cell or
+// face together, so that one 16-byte access moves them (the step is bound by its instruction count, and its faces and
+// ring cells read whole states); otherwise one plane per variable, also for WENO-5 (H = 3), whose six cells per
+// face then hold too many registers at once (603 x 501: 2131 us per 48 steps in planes, 2271 together).  48 steps in
+// double-state form, 1024^2: 4328 us in planes, 4164 together; 1024 x 384: 1959 and 1891.
+template <int D, class R, int H, int N> struct CellData {
+  static constexpr bool AOS = D == 2 && sizeof(R) == sizeof(float) && H == 2;
+  __device__ __forceinline__ static int at(int v, int l) { return AOS ? 4 * l + v : v * N + l; }
+  __device__ __forceinline__ static void get(const R* p, int l, R* w) {
+    if constexpr (AOS) {
+      const float4 q = reinterpret_cast<const float4*>(p)[l];
+      w[0] = q.x;
+      w[1] = q.y;
+      w[2] = q.z;
+      w[3] = q.w;
+    } else {
+#pragma unroll
+      for (int v = 0; v < D + 2; ++v) w[v] = p[v * N + l];
+    }
+  }
+  __device__ __forceinline__ static void put(R* p, int l, const R* w) {
+    if constexpr (AOS) {
+      reinterpret_cast<float4*>(p)[l] = make_float4(w[0], w[1], w[2], w[3]);
+    } else {
+#pragma unroll
+      for (int v = 0; v < D + 2; ++v) p[v * N + l] = w[v];
+    }
+  }
+};
+
 template <class R>
 __device__ __forceinline__ R load_field(const StepArgs& A, const void* f, int D, int i, int j, int k) {
   return ((const R*)f)[field_cell(A.g, D, i, j, k)];
@@ -434,11 +464,12 @@ __device__ __forceinline__ R load_field(const StepArgs& A, const void* f, int D,
 
 // Turbulent part of the relaxation time of one cell (Eqs. tauttrivial, tautchen, tautchenadjusted
 // with T = p/rho); S = sqrt(2 S_ij S_ij) from central differences of the velocity.
-// igrad[a][p] = 1 / (distance between the centres of halo cells p - 1 and p + 1 along axis a).
+// igrad[a][p] = 1 / (distance between the centres of halo cells p - 1 and p + 1 along axis a); ims[a] and ips[a] are the
+// indices of the two neighbours along axis a.
 template <int D, class R>
 __device__ __forceinline__ R tau_turb_cell(int turb_model, bool cons, const Consts<R>& kc, const R* Ws, int stride_v,
-                                           int idx, const int* strides, const R* const* igrad, const int* pos,
-                                           R f1, R f2) {
+                                           int idx, const int* ims, const int* ips, const R* const* igrad,
+                                           const int* pos, R f1, R f2) {
   if (turb_model == TURB_NONE) return R(0);
   R w[D + 2];
 #pragma unroll
@@ -453,7 +484,7 @@ __device__ __forceinline__ R tau_turb_cell(int turb_model, bool cons, const Cons
   R grad[D][D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    const int im = idx - strides[a], ip = idx + strides[a];
+    const int im = ims[a], ip = ips[a];
     const R id = igrad[a][pos[a]];
     const R irm = g_rcp(Ws[im]), irp = g_rcp(Ws[ip]);
 #pragma unroll
@@ -485,8 +516,8 @@ __device__ __forceinline__ R tau_turb_cell(int turb_model, bool cons, const Cons
 // epsilon|omega case selected to zero at the end.
 template <int D, class R>
 __device__ __forceinline__ R tau_turb_two_eq(bool keps, bool cons, const Consts<R>& kc, const R* Ws, int stride_v,
-                                             int idx, const int* strides, const R* const* igrad, const int* pos,
-                                             R f1, R f2) {
+                                             int idx, const int* ims, const int* ips, const R* const* igrad,
+                                             const int* pos, R f1, R f2) {
   R w[D + 2];
 #pragma unroll
   for (int v = 0; v < D + 2; ++v) w[v] = Ws[v * stride_v + idx];
@@ -498,7 +529,7 @@ __device__ __forceinline__ R tau_turb_two_eq(bool keps, bool cons, const Consts<
   R grad[D][D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    const int im = idx - strides[a], ip = idx + strides[a];
+    const int im = ims[a], ip = ips[a];
     const R id = igrad[a][pos[a]];
     const R irm = g_rcp(Ws[im]), irp = g_rcp(Ws[ip]);
 #pragma unroll
@@ -673,7 +704,10 @@ __device__ __noinline__ void ring_phase(const Consts<typename PrecT<PREC>::R> kc
   constexpr int kThreads = G::T, nv = D + 2, HX = G::HX, HY = G::HY;
   constexpr bool PRE = pre_slopes<D, PREC, V>();
   const int tid = threadIdx.x;
-  const int strides[3] = {1, HX, HX * HY};
+  using CW = CellData<D, R, H, G::NH>;
+  using CS = CellData<D, R, H, G::NR>;
+  constexpr int el = CW::AOS ? 4 : 1, ev = CW::AOS ? 1 : G::NH;  // elements from cell to cell, variable to variable
+  const int strides[3] = {el, el * HX, el * HX * HY};
   const R* igrad[3] = {igx, igy, igz};
   const R* icent[3] = {icx, icy, icz};
   constexpr int NU = ring_used<D, G>();
@@ -699,13 +733,35 @@ __device__ __noinline__ void ring_phase(const Consts<typename PrecT<PREC>::R> kc
         const int hi = ri + H - 1, hj = D >= 2 ? rj + H - 1 : 0, hk = D >= 3 ? rk + H - 1 : 0;
         const int idx = (hk * HY + hj) * HX + hi;
         const int pos[3] = {hi, hj, hk};
+        // when a cell's values lie together, the cell (4) and its neighbours along x and y in registers
+        R nb[CW::AOS ? 5 : 1][nv];
+        if constexpr (CW::AOS) {
+          const int off[5] = {-1, 1, -HX, HX, 0};
+#pragma unroll
+          for (int k = 0; k < 5; ++k) CW::get(Ws, idx + off[k], nb[k]);
+        }
+        const R* Wt = CW::AOS ? &nb[0][0] : Ws;
+        const int it = CW::AOS ? 4 * nv : idx;
+        const int ims[3] = {CW::AOS ? 0 : idx - strides[0], CW::AOS ? 2 * nv : idx - strides[1], idx - strides[2]};
+        const int ips[3] = {CW::AOS ? nv : idx + strides[0], CW::AOS ? 3 * nv : idx + strides[1], idx + strides[2]};
         if constexpr (TWO_EQ)
-          tv[q] = tau_turb_two_eq<D, R>(KEPS, cons, kc, Ws, G::NH, idx, strides, igrad, pos, Fl[l],
-                                        Fl[G::NR + l]);
+          tv[q] = tau_turb_two_eq<D, R>(KEPS, cons, kc, Wt, ev, it, ims, ips, igrad, pos, Fl[l], Fl[G::NR + l]);
         else
-          tv[q] = tau_turb_cell<D, R>(turb_model, cons, kc, Ws, G::NH, idx, strides, igrad, pos,
+          tv[q] = tau_turb_cell<D, R>(turb_model, cons, kc, Wt, ev, it, ims, ips, igrad, pos,
                                       turb_model == TURB_NONE ? R(0) : Fl[l], R(0));
-        if constexpr (PRE && PAIRXY) {
+        if constexpr (PRE && PAIRXY && CW::AOS) {
+          const F2 im2(icent[0][pos[0]], icent[1][pos[1]]), ip2(icent[0][pos[0] + 1], icent[1][pos[1] + 1]);
+#pragma unroll
+          for (int v = 0; v < nv; ++v) {
+            const F2 c(nb[4][v]);
+            const F2 dm = F2((c - F2(nb[0][v], nb[2][v])) * im2);
+            const F2 dp = F2((F2(nb[1][v], nb[3][v]) - c) * ip2);
+            const F2 ab = F2(dm * dp), den = dm + dp;
+            const F2 lim = F2((ab + ab) * g_rcp(den));
+            sv[q][v] = ab.v.x > 0.0f ? lim.v.x : 0.0f;
+            sv[q][nv + v] = ab.v.y > 0.0f ? lim.v.y : 0.0f;
+          }
+        } else if constexpr (PRE && PAIRXY) {
           const F2 im2(icent[0][pos[0]], icent[1][pos[1]]), ip2(icent[0][pos[0] + 1], icent[1][pos[1] + 1]);
 #pragma unroll
           for (int v = 0; v < nv; ++v) {
@@ -734,7 +790,7 @@ __device__ __noinline__ void ring_phase(const Consts<typename PrecT<PREC>::R> kc
             const R im = icent[a][pos[a]], ip = icent[a][pos[a] + 1];
 #pragma unroll
             for (int v = 0; v < nv; ++v) {
-              const R* pc = Ws + v * G::NH + idx;
+              const R* pc = Ws + CW::at(v, idx);
               sv[q][a * nv + v] = limiter<R>(LIM, (pc[0] - pc[-strides[a]]) * im, (pc[strides[a]] - pc[0]) * ip);
             }
           }
@@ -748,7 +804,7 @@ __device__ __noinline__ void ring_phase(const Consts<typename PrecT<PREC>::R> kc
         taus[l] = tv[q];
         if constexpr (PRE) {
 #pragma unroll
-          for (int j = 0; j < NS; ++j) Ss[j * G::NR + l] = sv[q][j];
+          for (int a = 0; a < D; ++a) CS::put(Ss + a * nv * G::NR, l, &sv[q][a * nv]);
         }
       }
     }
@@ -798,6 +854,9 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
   R* Ss = Fs + (size_t)nv * G::NF;          // PRE: [D][nv][NR] limited slopes of the ring cells along each axis
   R* Fl = Ss + (PRE ? (size_t)D * nv * G::NR : 0);  // [2][NR] turbulence fields of the ring cells
   float* Lo = (float*)(Fl + 2 * G::NR);             // PREC_F32: [nv][NC] low words of the tile's cells
+  using CW = CellData<D, R, H, G::NH>;
+  using CS = CellData<D, R, H, G::NR>;
+  using CF = CellData<D, R, H, G::NF>;
   // the stored type is the arithmetic type (FP64, FP32 pair): cells that are plain copies of grid
   // cells are copied as they are
   constexpr bool ASYNC = sizeof(S) == sizeof(R);
@@ -868,10 +927,14 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       const S* src = (const S*)A.Win + cell_index(g, ox + hi - H, D >= 2 ? oy + hj - H : 0, D >= 3 ? oz + hk - H : 0);
 #pragma unroll
       for (int v = 0; v < nv; ++v) {
-        if constexpr (DSTAGE)
+        if constexpr (DSTAGE) {
           cp_async<16>(&Wd[v * G::NH + l], src + (long)v * g.ncell);
-        else
+        } else if constexpr (CW::AOS) {
+          cp_async<sizeof(S)>(&Ws[CW::at(v, l)], src + (long)v * g.ncell);
+          cp_async<sizeof(S)>(&Ws[CW::at(v, l + 1)], src + (long)v * g.ncell + 1);
+        } else {
           cp_async<2 * sizeof(S)>(&Ws[v * G::NH + l], src + (long)v * g.ncell);
+        }
       }
     }
   }
@@ -887,7 +950,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
         for (int v = 0; v < nv; ++v) cp_async<8>(&Wd[v * G::NH + l], src + (long)v * g.ncell);
       } else {
 #pragma unroll
-        for (int v = 0; v < nv; ++v) cp_async<sizeof(S)>(&Ws[v * G::NH + l], src + (long)v * g.ncell);
+        for (int v = 0; v < nv; ++v) cp_async<sizeof(S)>(&Ws[CW::at(v, l)], src + (long)v * g.ncell);
       }
     } else if constexpr (DSTAGE) {
       // wall image or Dirichlet ghost: the boundary rule in double precision, converted with the rest
@@ -898,8 +961,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     } else {
       R w[nv];
       load_cell<D, PREC>(g, A.Win, kc, gi, gj, gk, w);
-#pragma unroll
-      for (int v = 0; v < nv; ++v) Ws[v * G::NH + l] = w[v];
+      CW::put(Ws, l, w);
     }
   }
   if (g.turb_model != TURB_NONE) {
@@ -999,16 +1061,21 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     // before the conversion (the same cell-to-thread assignment as the staging loops above)
     if (pairs) {
       for (int l2 = tid; l2 < G::NH / 2; l2 += kThreads) {
+        R a[nv], b[nv];
 #pragma unroll
         for (int v = 0; v < nv; ++v) {
-          Ws[v * G::NH + 2 * l2] = d2f(Wd[v * G::NH + 2 * l2]);
-          Ws[v * G::NH + 2 * l2 + 1] = d2f(Wd[v * G::NH + 2 * l2 + 1]);
+          a[v] = d2f(Wd[v * G::NH + 2 * l2]);
+          b[v] = d2f(Wd[v * G::NH + 2 * l2 + 1]);
         }
+        CW::put(Ws, 2 * l2, a);
+        CW::put(Ws, 2 * l2 + 1, b);
       }
     } else {
       for (int l = tid; l < G::NH; l += kThreads) {
+        R a[nv];
 #pragma unroll
-        for (int v = 0; v < nv; ++v) Ws[v * G::NH + l] = d2f(Wd[v * G::NH + l]);
+        for (int v = 0; v < nv; ++v) a[v] = d2f(Wd[v * G::NH + l]);
+        CW::put(Ws, l, a);
       }
     }
   }
@@ -1105,29 +1172,60 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       R* cr = in.cr;
       R* sl = in.sl;
       R* sr = in.sr;
+      // the values of cell (or ring cell) l in the face's frame
+      auto in_frame = [&](const R* base, auto cells, int l, R* w) {
+        using C = decltype(cells);
+        if constexpr (C::AOS) {
+          C::get(base, l, w);
+          if (ax == 1) {
+            const R t = w[1];
+            w[1] = w[2];
+            w[2] = t;
+          }
+        } else {
+#pragma unroll
+          for (int v = 0; v < nv; ++v) w[v] = base[C::at((v >= 1 && v <= D) ? 1 + perm[v - 1] : v, l)];
+        }
+      };
+      R w1[nv], w2[nv];                                     // the two cells
+      [[maybe_unused]] R b1[nv], b2[nv];                    // their slopes along the normal
+      in_frame(Ws, CW{}, hc - sn, w1);
+      in_frame(Ws, CW{}, hc, w2);
+      [[maybe_unused]] R o1[nv], o2[nv], oo1[nv], oo2[nv];  // the next cells outward, and the next (WENO-5)
+      if constexpr (RECON != RECON_MUSCL2) {
+        in_frame(Ws, CW{}, hc - 2 * sn, o1);
+        in_frame(Ws, CW{}, hc + sn, o2);
+        if constexpr (RECON == RECON_WENO5) {
+          in_frame(Ws, CW{}, hc - 3 * sn, oo1);
+          in_frame(Ws, CW{}, hc + 2 * sn, oo2);
+        }
+      } else if constexpr (PRE) {
+        in_frame(Ss + ax * nv * G::NR, CS{}, rl, b1);
+        in_frame(Ss + ax * nv * G::NR, CS{}, rc, b2);
+      }
 #pragma unroll
       for (int v = 0; v < nv; ++v) {
-        const int sv = (v >= 1 && v <= D) ? 1 + perm[v - 1] : v;
-        const R* p = Ws + sv * G::NH + hc;
-        const R s1 = p[-sn], s2 = p[0];
+        const R s1 = w1[v], s2 = w2[v];
         if constexpr (RECON != RECON_MUSCL2) {
           // higher-order face values from the normal stencil (cells pn-3 .. pn+2); the normal
           // slopes are the one-sided differences to them
           if constexpr (RECON == RECON_WENO5) {
-            weno5_sides(p[-3 * sn], p[-2 * sn], s1, s2, p[sn], p[2 * sn], wl[v], wr[v]);
+            weno5_sides(oo1[v], o1[v], s1, s2, o2[v], oo2[v], wl[v], wr[v]);
           } else {
-            wl[v] = muscl3_right<R>(p[-2 * sn], s1, s2);
-            wr[v] = muscl3_left<R>(s1, s2, p[sn]);
+            wl[v] = muscl3_right<R>(o1[v], s1, s2);
+            wr[v] = muscl3_left<R>(s1, s2, o2[v]);
           }
           sl[v] = (wl[v] - s1) * i2h1;
           sr[v] = (s2 - wr[v]) * i2h2;
         } else if (PRE) {
-          sl[v] = Ss[(ax * nv + sv) * G::NR + rl];
-          sr[v] = Ss[(ax * nv + sv) * G::NR + rc];
+          sl[v] = b1[v];
+          sr[v] = b2[v];
           wl[v] = s1 + R(0.5) * h1 * sl[v];
           wr[v] = s2 - R(0.5) * h2 * sr[v];
         } else {
           // MUSCL with the tabulated inverse centre distances (cells pn-2 .. pn+1 along the normal)
+          const R* p = Ws + CW::at((v >= 1 && v <= D) ? 1 + perm[v - 1] : v, hc);
+          static_assert(PRE || !CW::AOS, "p steps by cells of a plane");
           const R dm = (s1 - p[-2 * sn]) * icn[pn - 1], dc = (s2 - s1) * icn[pn], dp = (p[sn] - s2) * icn[pn + 1];
           sl[v] = limiter<R>(g.limiter, dm, dc);
           sr[v] = limiter<R>(g.limiter, dc, dp);
@@ -1155,12 +1253,8 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
 #pragma unroll
         for (int s = 0; s < D - 1; ++s) {
           const int ta = perm[1 + s];
-#pragma unroll
-          for (int v = 0; v < nv; ++v) {
-            const int sv = (v >= 1 && v <= D) ? 1 + perm[v - 1] : v;
-            in.tl[s][v] = Ss[(ta * nv + sv) * G::NR + rl];
-            in.tr[s][v] = Ss[(ta * nv + sv) * G::NR + rc];
-          }
+          in_frame(Ss + ta * nv * G::NR, CS{}, rl, in.tl[s]);
+          in_frame(Ss + ta * nv * G::NR, CS{}, rc, in.tr[s]);
         }
       } else if (MULTID) {
 #pragma unroll
@@ -1192,10 +1286,16 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     // the face's time-integrated mass flux
     auto store = [&](int f, const FaceIn& in, const R* F, auto ax_tag) {
       constexpr int AX = decltype(ax_tag)::value;  // the face's axis if known at compile time, else -1
-      Fs[0 * G::NF + f] = F[0];
+      if constexpr (CF::AOS) {
+        const bool y = AX >= 0 ? AX == 1 : in.ax == 1;
+        const R Fg[nv] = {F[0], y ? F[2] : F[1], y ? F[1] : F[2], F[3]};
+        CF::put(Fs, f, Fg);
+      } else {
+        Fs[0 * G::NF + f] = F[0];
 #pragma unroll
-      for (int k = 0; k < D; ++k) Fs[(1 + (AX >= 0 ? face_perm_c<D>(AX, k) : in.perm[k])) * G::NF + f] = F[1 + k];
-      Fs[(D + 1) * G::NF + f] = F[D + 1];
+        for (int k = 0; k < D; ++k) Fs[(1 + (AX >= 0 ? face_perm_c<D>(AX, k) : in.perm[k])) * G::NF + f] = F[1 + k];
+        Fs[(D + 1) * G::NF + f] = F[D + 1];
+      }
       if (A.mflux[0]) {
         // global face (cell c = tile origin + (ci, cj, ck), face c - 1/2 along ax)
         const int gc[3] = {ox + in.ci, oy + in.cj, oz + in.ck};
@@ -1335,13 +1435,25 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
 #pragma unroll
     for (int d = 0; d < D; ++d) ih[d] = (d == 0 ? iwx[li + H] : (d == 1 ? iwy[lj + H] : iwz[lk + H]));
     R wn[nv];
+    [[maybe_unused]] R dF[CF::AOS ? D : 1][nv], w0[nv];  // flux differences and the staged state, read whole
+    if constexpr (CF::AOS) {
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        R a[nv];
+        CF::get(Fs, fm[d], a);
+        CF::get(Fs, fp[d], dF[d]);
+#pragma unroll
+        for (int v = 0; v < nv; ++v) dF[d][v] -= a[v];
+      }
+    }
     // the cell's old state: staged in shared memory (FP64, float pair), else loaded into wold above
     const int hidx = ((lk + (D >= 3 ? H : 0)) * HY + (lj + (D >= 2 ? H : 0))) * HX + (li + H);
+    CW::get(Ws, hidx, w0);
 #pragma unroll
     for (int v = 0; v < nv; ++v) {
       const long gidx = (long)v * g.ncell + c;
       if constexpr (PREC == PREC_F64) {
-        double w = (double)Ws[v * G::NH + hidx];
+        double w = (double)w0[v];
 #pragma unroll
         for (int d = 0; d < D; ++d) w -= ((double)Fs[v * G::NF + fp[d]] - (double)Fs[v * G::NF + fm[d]]) * (double)ih[d];
         ((double*)A.Wout)[gidx] = w;
@@ -1349,10 +1461,11 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       } else {
         R inc = R(0);
 #pragma unroll
-        for (int d = 0; d < D; ++d) inc -= (Fs[v * G::NF + fp[d]] - Fs[v * G::NF + fm[d]]) * ih[d];
+        for (int d = 0; d < D; ++d)
+          inc -= (CF::AOS ? dF[CF::AOS ? d : 0][v] : Fs[v * G::NF + fp[d]] - Fs[v * G::NF + fm[d]]) * ih[d];
         if constexpr (PREC == PREC_F32) {
           // (hi, lo) += inc with an error-free sum, then renormalise
-          const float hi = (float)Ws[v * G::NH + hidx], lo = Lo[v * G::NC + l];
+          const float hi = (float)w0[v], lo = Lo[v * G::NC + l];
           const float s = hi + inc;
           const float bb = s - hi;
           const float err = (hi - (s - bb)) + (inc - bb);
@@ -1365,7 +1478,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
         } else {
           const double w = wold[qc][v] + f2d(inc);
           ((double*)A.Wout)[gidx] = w;
-          wn[v] = (float)Ws[v * G::NH + hidx] + inc;  // the new state in float, for the rate and status
+          wn[v] = (float)w0[v] + inc;  // the new state in float, for the rate and status
         }
       }
     }
