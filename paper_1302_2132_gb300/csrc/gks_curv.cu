@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(KwTile::T) curv_komega_kernel(const __grid_con
   if (K.sources) {
     const int sc = (lj + 2) * SX + li + 2;
     R Sk, Sw;
-    kw_sources<R, SX>(sk, sw, sr, su, sv, sc, gsx, gsy, A, alpha, beta_star, sigma_do, C_lim, Sk, Sw);
+    kw_sources<R, SX>(sk, sw, sr[sc], su, sv, sc, gsx, gsy, A, alpha, beta_star, sigma_do, C_lim, Sk, Sw);
     const R w0 = sw[sc];
     ak += dt * Sk;
     aw += dt * Sw;
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(KwTile::T) steady_komega_kernel(const __grid_c
   dw = base + dw / rho;
   if (K.sources) {
     R Sk, Sw;
-    kw_sources<R, SX>(sk, sw, sr, su, sv, sc, gsx, gsy, A, alpha, beta_star, sigma_do, C_lim, Sk, Sw);
+    kw_sources<R, SX>(sk, sw, sr[sc], su, sv, sc, gsx, gsy, A, alpha, beta_star, sigma_do, C_lim, Sk, Sw);
     const R w0 = sw[sc];
     rk -= A * (Sk - beta_star * w0 * rk0);
     rw -= A * (Sw - beta0 * w0 * rw0);

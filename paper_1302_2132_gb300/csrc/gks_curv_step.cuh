@@ -122,10 +122,10 @@ __device__ __forceinline__ void kw_face(const R* vk, const R* vw, R rl, R rr, co
 // Green-Gauss gradients from the staged neighbours (face values the means of the two cells);
 // gsx, gsy: the outward n_x L, n_y L of the faces i-1/2, i+1/2, j-1/2, j+1/2.
 template <class R, int SX>
-__device__ __forceinline__ void kw_sources(const R* sk, const R* sw, const R* sr, const R* su, const R* sv, int sc,
+__device__ __forceinline__ void kw_sources(const R* sk, const R* sw, R rho, const R* su, const R* sv, int sc,
                                            const R* gsx, const R* gsy, R A, R alpha, R beta_star, R sigma_do, R C_lim,
                                            R& Sk, R& Sw) {
-  const R rho = sr[sc], k0 = sk[sc], w0 = sw[sc];
+  const R k0 = sk[sc], w0 = sw[sc];
   const int nb[4] = {sc - 1, sc + 1, sc - SX, sc + SX};
   const R uc[2] = {su[sc], sv[sc]};
   R gu[2][2] = {{R(0), R(0)}, {R(0), R(0)}}, gk[2] = {R(0), R(0)}, gw[2] = {R(0), R(0)};
@@ -203,6 +203,21 @@ struct CurvTileGeom {
   }
 };
 
+// Limiter of two variables' differences (van Leer on the paired instructions) into s[0], s[1].  The step issues
+// instructions most of its time, and the slopes of a face are 8 to 16 limiters: two at a time, out of states whose
+// values lie together (CellData; alone within 1 us), 96 steps at 528 x 136 took 1349 us before and 1273 after,
+// 1056 x 272 3513 and 3354.
+__device__ __forceinline__ void limiter_pair(int lim, F2 a, F2 b, float* s) {
+  if (lim == LIM_VANLEER) {
+    const F2 ab = a * b, q = (ab + ab) * g_rcp(F2(a + b));
+    s[0] = ab.v.x > 0.0f ? q.v.x : 0.0f;
+    s[1] = ab.v.y > 0.0f ? q.v.y : 0.0f;
+  } else {
+    s[0] = limiter<float>(lim, a.v.x, b.v.x);
+    s[1] = limiter<float>(lim, a.v.y, b.v.y);
+  }
+}
+
 // MODE 0: one time step (A.Win -> A.Wout, control block as the rectilinear step).  MODE 1: the
 // steady residual of A.Win (SteadyArgs): the local steps s of the tile and its first ring (the ghost ring
 // takes its source cell's; stored for the tile cells), face windows cfl_flux min(s_l, s_r), flux rates times
@@ -236,6 +251,9 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
   constexpr bool CONS = TR || SEPARATE_KW;
   constexpr int NFX = TG::NFX, NF = TG::NF, TX = TG::TX, NT = TG::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  // states, face records (two groups of four) and fluxes in the layouts of CellData
+  using CW = CellData<2, R, H, NH>;
+  using CF = CellData<2, R, H, NF>;
   R* Ws = (R*)smem_raw;    // [4][NH] state of the tile and its halo
   R* Gs = Ws + 4 * NH;     // [8][NF] face records: i-faces (X + 1) x Y, then j-faces X x (Y + 1)
   R* Fs = Gs + 8 * NF;     // [4][NF] face fluxes times length
@@ -280,7 +298,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
     }
     const R* src = (const R*)G.face[a];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) cp_async<sizeof(R)>(&Gs[q * NF + l], &src[(long)q * nf + gf]);
+    for (int q = 0; q < 8; ++q) cp_async<sizeof(R)>(&Gs[(q & 4) * NF + CF::at(q & 3, l)], &src[(long)q * nf + gf]);
   }
   // everything below may read what the previous kernel in the stream wrote: with a programmatic
   // (early) launch of this kernel, wait here for that kernel's completion; the face records
@@ -308,7 +326,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
     if (PREC != PREC_F32D && gi >= 0 && gi < n0 && gj >= 0 && gj < n1) {
       const S* src = (const S*)A.Win + (long)gj * n0 + gi;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) cp_async<sizeof(R)>(&Ws[v * NH + l], src + (long)v * g.ncell);
+      for (int v = 0; v < 4; ++v) cp_async<sizeof(R)>(&Ws[CW::at(v, l)], src + (long)v * g.ncell);
       continue;
     }
     if (gi >= -H && gi < n0 + H && gj >= -H && gj < n1 + H) {
@@ -318,8 +336,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       w[1] = w[2] = R(0);
       w[3] = R(1);
     }
-#pragma unroll
-    for (int v = 0; v < 4; ++v) Ws[v * NH + l] = w[v];
+    CW::put(Ws, l, w);
   }
   if (PREC == PREC_F32 && MODE == 0)
     for (int l = tid; l < X * Y; l += T) {
@@ -369,8 +386,10 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       const R rho_s = (R)((const S*)A.Win)[sc];
       Ks[l] = g_div(((const R*)A.f1)[sc], rho_s);
       Os[l] = g_div(((const R*)A.f2)[sc], rho_s);
-      Us[l] = g_div(Ws[NH + l], Ws[l]);
-      Vs[l] = g_div(Ws[2 * NH + l], Ws[l]);
+      R w[4];
+      CW::get(Ws, l, w);
+      Us[l] = g_div(w[1], w[0]);
+      Vs[l] = g_div(w[2], w[0]);
     }
     if (g.turb_model == TURB_NONE) __syncthreads();  // else the tau phase's barrier follows
   }
@@ -385,12 +404,11 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       if (gi >= 0 && gi < n0 && gj >= 0 && gj < n1) {
         const int h0 = (tj + H) * HX + (ti + H);
         const int off[5] = {-1, 1, -HX, HX, 0};
-        if (turb)
-          t = tau_gg<R, CONS>(g, kc, G, A.f1, A.f2, gi, gj, [&](int q, int v) { return Ws[v * NH + h0 + off[q]]; });
-        if (MODE == 1) {
-          const R w[4] = {Ws[h0], Ws[NH + h0], Ws[2 * NH + h0], Ws[3 * NH + h0]};
-          sl = g_rcp(curv_rate<R>(w, kc.gamma, G, n0, gi, gj, (long)gj * n0 + gi));
-        }
+        R nb[5][4];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) CW::get(Ws, h0 + off[q], nb[q]);
+        if (turb) t = tau_gg<R, CONS>(g, kc, G, A.f1, A.f2, gi, gj, [&](int q, int v) { return nb[q][v]; });
+        if (MODE == 1) sl = g_rcp(curv_rate<R>(nb[4], kc.gamma, G, n0, gi, gj, (long)gj * n0 + gi));
       } else if (gi >= -1 && gi <= n0 && gj >= -1 && gj <= n1) {  // a ghost cell takes its source cell's value
         const long sc = field_cell(g, 2, gi, gj, 0);
         const int si = (int)(sc % n0), sj = (int)(sc / n0);
@@ -435,20 +453,23 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
         valid = ox + li < n0 && oy + lj <= n1;
       }
       if (!valid) continue;
-      const R nx = Gs[l], ny = Gs[NF + l], L = Gs[2 * NF + l];
-      const R i01 = Gs[3 * NF + l], i12 = Gs[4 * NF + l], i23 = Gs[5 * NF + l];
-      const R dl = Gs[6 * NF + l], dr = Gs[7 * NF + l];
+      R fr[8];
+      CF::get(Gs, l, fr);
+      CF::get(Gs + 4 * NF, l, fr + 4);
+      const R nx = fr[0], ny = fr[1], L = fr[2];
+      const R i01 = fr[3], i12 = fr[4], i23 = fr[5];
+      const R dl = fr[6], dr = fr[7];
       // stencil: cells li - 2 .. li + 1 along the face normal's grid line (WENO-5 also li - 3 and
       // li + 2), rotated into the face frame
       const int base = a == 0 ? (lj + H) * HX + li + H - 2 : (lj + H - 2) * HX + li + H;
       const int stride = a == 0 ? 1 : HX;
       auto rotated = [&](int h, R* r) {
-        const R w0 = Ws[h], w1 = Ws[NH + h], w2 = Ws[2 * NH + h], w3 = Ws[3 * NH + h];
-        r[0] = w0;
+        CW::get(Ws, h, r);
+        const R w1 = r[1], w2 = r[2];
         r[1] = w1 * nx + w2 * ny;
         r[2] = -w1 * ny + w2 * nx;
-        r[3] = w3;
       };
+      constexpr bool PAIRED = std::is_same<R, float>::value;  // two variables' slopes on the paired instructions
       R S4[4][4];
 #pragma unroll
       for (int s = 0; s < 4; ++s) rotated(base + s * stride, S4[s]);
@@ -456,10 +477,24 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       if (RC == 0) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const R dm = (S4[1][v] - S4[0][v]) * i01, dc = (S4[2][v] - S4[1][v]) * i12,
-                  dp = (S4[3][v] - S4[2][v]) * i23;
-          sl[v] = FO ? R(0) : limiter<R>(g.limiter, dm, dc);
-          sr[v] = FO ? R(0) : limiter<R>(g.limiter, dc, dp);
+          if constexpr (FO) {
+            sl[v] = sr[v] = R(0);
+          } else if constexpr (PAIRED) {
+            if (v & 1) continue;  // with its predecessor
+            auto two = [&](const R* w) { return F2(w[v], w[v + 1]); };
+            const F2 dm = (two(S4[1]) - two(S4[0])) * F2(i01), dc = (two(S4[2]) - two(S4[1])) * F2(i12),
+                     dp = (two(S4[3]) - two(S4[2])) * F2(i23);
+            limiter_pair(g.limiter, dm, dc, &sl[v]);
+            limiter_pair(g.limiter, dc, dp, &sr[v]);
+          } else {
+            const R dm = (S4[1][v] - S4[0][v]) * i01, dc = (S4[2][v] - S4[1][v]) * i12,
+                    dp = (S4[3][v] - S4[2][v]) * i23;
+            sl[v] = limiter<R>(g.limiter, dm, dc);
+            sr[v] = limiter<R>(g.limiter, dc, dp);
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
           wl[v] = S4[1][v] + dl * sl[v];
           wr[v] = S4[2][v] - dr * sr[v];
           cl[v] = S4[1][v];
@@ -516,24 +551,18 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
           const int h0 = a == 0 ? (lj + H) * HX + li + H - 1 + side : (lj + H - 1 + side) * HX + li + H;
           const R ihm = tg[(long)(2 * side) * nfa + gf], ihp = tg[(long)(2 * side + 1) * nfa + gf];
           R rm[4], rp[4];
+          rotated(h0 - step, rm);
+          rotated(h0 + step, rp);
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int h = q == 0 ? h0 - step : h0 + step;
-            const R w0 = Ws[h], w1 = Ws[NH + h], w2 = Ws[2 * NH + h], w3 = Ws[3 * NH + h];
-            R* r = q == 0 ? rm : rp;
-            r[0] = w0;
-            r[1] = w1 * nx + w2 * ny;
-            r[2] = -w1 * ny + w2 * nx;
-            r[3] = w3;
-          }
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            const R c0 = S4[1 + side][v];
-            const R t = limiter<R>(g.limiter, (c0 - rm[v]) * ihm, (rp[v] - c0) * ihp);
-            if (side == 0)
-              tl[0][v] = t;
-            else
-              trr[0][v] = t;
+          for (int v = 0; v < 4; v += PAIRED ? 2 : 1) {
+            R* t = side == 0 ? &tl[0][v] : &trr[0][v];
+            if constexpr (PAIRED) {
+              const F2 c0(S4[1 + side][v], S4[1 + side][v + 1]);
+              limiter_pair(g.limiter, (c0 - F2(rm[v], rm[v + 1])) * F2(ihm), (F2(rp[v], rp[v + 1]) - c0) * F2(ihp), t);
+            } else {
+              const R c0 = S4[1 + side][v];
+              *t = limiter<R>(g.limiter, (c0 - rm[v]) * ihm, (rp[v] - c0) * ihp);
+            }
           }
         }
       }
@@ -564,10 +593,8 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       else
         face_flux<2, R, MD, RAR>(wl, wr, cl, cr, sl, sr, tl, trr, dl, dr, tau_t, win, gas, g.abar_t0, F, &tau);
       const R L_ = Lw;
-      Fs[l] = F[0] * L_;
-      Fs[NF + l] = (F[1] * nx - F[2] * ny) * L_;
-      Fs[2 * NF + l] = (F[1] * ny + F[2] * nx) * L_;
-      Fs[3 * NF + l] = F[3] * L_;
+      const R Fg[4] = {F[0] * L_, (F[1] * nx - F[2] * ny) * L_, (F[1] * ny + F[2] * nx) * L_, F[3] * L_};
+      CF::put(Fs, l, Fg);
       if (TR) {
         R vk[4], vw[4];
 #pragma unroll
@@ -577,7 +604,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
         }
         const bool kf = sizeof(R) == sizeof(float);
         const R sigk = kf ? (R)A.kw_fsigma_star : (R)A.kw_sigma_star, sigw = kf ? (R)A.kw_fsigma : (R)A.kw_sigma;
-        const R fvr[7] = {Fs[l], L, i01, i12, i23, dl, dr};
+        const R fvr[7] = {Fg[0], L, i01, i12, i23, dl, dr};
         R out[2];
         kw_face<R>(vk, vw, S4[1][0], S4[2][0], fvr, dt, kc.mu, sigk, sigw, g.limiter, A.kw_diffusion, out);
         Gk[l] = out[0];
@@ -586,12 +613,22 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       if (SEPARATE_KW && A.mflux[0]) {  // the face's mass flux times L for a separate transport step:
                                         // time-integrated, or the rate over the residual's window
         const long gfm = a == 0 ? (long)(oy + lj) * (n0 + 1) + ox + li : (long)(oy + lj) * n0 + ox + li;
-        ((R*)A.mflux[a])[gfm] = Fs[l];
+        ((R*)A.mflux[a])[gfm] = Fg[0];
       }
     }
   }
   __syncthreads();
 
+  // sum of a cell's outward fluxes times length: faces fa, fa + 1 along i, fc, fc + X along j
+  auto cell_sum = [&](int fa, int fc, R* net) {
+    R f0[4], f1[4], f2[4], f3[4];
+    CF::get(Fs, fa + 1, f0);
+    CF::get(Fs, fa, f1);
+    CF::get(Fs, fc + X, f2);
+    CF::get(Fs, fc, f3);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) net[v] = f0[v] - f1[v] + f2[v] - f3[v];
+  };
   if (MODE == 1) {  // steady residual: sum of the outward flux rates times L, plus the forcing
     double s2 = 0.0;
     for (int l = tid; l < X * Y; l += T) {
@@ -600,14 +637,17 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       if (gi >= n0 || gj >= n1) continue;
       const long c = (long)gj * n0 + gi;
       const int fa = lj * (X + 1) + li, fc = NFX + lj * X + li;
+      R net[4], w0[4];
+      cell_sum(fa, fc, net);
+      CW::get(Ws, (lj + H) * HX + li + H, w0);
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        R r = Fs[v * NF + fa + 1] - Fs[v * NF + fa] + Fs[v * NF + fc + X] - Fs[v * NF + fc];
+        R r = net[v];
         const long q = (long)v * g.ncell + c;
         if (SA.forcing) r += ((const R*)SA.forcing)[q];
         if (SA.forcing_io) {  // FAS forcing of a coarse level; the level's state starts from this one
           ((R*)SA.forcing_io)[q] -= r;
-          ((S*)SA.W_start)[q] = (S)Ws[v * NH + (lj + H) * HX + li + H];
+          ((S*)SA.W_start)[q] = (S)w0[v];
         } else {
           ((R*)SA.R)[q] = r;
         }
@@ -637,20 +677,22 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
     const int fa = lj * (X + 1) + li, fc = NFX + lj * X + li;
     const int hidx = (lj + H) * HX + (li + H);
     const R ia = ((const R*)G.iarea)[c];
-    R wn[4];
+    R wn[4], w0[4], sum[4];
+    cell_sum(fa, fc, sum);
+    CW::get(Ws, hidx, w0);
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const R net = Fs[v * NF + fa + 1] - Fs[v * NF + fa] + Fs[v * NF + fc + X] - Fs[v * NF + fc];
+      const R net = sum[v];
       const long gidx = (long)v * g.ncell + c;
       if (PREC == PREC_F64) {
-        const double w_old = (double)Ws[v * NH + hidx];
+        const double w_old = (double)w0[v];
         const double w = w_old - (double)net * (double)ia;
         ((double*)A.Wout)[gidx] = w;
         wn[v] = (R)w;
       } else {
         const R inc = -net * ia;
         if (PREC == PREC_F32) {
-          const float hi = (float)Ws[v * NH + hidx], lo = Lo[v * X * Y + l];
+          const float hi = (float)w0[v], lo = Lo[v * X * Y + l];
           const float s_ = hi + inc;
           const float bb = s_ - hi;
           const float err = (hi - (s_ - bb)) + (inc - bb);
@@ -684,16 +726,18 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const R sgn = (q & 1) ? R(1) : R(-1);
-          gsx[q] = sgn * Gs[fq[q]] * Gs[2 * NF + fq[q]];
-          gsy[q] = sgn * Gs[NF + fq[q]] * Gs[2 * NF + fq[q]];
+          R fr[4];
+          CF::get(Gs, fq[q], fr);
+          gsx[q] = sgn * fr[0] * fr[2];
+          gsy[q] = sgn * fr[1] * fr[2];
         }
         R Sk, Sw;
-        kw_sources<R, HX>(Ks, Os, Ws, Us, Vs, hidx, gsx, gsy, Ac, alpha, kc.beta_star, sigma_do, C_lim, Sk, Sw);
-        const R w0 = Os[hidx];
+        kw_sources<R, HX>(Ks, Os, w0[0], Us, Vs, hidx, gsx, gsy, Ac, alpha, kc.beta_star, sigma_do, C_lim, Sk, Sw);
+        const R om = Os[hidx];
         ak += dt * Sk;
         aw += dt * Sw;
-        rate_k = kc.beta_star * w0;
-        rate_w = beta0 * w0;
+        rate_k = kc.beta_star * om;
+        rate_w = beta0 * om;
       }
       ak /= R(1) + dt * rate_k;
       aw /= R(1) + dt * rate_w;
@@ -707,7 +751,11 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
     const int fl[4] = {fa, fa + 1, fc, fc + X};
     R r = R(0);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) r += (g_abs(u * Gs[fl[q]] + vv * Gs[NF + fl[q]]) + cs) * Gs[2 * NF + fl[q]];
+    for (int q = 0; q < 4; ++q) {
+      R fr[4];
+      CF::get(Gs, fl[q], fr);
+      r += (g_abs(u * fr[0] + vv * fr[1]) + cs) * fr[2];
+    }
     rmax = fmax(rmax, R(0.5) * r * ia);
   }
   const unsigned long long bmax = block_max_rate<R>(rmax, red);
