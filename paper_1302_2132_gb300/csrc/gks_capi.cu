@@ -454,8 +454,10 @@ gks_status sticky_status(gks_handle* h) {
 
 // Tile-shape autotuner: each candidate shape runs the step that is about to be taken from the current
 // state (the results are identical, and the step is then taken for real) five times, round robin
-// over the shapes, each launch timed with CUDA events; the shape with the fastest launch is kept for
-// the handle and for later handles of the same grid.
+// over the shapes, each trial timed with CUDA events; the shape with the fastest trial is kept for
+// the handle and for later handles of the same grid.  A trial is one launch, or on a grid of up to 2^18 cells four
+// launches one after another, as steps are: a launch of 10 to 30 us alone is mostly latency that the next one hides,
+// and picked the second-best shape of a 528 x 136 body-fitted grid (1450 for 1270 us per 96 steps) in one process of six.
 struct TuneKey {
   int n0, n1, multid;
   bool operator<(const TuneKey& o) const {
@@ -518,12 +520,13 @@ gks_status autotune(gks_handle* h) {
   const StepArgs A = step_args(h, h->step);
   std::vector<float> fastest(cand.size(), 1e30f);
   for (int v : cand) launch_step_variant(h, A, v);  // warm-up
-  // round robin, each launch timed alone, the fastest launch of each shape kept: a clock that is
+  // round robin, each trial timed alone, the fastest trial of each shape kept: a clock that is
   // still ramping up penalises no shape in particular
+  const int burst = (long)h->n[0] * h->n[1] * h->n[2] <= (1l << 18) ? 4 : 1;
   for (int r = 0; r < 5; ++r)
     for (size_t k = 0; k < cand.size(); ++k) {
       GKS_CK(h, cudaEventRecord(e0, h->stream));
-      launch_step_variant(h, A, cand[k]);
+      for (int q = 0; q < burst; ++q) launch_step_variant(h, A, cand[k]);
       GKS_CK(h, cudaEventRecord(e1, h->stream));
       GKS_CK(h, cudaEventSynchronize(e1));
       float ms = 0.0f;
