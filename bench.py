@@ -631,10 +631,10 @@ def run_ours(args):
                      "moment_table_ops_per_face": table_ops,
                      "peak_basis": "152 SMs x %d %s lanes x 2 (FMA) x 2070 MHz (derived)" % (lanes, "FP64" if fp64
                                                                                             else "FP32")},
-        # per bench step: state_in + rate kernels, one step kernel per time step (plus, with k-omega
+        # per bench step: state_in + rate kernels, one step kernel per time step, the residual norms (plus, with k-omega
         # transport, the four field conversions of set_turbulence and, unless it is fused into the
         # body-fitted step, one transport kernel per time step)
-        "gpu_launches": args.steps * (((nsteps if fused_tr else 2 * nsteps) + 2 + 4) if transport else (nsteps + 3)),
+        "gpu_launches": args.steps * (((nsteps if fused_tr else 2 * nsteps) + 3 + 4) if transport else (nsteps + 4)),
         "clocks": clock_info,
         "e2e": e2e,
         "final_time": t_end,

@@ -10,11 +10,11 @@
 // 1/(2 lambda) = p/rho and the gradients (r = rho'/rho, U', theta') of the macroscopic variables.  The time slope A is
 // then the Euler equations' time derivative, the full-line moments are the Navier-Stokes fluxes of those
 // gradients, and the transverse velocities average out of a half-line moment before it is taken: what
-// is left on a half line are one cubic and one quadratic polynomial in the normal velocity.  889
-// operations per 2D multi-dimensional face and 1192 in 3D (moment tables: 1674 and 2767).  The kernels are bound
+// is left on a half line are one cubic and one quadratic polynomial in the normal velocity.  890
+// operations per 2D multi-dimensional face and 1193 in 3D (moment tables: 1674 and 2767).  The kernels are bound
 // by their instruction count, in single precision (issue and FP32 pipe about 58% busy) and in double (FP64 pipe 88%
-// busy), so the step times follow: 1024^2 with the double state 122 -> 98 us, 512^2 in FP64 1.88 -> 1.33 ms, 160^3
-// 1.59 -> 1.11 ms.
+// busy), so the step times followed: 1024^2 with the double state 122 -> 98 us, 512^2 in FP64 1.88 -> 1.33 ms, 160^3
+// 1.59 -> 1.11 ms (85 us, 1.13 ms and 0.88 ms with the changes noted where they stand).
 #pragma once
 #ifndef GKS_HOST_COUNT
 #include <cuda_runtime.h>
