@@ -207,7 +207,6 @@ GKS_FN F2 g_erfc(F2 x) {
   const F2 r = F2(t * g_exp(p - z * z));
   return F2(x.v.x >= 0.0f ? r.v.x : 2.0f - r.v.x, x.v.y >= 0.0f ? r.v.y : 2.0f - r.v.y);
 }
-GKS_FN F2 f2_select(bool cx, bool cy, F2 a, F2 b) { return F2(cx ? a.v.x : b.v.x, cy ? a.v.y : b.v.y); }
 // a pending product as the argument: rounded first (exact overloads, so the templates above are not
 // deduced with the product type)
 GKS_FN F2 g_rcp(F2Mul x) { return g_rcp(F2(x)); }
@@ -393,19 +392,6 @@ GKS_FN void weno5_sides(R a, R b, R c, R d, R e, R f, R& wl, R& wr) {
     wl = weno5<R>(a, b, c, d, e);
     wr = weno5<R>(f, e, d, c, b);
   }
-}
-
-// MUSCL on one variable at the face between cells 1 and 2 of the stencil s0..s3 with widths
-// h0..h3: limited slopes of cells 1 and 2 and the face values left and right.
-template <class R>
-GKS_FN void muscl(int lim, R s0, R s1, R s2, R s3, R h0, R h1, R h2, R h3, R& wl, R& wr, R& sl, R& sr) {
-  const R dm = g_div(s1 - s0, R(0.5) * (h0 + h1));
-  const R dc = g_div(s2 - s1, R(0.5) * (h1 + h2));
-  const R dp = g_div(s3 - s2, R(0.5) * (h2 + h3));
-  sl = limiter<R>(lim, dm, dc);
-  sr = limiter<R>(lim, dc, dp);
-  wl = s1 + R(0.5) * h1 * sl;
-  wr = s2 - R(0.5) * h2 * sr;
 }
 
 // Time integrals over [0, dt] of Eq. resultingf, e = exp(-t/tau):
