@@ -249,11 +249,9 @@ def make_workload(name, precision):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the step kernel, taken from
 # one ncu capture of the same kernel build, keyed by workload and tile variant; a combination that
 # was not captured (or whose kernel changed since) reports null.
-# The shock / boundary-layer kernels were captured before the flux's last two changes, so that workload
-# reports null.
-TRAFFIC_PER_LAUNCH = {("turb2d_1024_keps_multid_fp32_acc64", 3): 43.06e6,
+TRAFFIC_PER_LAUNCH = {("turb2d_1024_keps_multid_fp32_acc64", 3): 44.82e6,
                       # 160^3 capture of the same kernel scaled by cells (x 4.096): the state streams at both sizes
-                      ("turb3d_256_fp32_acc64", 2): 1.3804e9}
+                      ("turb3d_256_fp32_acc64", 2): 1.3762e9}
 
 
 def faces_of(n, bc=None):
