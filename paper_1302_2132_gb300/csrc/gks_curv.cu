@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(KwTile::T) steady_komega_kernel(const __grid_c
       const R phiL = v[1] + sa * dl, phiR = v[2] - sb * dr;
       gq[e] = m * (m >= R(0) ? phiL : phiR);
       if (K.diffusion) {
-        const R mdl = g_div(rl * vk[1], vw[1]), mdr = g_div(rr * vk[2], vw[2]);
+        const R mdl = g_div_full(rl * vk[1], vw[1]), mdr = g_div_full(rr * vk[2], vw[2]);
         cond[e] = (kc.mu + (e == 0 ? sigk : sigw) * R(0.5) * (mdl + mdr)) * L * i12;
         gq[e] -= cond[e] * (v[2] - v[1]);
       }

@@ -109,7 +109,7 @@ __device__ __forceinline__ void kw_face(const R* vk, const R* vw, R rl, R rr, co
     const R phiR = v[2] - s1 * (dr + R(0.5) * g_div(fr, rr * L));
     R gq = fr * (fr >= R(0) ? phiL : phiR);
     if (diffusion) {
-      const R mdl = g_div(rl * vk[1], vw[1]), mdr = g_div(rr * vk[2], vw[2]);
+      const R mdl = g_div_full(rl * vk[1], vw[1]), mdr = g_div_full(rr * vk[2], vw[2]);
       const R coef = mu + (q == 0 ? sigk : sigw) * R(0.5) * (mdl + mdr);
       gq -= dt * coef * (v[2] - v[1]) * i12 * L;
     }

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(256) komega_kernel(const __grid_constant__ KOm
       ssl[(0 * D + a) * G::NR + r] = limiter<R>(g.limiter, (sk[h] - sk[h - st]) * im, (sk[h + st] - sk[h]) * ip);
       ssl[(1 * D + a) * G::NR + r] = limiter<R>(g.limiter, (sw[h] - sw[h - st]) * im, (sw[h + st] - sw[h]) * ip);
     }
-    smd[r] = g_div(sr[h] * sk[h], sw[h]);
+    smd[r] = g_div_full(sr[h] * sk[h], sw[h]);
   }
   __syncthreads();
 
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(256) komega_kernel(const __grid_constant__ KOm
     const R bstar = c_bstar;
     const R lim = c_clim * g_sqrt(g_div(R(2) * SbSb, bstar));
     const R wt = om > lim ? om : lim;
-    const R muT = g_div(rho * kk, wt);
+    const R muT = g_div_full(rho * kk, wt);
     const R Pk = muT * X - g_div(R(2), R(3)) * rho * kk * div;
     R chi = R(0);
     if (D == 3) {
@@ -273,8 +273,14 @@ __global__ void __launch_bounds__(256) komega_kernel(const __grid_constant__ KOm
         for (int b = 0; b < 3; ++b)
 #pragma unroll
           for (int e = 0; e < 3; ++e) t += Om[a][b] * Om[b][e] * (Sm[e][a] - (e == a ? R(0.5) * div : R(0)));
+      // (beta* omega)^3 leaves single precision's normal range below omega = 2.5e-12, and the default floor is
+      // 1e-12: the cube is formed of the scaled factor (powers of two, exact), and a chi too large to be
+      // represented takes the limit of f_beta
       const R bo = bstar * om;
-      chi = g_abs(g_div(t, bo * bo * bo));
+      const R up = bo < R(2.3283064365386963e-10) ? R(1099511627776.0) : R(1);  // 2^-32, 2^40
+      const R b = up * bo;
+      chi = g_abs(g_div_full(t, b * b * b)) * (up * up * up);
+      chi = chi < R(1e30) ? chi : R(1e30);
     }
     const R fbeta = g_div(R(1) + R(85) * chi, R(1) + R(100) * chi);
     const R beta = c_beta0 * fbeta;
@@ -282,10 +288,10 @@ __global__ void __launch_bounds__(256) komega_kernel(const __grid_constant__ KOm
 #pragma unroll
     for (int a = 0; a < D; ++a) dkdw += gk[a] * gw[a];
     const R sd = dkdw > R(0) ? c_sdo : R(0);
-    const R CD = g_div(sd * rho, om) * dkdw;
+    const R CD = g_div_full(sd * rho, om) * dkdw;
     const R alpha = c_alpha;
     ak += dt * Pk;
-    aw += dt * (alpha * rho * g_div(om, wt) * X - g_div(R(2), R(3)) * alpha * rho * om * div + CD);
+    aw += dt * (alpha * rho * g_div_full(om, wt) * X - g_div(R(2), R(3)) * alpha * rho * om * div + CD);
     rate_k = bstar * om;
     rate_w = beta * om;
   }
