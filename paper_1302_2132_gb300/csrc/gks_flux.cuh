@@ -92,9 +92,12 @@ template <> GKS_FN double g_fma_rn<double>(double a, double b, double c) { retur
 template <class T> GKS_FN T g_div(T a, T b) { return a / b; }
 template <class T> GKS_FN T g_rcp(T x) { return T(1) / x; }
 template <class T> GKS_FN T g_div_full(T a, T b) { return a / b; }
-// a density as a divisor: at least the smallest normal number
+// a density as a divisor: at least the smallest normal number (the host's quotients take any).  On the device
+// each arithmetic type has its own, so that none goes without.
+#ifdef GKS_HOST_COUNT
 template <class T> GKS_FN T g_normal(T x) { return x; }
-#ifndef GKS_HOST_COUNT
+#else
+template <class T> GKS_FN T g_normal(T x);
 template <> GKS_FN float g_rcp<float>(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -103,6 +106,8 @@ template <> GKS_FN float g_rcp<float>(float x) {
 template <> GKS_FN float g_div<float>(float a, float b) { return a * g_rcp<float>(b); }
 template <> GKS_FN float g_div_full<float>(float a, float b) { return __fdividef(a, b); }
 template <> GKS_FN float g_normal<float>(float x) { return fmaxf(x, 1.17549435e-38f); }
+template <> GKS_FN double g_normal<double>(double x) { return fmax(x, 2.2250738585072014e-308); }
+template <> GKS_FN F2 g_normal<F2>(F2 x) { return F2(g_normal<float>(x.v.x), g_normal<float>(x.v.y)); }
 template <> GKS_FN float g_exp<float>(float x) { return __expf(x); }
 // Double reciprocal and reciprocal square root of normal positive numbers (densities, temperatures, widths,
 // sums of them): the hardware's approximation and one third-order step, r (1 + e + e^2) with e = 1 - x r, and
