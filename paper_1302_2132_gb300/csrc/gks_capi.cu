@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -198,33 +199,30 @@ bool fused_transport(const gks_handle* h) {
   return h->curv && h->transport && h->recon == GKS_RECON_MUSCL2 && h->prec != PREC_F32D && !h->base.g.rar;
 }
 
-void launch_step_variant(gks_handle* h, const StepArgs& A, int variant) {
+// False if there is no kernel of this kind and shape (nothing is launched then).
+bool launch_step_variant(gks_handle* h, const StepArgs& A, int variant) {
   if (h->base.g.rar) {  // the rarefaction option: one tile shape per grid kind
     if (h->curv)
       launch_curv_step_rar(h->prec, A, h->cg, h->multid, h->stream);
     else
       launch_step_rar(h->D, h->prec, h->multid, A, tiles_for(h, 0), h->stream);
-    return;
+    return true;
   }
   if (fused_transport(h)) {
     launch_curv_step_transport(h->prec, A, h->cg, variant, h->multid, h->stream);
-    return;
+    return true;
   }
   if (h->curv) {
     if (h->recon != GKS_RECON_MUSCL2)
       launch_curv_step_recon(h->prec, h->recon, A, h->cg, variant, h->multid, h->stream);
     else
       launch_curv_step(h->prec, A, h->cg, variant, h->multid, h->stream);
-    return;
+    return true;
   }
-  if (h->recon == GKS_RECON_MUSCL3) {
-    launch_step_muscl3(h->D, h->prec, h->multid, variant, A, tiles_for(h, variant), h->stream);
-    return;
-  }
-  if (h->recon == GKS_RECON_WENO5) {
-    launch_step_weno5(h->D, h->prec, h->multid, variant, A, tiles_for(h, variant), h->stream);
-    return;
-  }
+  if (h->recon == GKS_RECON_MUSCL3)
+    return launch_step_muscl3(h->D, h->prec, h->multid, variant, A, tiles_for(h, variant), h->stream);
+  if (h->recon == GKS_RECON_WENO5)
+    return launch_step_weno5(h->D, h->prec, h->multid, variant, A, tiles_for(h, variant), h->stream);
   if ((h->D == 1 && variant == 3) || (h->D == 2 && variant == kSmallTile2D))
     launch_step_small(h->D, h->prec, h->multid, A, tiles_for(h, variant), h->stream);
   else if (h->D == 1 && variant > 0)
@@ -241,13 +239,14 @@ void launch_step_variant(gks_handle* h, const StepArgs& A, int variant) {
     launch_step_d2(h->prec, h->multid, A, tiles_for(h, 0), h->stream);
   else
     launch_step_d3(h->prec, h->multid, A, h->nblocks, h->stream);
+  return true;
 }
 
 // One full step: the flow step and, with k-omega transport, the transport step of rho k and
 // rho omega (into the other buffer pair) with the same dt and the flow step's mass fluxes.
-void launch_step(gks_handle* h, const StepArgs& A) {
-  launch_step_variant(h, A, h->tile_variant);
-  if (!h->transport || fused_transport(h)) return;
+bool launch_step(gks_handle* h, const StepArgs& A) {
+  if (!launch_step_variant(h, A, h->tile_variant)) return false;
+  if (!h->transport || fused_transport(h)) return true;
   const int cur = A.Win == h->W[0] ? 0 : 1;
   KOmegaArgs K;
   std::memset(&K, 0, sizeof(K));
@@ -282,6 +281,7 @@ void launch_step(gks_handle* h, const StepArgs& A) {
     launch_curv_komega(h->prec, K, h->cg, h->stream);
   else
     launch_komega(h->D, h->prec, K, h->stream);
+  return true;
 }
 
 // Arguments of the step that starts at absolute step index s.
@@ -458,12 +458,9 @@ gks_status sticky_status(gks_handle* h) {
 // the handle and for later handles of the same grid.  A trial is one launch, or on a grid of up to 2^18 cells four
 // launches one after another, as steps are: a launch of 10 to 30 us alone is mostly latency that the next one hides,
 // and picked the second-best shape of a 528 x 136 body-fitted grid (1450 for 1270 us per 96 steps) in one process of six.
-struct TuneKey {
-  int n0, n1, multid;
-  bool operator<(const TuneKey& o) const {
-    return n0 != o.n0 ? n0 < o.n0 : (n1 != o.n1 ? n1 < o.n1 : multid < o.multid);
-  }
-};
+// The key is everything that decides which shapes are candidates, and the grid: arithmetic, expansion, reconstruction
+// and kind of grid (0 rectilinear, 1 body-fitted, 2 with fused transport).  A shape found under it is a candidate.
+using TuneKey = std::array<int, 8>;  // D, n0, n1, n2, arithmetic, multid, recon, kind
 std::map<TuneKey, int> g_tuned;
 std::mutex g_tuned_mutex;
 
@@ -504,8 +501,8 @@ gks_status autotune(gks_handle* h) {
       if (c == v) h->tile_variant = v;
     return GKS_OK;
   }
-  const TuneKey key{h->n[0] + 100000 * h->prec, h->n[1] * 4 + h->D,
-                    h->curv ? 2 + 4 * h->recon + 16 * (int)fused_transport(h) : (int)h->multid};
+  const TuneKey key{h->D,    h->n[0],           h->n[1],  h->n[2],
+                    h->prec, (int)h->multid, h->recon, (int)h->curv + (int)fused_transport(h)};
   {
     std::lock_guard<std::mutex> lk(g_tuned_mutex);
     auto it = g_tuned.find(key);
@@ -519,7 +516,8 @@ gks_status autotune(gks_handle* h) {
   GKS_CK(h, cudaEventCreate(&e1));
   const StepArgs A = step_args(h, h->step);
   std::vector<float> fastest(cand.size(), 1e30f);
-  for (int v : cand) launch_step_variant(h, A, v);  // warm-up
+  for (int v : cand)  // warm-up
+    if (!launch_step_variant(h, A, v)) return fail(h, GKS_EUNSUPPORTED, "no step kernel of this shape");
   // round robin, each trial timed alone, the fastest trial of each shape kept: a clock that is
   // still ramping up penalises no shape in particular
   const int burst = (long)h->n[0] * h->n[1] * h->n[2] <= (1l << 18) ? 4 : 1;
@@ -1027,9 +1025,14 @@ gks_status gks_step(gks_handle* h, double dt, double cfl, int nsteps, double t_e
       if (it == h->graphs.end()) {
         cudaGraph_t graph;
         GKS_CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        for (int k = 0; k < kGraphChunk; ++k) launch_step(h, step_args(h, k));
+        bool launched = true;
+        for (int k = 0; k < kGraphChunk; ++k) launched = launched && launch_step(h, step_args(h, k));
         cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
         if (e != cudaSuccess) return cuda_fail(h, e, "graph capture");
+        if (!launched) {
+          cudaGraphDestroy(graph);
+          return fail(h, GKS_EUNSUPPORTED, "no step kernel of this shape");
+        }
         cudaGraphExec_t exec;
         e = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
@@ -1042,6 +1045,7 @@ gks_status gks_step(gks_handle* h, double dt, double cfl, int nsteps, double t_e
       continue;
     }
     const StepArgs A = step_args(h, h->step);
+    bool launched = true;
     if (h->timing) {
       cudaEvent_t e0, e1;
       GKS_CK(h, cudaEventCreate(&e0));
@@ -1049,11 +1053,12 @@ gks_status gks_step(gks_handle* h, double dt, double cfl, int nsteps, double t_e
       h->ev.push_back(e0);
       h->ev.push_back(e1);
       GKS_CK(h, cudaEventRecord(e0, h->stream));
-      launch_step(h, A);
+      launched = launch_step(h, A);
       GKS_CK(h, cudaEventRecord(e1, h->stream));
     } else {
-      launch_step(h, A);
+      launched = launch_step(h, A);
     }
+    if (!launched) return fail(h, GKS_EUNSUPPORTED, "no step kernel of this shape");
     GKS_CK(h, cudaGetLastError());
     if (remaining == 1) {  // residual norms of the call's last step
       launch_residual(h, A);

@@ -28,6 +28,7 @@ bool launch_step_weno5(int D, int prec, bool multid, int variant, const StepArgs
     launch_step<2, PREC_F32, true, 3, RECON_WENO5>(A, nblocks, s);
     return true;
   }
+  if (variant != 0) return false;
   const bool f64 = prec == PREC_F64;
   if (D == 1) {
     if (f64) launch_step<1, PREC_F64, false, 0, RECON_WENO5>(A, nblocks, s);
