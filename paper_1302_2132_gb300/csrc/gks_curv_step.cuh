@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(CurvTile<V>::T, PREC == PREC_F64 ? 1 : 512 / C
       const long gidx = (long)v * g.ncell + c;
       if (PREC == PREC_F64) {
         const double w_old = (double)w0[v];
-        const double w = w_old - (double)net * (double)ia;
+        const double w = w_old - g_quot_r<double>((double)net, G.area[c], (double)ia);
         ((double*)A.Wout)[gidx] = w;
         wn[v] = (R)w;
       } else {

@@ -147,13 +147,25 @@ GKS_FN float erfc_cheb(float x) {
 template <> GKS_FN float g_erfc<float>(float x) { return erfc_cheb(x); }
 #endif
 
-// quotient of normal numbers whose quotient is normal
-template <class T> GKS_FN T g_quot(T a, T b) {
+// a / b from r, the reciprocal of b, for normal numbers whose quotient is normal.  In double the product is corrected by
+// its exact remainder (Markstein's last step, which rounds as a division does); in single precision the product, as g_div.
+template <class T> GKS_FN T g_quot_r(T a, T b, T r) {
+  const T q = g_mul_rn<T>(a, r);
   if constexpr (std::is_same<T, double>::value)
-    return a * g_rcp<T>(b);
+    return g_fma_rn<T>(g_fma_rn<T>(-q, b, a), r, q);
   else
-    return g_div(a, b);
+    return q;
 }
+template <class T> GKS_FN T g_quot(T a, T b) { return g_div(a, b); }
+#ifndef GKS_HOST_COUNT
+// (a reciprocal to 2^-40, by Newton's step, leaves the corrected quotient within 2^-28 units of the rounded one)
+template <> GKS_FN double g_quot<double>(double a, double b) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+  r = __fma_rn(r, __fma_rn(-b, r, 1.0), r);
+  return g_quot_r<double>(a, b, r);
+}
+#endif
 
 // erfc(x) and exp(-x^2) together.
 template <class T> GKS_FN void g_gauss(T x, T& c, T& e) {

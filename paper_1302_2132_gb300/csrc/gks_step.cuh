@@ -641,7 +641,7 @@ __device__ __forceinline__ R cell_rate_inv(const R* w, R gamma, const R* ih) {
   R q = g_mul_rn<R>(w[1], w[1]);
 #pragma unroll
   for (int d = 1; d < D; ++d) q = g_fma_rn<R>(w[1 + d], w[1 + d], q);
-  const R p = g_mul_rn<R>(gamma - R(1), g_fma_rn<R>(R(-0.5), g_mul_rn<R>(q, ir), w[D + 1]));
+  const R p = g_mul_rn<R>(gamma - R(1), g_fma_rn<R>(R(-0.5), g_quot_r<R>(q, w[0], ir), w[D + 1]));
   const R cs = g_sqrt(g_mul_rn<R>(g_mul_rn<R>(gamma, p), ir));
   R r = R(0);
 #pragma unroll
@@ -1434,6 +1434,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
     R ih[3];
 #pragma unroll
     for (int d = 0; d < D; ++d) ih[d] = (d == 0 ? iwx[li + H] : (d == 1 ? iwy[lj + H] : iwz[lk + H]));
+    [[maybe_unused]] const R h[3] = {wsx[li + H], D >= 2 ? wsy[lj + H] : R(1), D >= 3 ? wsz[lk + H] : R(1)};
     R wn[nv];
     [[maybe_unused]] R dF[CF::AOS ? D : 1][nv], w0[nv];  // flux differences and the staged state, read whole
     if constexpr (CF::AOS) {
@@ -1455,7 +1456,8 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       if constexpr (PREC == PREC_F64) {
         double w = (double)w0[v];
 #pragma unroll
-        for (int d = 0; d < D; ++d) w -= ((double)Fs[v * G::NF + fp[d]] - (double)Fs[v * G::NF + fm[d]]) * (double)ih[d];
+        for (int d = 0; d < D; ++d)
+          w -= g_quot_r<double>((double)Fs[v * G::NF + fp[d]] - (double)Fs[v * G::NF + fm[d]], (double)h[d], (double)ih[d]);
         ((double*)A.Wout)[gidx] = w;
         wn[v] = (R)w;
       } else {

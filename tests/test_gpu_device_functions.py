@@ -1,0 +1,55 @@
+"""The library's double-precision building blocks on the device, against the correctly rounded or extended-precision
+values on the host."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1302_2132_gb300", "csrc")
+SO = os.path.join(HERE, "_build", "libdevice_functions.so")
+
+
+@pytest.fixture(scope="module")
+def lib():
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    src = os.path.join(HERE, "device_functions.cu")
+    deps = [src] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
+    os.makedirs(os.path.dirname(SO), exist_ok=True)
+    if not os.path.exists(SO) or os.path.getmtime(SO) < max(os.path.getmtime(f) for f in deps):
+        subprocess.check_call([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-O3",
+                               "-Xcompiler", "-fPIC", "-shared", "-I", CSRC, "-I",
+                               os.path.join(os.path.dirname(os.path.dirname(CSRC)), "include"), "-o", SO + ".tmp", src])
+        os.replace(SO + ".tmp", SO)
+    return ctypes.CDLL(SO)
+
+
+def apply(f, outputs, *args):
+    """f(n, args..., outputs...) on device copies; args of n rows each."""
+    n = len(args[0])
+    dev = [torch.tensor(np.ascontiguousarray(a), device="cuda") for a in args]
+    out = [torch.empty(n, dtype=t, device="cuda") for t in outputs]
+    torch.cuda.synchronize()
+    assert f(ctypes.c_long(n), *(ctypes.c_void_p(t.data_ptr()) for t in dev + out)) == 0
+    return [t.cpu().numpy() for t in out]
+
+
+def test_quotients_round_as_the_division_does(lib):
+    rng = np.random.default_rng(4)
+    n = 1 << 21
+    a, b = (rng.uniform(1, 2, n) * 2.0 ** rng.integers(-40, 40, n) for _ in range(2))
+    a *= rng.choice([-1.0, 1.0], n)
+    b[:1000] = np.nextafter(2.0 ** rng.integers(-40, 40, 1000), 0)  # all ones in the significand
+    (q,) = apply(lib.dev_quotient, [torch.float64], a, b)
+    assert np.array_equal(q, a / b)
