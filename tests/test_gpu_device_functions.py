@@ -53,3 +53,16 @@ def test_quotients_round_as_the_division_does(lib):
     b[:1000] = np.nextafter(2.0 ** rng.integers(-40, 40, 1000), 0)  # all ones in the significand
     (q,) = apply(lib.dev_quotient, [torch.float64], a, b)
     assert np.array_equal(q, a / b)
+
+
+def test_double_states_near_zero_pressure(lib):
+    """Physical if and only if the pressure that the oracle evaluates is positive: energies within two units in the
+    last place of the kinetic energy."""
+    rng = np.random.default_rng(8)
+    n = 1 << 18
+    rho, mu = rng.uniform(0.1, 4.0, n), rng.uniform(1.0, 50.0, n)
+    kin = mu * mu / rho  # rounded as the oracle rounds it
+    E = 0.5 * kin * (1 + rng.integers(-2, 3, n) * 2.0 ** -52)
+    w = np.stack([rho, mu, np.zeros(n), E], 1)
+    (ok,) = apply(lib.dev_physical, [torch.int32], w)
+    assert np.array_equal(ok != 0, E > 0.5 * kin)
