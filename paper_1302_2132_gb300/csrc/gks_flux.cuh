@@ -174,33 +174,35 @@ template <class T> GKS_FN void g_gauss(T x, T& c, T& e) {
 }
 #ifndef GKS_HOST_COUNT
 // In double one exponential serves both: for a = |x| >= 0, erfc(a) = exp(-a^2) w(a), and (1 + sqrt(pi) a) w(a), which is 1 at
-// both ends, is a polynomial of degree 24 in t = (a - 3)/(a + 3) to 5e-17: its Chebyshev series on [-1, 1], computed
-// in 40 digits (the mapping of Schonfelder and of Shepherd and Laframboise for this function).  The rounding
-// of a^2 is carried into the exponential to first order.  Relative error of erfc at most 6.4e-16 where it is normal.
-// With it, the reciprocals above and the inverse widths in the update, the FP64 step takes 1.13 ms instead of 1.34 at
-// 512^2 (k-epsilon, multi-dimensional) and 29.7 us instead of 39.0 on the 400-cell shock tube.
+// both ends, is a polynomial of degree 24 in t = (a - 3)/(a + 3) to 1.2e-17: its Chebyshev series on [-1, 1], computed
+// in 60 digits (the mapping of Schonfelder and of Shepherd and Laframboise for this function), its leading coefficient
+// in two parts.  The roundings of a^2, of the polynomial's last step and of the quotient are carried to first order into
+// the last operation, so that of the error little more than the exponential's is left.  With it, the reciprocals above and
+// the inverse widths in the update, the FP64 step takes 1.13 ms instead of 1.34 at 512^2 (k-epsilon, multi-dimensional) and
+// 29.7 us instead of 39.0 on the 400-cell shock tube.
 template <> GKS_FN void g_gauss<double>(double x, double& c, double& e) {
-  const double m[25] = {1.13081499036531518, -0.15730767105387838, -0.0142078862510333066, 0.0978158787627484546, -0.0975498893780881991,
+  const double m0 = 1.130814990365315, m0l = 1.0122955773236472e-16;
+  const double m[24] = {-0.15730767105387838, -0.0142078862510333066, 0.0978158787627484546, -0.0975498893780881991,
                         0.0577612034134763832, -0.0205803575852415208, 0.00232213762002999957, 0.00160587866420396248, -0.00068595951686176365,
                         -0.0000859074652169480687, 0.000109403210195641532, 3.47842163101718717e-6, -0.0000175723862950109043, -5.05198940975773676e-7,
                         3.0437515559732887e-6, 2.88623899544377934e-7, -5.43060517125976003e-7, -1.1920154572965122e-7, 9.02620167290913922e-8,
                         3.54129561773177263e-8, -1.1890984470997693e-8, -7.14018809267724831e-9, 8.88513573014043976e-10, 7.32248898966643554e-10};
   const double a = fabs(x), s = a * a;
   e = exp(-s);
-  const double ec = __fma_rn(-e, __fma_rn(a, a, -s), e);
+  const double sl = __fma_rn(a, a, -s);
   const double d1 = a + 3.0, d2 = __fma_rn(1.7724538509055160273, a, 1.0);
   const double r = g_rcp(d1 * d2);
   const double rt = r * d2;  // 1 / d1
   double t = (a - 3.0) * rt;
   t = __fma_rn(__fma_rn(-t, d1, a - 3.0), rt, t);
-  double p = m[24];
+  double p = m[23];
 #pragma unroll
-  for (int i = 23; i >= 0; --i) p = __fma_rn(p, t, m[i]);
+  for (int i = 22; i >= 0; --i) p = __fma_rn(p, t, m[i]);
+  const double ph = __fma_rn(p, t, m0), pl = __fma_rn(p, t, m0 - ph) + m0l;
   const double rd = r * d1;  // 1 / d2
-  double w = p * rd;
-  w = __fma_rn(__fma_rn(-w, d2, p), rd, w);
+  const double w = ph * rd, wl = (__fma_rn(-w, d2, ph) + pl) * rd;
   // (far out the quotients are infinity times zero: erfc is zero there)
-  const double q = a < 28.0 ? w * ec : 0.0;
+  const double q = a >= 28.0 ? 0.0 : __fma_rn(e, w, e * __fma_rn(-w, sl, wl));
   c = x >= 0.0 ? q : 2.0 - q;
 }
 #endif

@@ -66,3 +66,31 @@ def test_double_states_near_zero_pressure(lib):
     w = np.stack([rho, mu, np.zeros(n), E], 1)
     (ok,) = apply(lib.dev_physical, [torch.int32], w)
     assert np.array_equal(ok != 0, E > 0.5 * kin)
+
+
+def test_reciprocal_square_root(lib):
+    """No further from the exact value than 1 / sqrt(x) by two IEEE operations."""
+    rng = np.random.default_rng(5)
+    x = rng.uniform(1, 4, 1 << 20) * 4.0 ** rng.integers(-30, 30, 1 << 20)
+    (y,) = apply(lib.dev_rsqrt, [torch.float64], x)
+    exact = 1 / np.sqrt(x.astype(np.longdouble))
+    ours, ieee = (np.abs((v - exact) / exact) for v in (y, 1 / np.sqrt(x)))
+    assert ours.max() <= ieee.max() and np.mean(ours ** 2) <= np.mean(ieee ** 2)
+
+
+def test_erfc_and_exponential(lib):
+    """No further from the exact values than CUDA's own functions, in the largest and in the mean error, over the
+    arguments whose erfc is a normal number; zero beyond."""
+    rng = np.random.default_rng(6)
+    x = np.concatenate([rng.uniform(-6, 26.5, 400000), rng.uniform(-3, 3, 400000), 10.0 ** rng.uniform(-12, 0, 50000)])
+    c, e, cc, ce = apply(lib.dev_gauss, [torch.float64] * 4, x)
+    assert np.array_equal(e, ce)
+    hi, lo = np.empty_like(x), np.empty_like(x)
+    ptr = lambda a: ctypes.c_void_p(a.ctypes.data)
+    lib.host_erfc(ctypes.c_long(x.size), ptr(x), ptr(hi), ptr(lo))
+    ours, theirs = (np.abs(((y - hi) - lo) / hi) for y in (c, cc))
+    print("largest %.3g %.3g mean square root %.3g %.3g" % (ours.max(), theirs.max(), np.sqrt(np.mean(ours ** 2)),
+                                                           np.sqrt(np.mean(theirs ** 2))))
+    assert ours.max() <= theirs.max() and np.mean(ours ** 2) <= np.mean(theirs ** 2)
+    c, e, _, _ = apply(lib.dev_gauss, [torch.float64] * 4, np.array([28.0, 40.0, 1e200, np.inf, -28.0, -np.inf, np.nan]))
+    assert np.array_equal(c, [0, 0, 0, 0, 2, 2, np.nan], equal_nan=True) and not e[1:6].any() and np.isnan(e[6])
