@@ -116,8 +116,9 @@ __global__ void __launch_bounds__(kThreads) rate_kernel(const __grid_constant__ 
 
 // Residual norms of the step that took Win to Wout: l2 += (dW/dt)^2, linf = max |dW|/dt, total += W volume (area: per
 // cell, body-fitted grids; null: the product of the widths).  It runs after the last step of a call only, so the
-// step kernels carry none of it.  Doubles run at 1/64 of the FP32 rate on this part and bound it: three double
-// operations per value, dt divided out once per CTA, and a reduction in shared memory in which one warp
+// step kernels carry none of it.  The increment is the difference of the stored states, in double in every
+// precision.  Doubles run at 1/64 of the FP32 rate on this part and bound it: four double operations per value (six of
+// a float pair), dt divided out once per CTA, and a reduction in shared memory in which one warp
 // adds up one quantity (T/32 + 5 additions a lane, against five per quantity in every warp).
 // Accumulated inside the step kernel the norms took 115 us of that step at 1024^2 with the double state, and
 // their code 5% of every other step (the 49-step call 4.82 -> 4.53 ms, 160^3 x 7 steps 7.65 -> 6.67 ms).
@@ -125,19 +126,16 @@ template <int D, int PREC>
 __global__ void __launch_bounds__(kThreads) residual_kernel(const __grid_constant__ StepArgs A, const double* area) {
   using S = typename PrecT<PREC>::S;
   constexpr int NV = D + 2, T = kThreads, NW = T / 32;
-  using M = S;
   __shared__ double sums[2 * NV * T];
-  __shared__ M maxs[NV * T];
+  __shared__ double maxs[NV * T];
   const DevGrid& g = A.g;
   const double dt = A.ctrl->last_dt;
   if (dt == 0.0) return;  // past t_end: the state was carried over
   const int tid = threadIdx.x;
-  double s2[NV], tot[NV];
-  M mx[NV];
+  double s2[NV], tot[NV], mx[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    s2[v] = tot[v] = 0.0;
-    mx[v] = M(0);
+    s2[v] = tot[v] = mx[v] = 0.0;
   }
   const S* W0 = (const S*)A.Win;
   const S* W1 = (const S*)A.Wout;
@@ -154,17 +152,14 @@ __global__ void __launch_bounds__(kThreads) residual_kernel(const __grid_constan
     for (int v = 0; v < NV; ++v) {
       const long i = (long)v * g.ncell + c;
       double w, r;
-      if constexpr (PREC == PREC_F32) {  // float pairs: the difference of the high words is exact up to rounding
-        const float h1 = W1[i], l1 = A.Wout_lo[i];
-        const float d = (h1 - W0[i]) + (l1 - A.Win_lo[i]);
-        w = f2d(h1) + f2d(l1);
-        r = f2d(d);
-        mx[v] = fmaxf(mx[v], fabsf(d));
+      if constexpr (PREC == PREC_F32) {  // a float pair is its sum, exactly
+        w = f2d(W1[i]) + f2d(A.Wout_lo[i]);
+        r = w - (f2d(W0[i]) + f2d(A.Win_lo[i]));
       } else {
         w = W1[i];
         r = w - W0[i];
-        mx[v] = fmax(mx[v], fabs(r));
       }
+      mx[v] = fmax(mx[v], fabs(r));
       s2[v] += r * r;
       tot[v] += w * vol;
     }
@@ -191,12 +186,12 @@ __global__ void __launch_bounds__(kThreads) residual_kernel(const __grid_constan
           atomicAdd(&A.ctrl->total[q - NV], s);
       }
     } else {
-      M m = maxs[(q - 2 * NV) * T + lane];
+      double m = maxs[(q - 2 * NV) * T + lane];
 #pragma unroll
       for (int k = 1; k < NW; ++k) m = fmax(m, maxs[(q - 2 * NV) * T + lane + 32 * k]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) atomic_max_nonneg(&A.ctrl->linf[q - 2 * NV], (double)m / dt);
+      if (lane == 0) atomic_max_nonneg(&A.ctrl->linf[q - 2 * NV], m / dt);
     }
   }
 }
