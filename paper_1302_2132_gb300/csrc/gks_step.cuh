@@ -1399,7 +1399,9 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       }
     }
   }
-  // double state: the old doubles of this thread's cells are loaded while the CTA meets at the barrier
+  // double state: the old doubles of this thread's cells are loaded while the CTA meets at the barrier.  (Coherent loads:
+  // launched as a programmatic dependent this kernel is alive while the previous step writes them, which the
+  // read-only path does not allow and lets the compiler move above the wait.)
   constexpr int NCI = (G::NC + kThreads - 1) / kThreads;
   double wold[PREC == PREC_F32D ? NCI : 1][nv];
   if constexpr (PREC == PREC_F32D) {
@@ -1411,7 +1413,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
       if (l >= G::NC || gi >= g.n[0] || (D >= 2 && gj >= g.n[1]) || (D >= 3 && gk >= g.n[2])) continue;
       const long c = cell_index(g, gi, gj, gk);
 #pragma unroll
-      for (int v = 0; v < nv; ++v) wold[q][v] = __ldg((const double*)A.Win + (long)v * g.ncell + c);
+      for (int v = 0; v < nv; ++v) wold[q][v] = ((const double*)A.Win)[(long)v * g.ncell + c];
     }
   }
   __syncthreads();
