@@ -77,12 +77,14 @@ __global__ void __launch_bounds__(kFaceT) face_kernel(int abar_t0, Gas<double> g
   to_arith(gas_d.K, gas.K);
   to_arith(gas_d.mu, gas.mu);
   to_arith(gas_d.C_a, gas.C_a);
+  // the distances are the caller's: infinity stands for a side without a gradient, and its reciprocal is zero
+  const R idxl = g_div_full(R(1), dxl), idxr = g_div_full(R(1), dxr);
   // the same flux code as the step kernels: in single precision the two sides
   // of the face on the paired FP32 instructions
   if constexpr (std::is_same<R, float>::value)
-    face_flux_ps<D, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, dxl, dxr, tau_t, dtr, gas, abar_t0, F, &tau);
+    face_flux_ps_inv<D, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, idxl, idxr, tau_t, dtr, gas, abar_t0, F, &tau);
   else
-    face_flux<D, R, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, dxl, dxr, tau_t, dtr, gas, abar_t0, F, &tau);
+    face_flux_inv<D, R, MULTID, RAR>(wl, wr, cl, cr, sl, sr, tl, tr, idxl, idxr, tau_t, dtr, gas, abar_t0, F, &tau);
   if (tid < nf) {
 #pragma unroll
     for (int v = 0; v < nv; ++v) rec[tid * nv + v] = (double)F[v];

@@ -460,7 +460,7 @@ GKS_FN void phi_series(T x, T& p1, T& p2, T& p3, T& e) {
 template <class T>
 GKS_FN void time_coeffs(T dt, T tau, TimeCoef<T>& c) {
   const T x = g_div(dt, tau);
-  const T y = tau * g_rcp(dt);
+  const T y = tau * g_rcp(g_normal(dt));
   if (x < T(1)) {
     // series branch (phi_k summed, no cancellation) in the arithmetic type
     T p1, p2, p3, e;
