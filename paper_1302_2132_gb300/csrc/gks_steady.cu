@@ -382,7 +382,7 @@ size_t rbytes(int prec) { return prec == PREC_F64 ? 8 : 4; }
 
 void free_level(SteadyLevel& l) {
   void* ps[] = {l.nodes, l.W, l.W0, l.R, l.P, l.s, l.hl[0], l.hl[1], l.f1, l.f2, l.G.face[0], l.G.face[1],
-                l.G.iarea, l.G.area, l.G.tau, l.G.flux[0], l.G.flux[1], l.G.tang[0], l.G.tang[1], l.dir[0][0],
+                l.G.iarea, l.G.area, l.G.flux[0], l.G.flux[1], l.G.tang[0], l.G.tang[1], l.dir[0][0],
                 l.dir[0][1], l.dir[1][0],
                 l.dir[1][1]};
   for (void* p : ps)
@@ -702,7 +702,6 @@ gks_status gks_steady_create(const gks_grid* grid, const gks_gas* gas, const gks
     }
     alloc(&G.iarea, rb * lev.ncell);
     alloc((void**)&G.area, sizeof(double) * lev.ncell);
-    alloc(&G.tau, rb * lev.ncell);
     alloc(&lev.W, rb * 4 * lev.ncell);
     alloc(&lev.W0, rb * 4 * lev.ncell);
     alloc(&lev.R, rb * 4 * lev.ncell);
