@@ -320,11 +320,11 @@ void launch_group(gks_server* s, int g, int phase, cudaStream_t st) {
     launch_batch_d2(s->prec, s->var[g], g == GROUP_2D_MULTID, B, s->blocks[g], st);
 }
 
-// The steps of a chunk: the groups share no solve and each counts its own steps, so their launches are
+// Steps of all groups (a multiple of six: the phases start over): the groups share no solve and each counts its own steps, so their launches are
 // branches of the graph that run side by side (a small group's launch leaves most of the chip idle, and an
 // empty one costs its launch latency).  A burst of
 // 16 solves (8 in 1D, 8 in 2D up to 256^2, 40 to 120 steps) 5.66 -> 4.56 ms against one stream for all.
-bool capture_chunk(gks_server* s) {
+bool capture_steps(gks_server* s, int steps, cudaGraphExec_t* exec) {
   cudaEvent_t ev[NGROUPS] = {nullptr, nullptr, nullptr};
   cudaStream_t side[NGROUPS] = {s->stream, nullptr, nullptr};
   bool ok = true;
@@ -336,13 +336,13 @@ bool capture_chunk(gks_server* s) {
     ok = cudaEventRecord(ev[0], s->stream) == cudaSuccess;
     for (int g = 1; g < NGROUPS; ++g) ok = ok && cudaStreamWaitEvent(side[g], ev[0], 0) == cudaSuccess;
     for (int g = 0; g < NGROUPS && ok; ++g)
-      for (int k = 0; k < s->chunk; ++k) launch_group(s, g, k % 6, side[g]);
+      for (int k = 0; k < steps; ++k) launch_group(s, g, k % 6, side[g]);
     for (int g = 1; g < NGROUPS; ++g)
       ok = ok && cudaEventRecord(ev[g], side[g]) == cudaSuccess &&
            cudaStreamWaitEvent(s->stream, ev[g], 0) == cudaSuccess;
     cudaGraph_t graph = nullptr;
     ok = cudaStreamEndCapture(s->stream, &graph) == cudaSuccess && ok;
-    ok = ok && cudaGraphInstantiate(&s->graph, graph, 0) == cudaSuccess;
+    ok = ok && cudaGraphInstantiate(exec, graph, 0) == cudaSuccess;
     if (graph) cudaGraphDestroy(graph);
   } else {
     ok = false;
@@ -355,7 +355,7 @@ bool capture_chunk(gks_server* s) {
 }
 
 bool run_chunk(gks_server* s) {
-  if (!s->graph && !capture_chunk(s)) return false;
+  if (!s->graph && !capture_steps(s, s->chunk, &s->graph)) return false;
   if (cudaGraphLaunch(s->graph, s->stream) != cudaSuccess) return false;
   return cudaStreamSynchronize(s->stream) == cudaSuccess;
 }
@@ -437,8 +437,12 @@ void worker_main(gks_server* s) {
 
 // Tile shape of each group, timed once per process and device on a synthetic batch (every server of
 // the process then uses the same shapes, so a solve's result does not depend on which server or mix
-// it runs in): for each group, a batch of periodic solves of typical sizes is admitted and each
-// candidate shape runs three rounds of six batch steps (CUDA events); the fastest round decides.
+// it runs in): a batch of periodic solves of typical sizes is admitted to every group, and group by group each
+// candidate shape runs three rounds of six batch steps of all groups side by side, as a chunk runs them (CUDA
+// events).  The fastest round decides; a shape later in the list has to be faster by 2%, since a group that is not the
+// longest branch says little.  (Timed alone on the chip, two shapes of a 2D group took turns from one
+// process to the next, and with one of them a burst of 400 solves ran at 842 to 856 solves/s, with the other at 905 to 929.
+// This way six processes of six found the first shapes, 902 to 923.)
 // GKS_BATCH_TILES="v1d,v2d,v2d_multid" forces the shapes.
 std::mutex g_tune_mu;
 std::map<int, std::vector<int>> g_tuned_batch;
@@ -524,47 +528,56 @@ bool tune_batch(gks_server* s, const int* res1, const int* res2, int sms) {
         ++admitted[e ? GROUP_2D_MULTID : GROUP_2D];
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   bool ok = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
-  int phase = 0;
-  for (int g = 0; g < NGROUPS && ok; ++g) {
-    if (!admitted[g]) {
-      s->var[g] = cand[g][0];
-      set_blocks(g);
-      continue;
+  auto set_shape = [&](int g, int v) {
+    s->var[g] = v;
+    set_blocks(g);
+    int n = 0;
+    for (Req* r : reqs)
+      if (r->group == g) {
+        r->tiles = tiles_of(r->q, v);
+        for (int t = 0; t < r->tiles; ++t) s->h_items[(size_t)g * s->max_items + n++] = make_int2(r->slot, t);
+      }
+    s->h_nitems[g] = n;
+    cudaMemcpyAsync(s->d_items[g], s->h_items + (size_t)g * s->max_items, sizeof(int2) * n, cudaMemcpyHostToDevice,
+                    s->stream);
+    cudaMemcpyAsync(s->d_nitems, s->h_nitems, sizeof(int) * NGROUPS, cudaMemcpyHostToDevice, s->stream);
+    return cudaStreamSynchronize(s->stream) == cudaSuccess;
+  };
+  // the fastest of three rounds of six steps of all groups, after one to warm up; negative on failure
+  auto fastest_round = [&]() {
+    cudaGraphExec_t exec = nullptr;
+    if (!capture_steps(s, 6, &exec)) return -1.0f;
+    float best = 1e30f;
+    for (int round = 0; round < 4; ++round) {
+      float ms = 0.0f;
+      if (cudaEventRecord(e0, s->stream) != cudaSuccess || cudaGraphLaunch(exec, s->stream) != cudaSuccess ||
+          cudaEventRecord(e1, s->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+          cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+        best = -1.0f;
+        break;
+      }
+      if (round > 0) best = std::min(best, ms);
     }
+    cudaGraphExecDestroy(exec);
+    return best;
+  };
+  for (int g = 0; g < NGROUPS && ok; ++g) ok = set_shape(g, cand[g][0]);
+  for (int g = 0; g < NGROUPS && ok; ++g) {
+    if (!admitted[g]) continue;
     float best = 1e30f;
     int best_v = cand[g][0];
     for (int v : cand[g]) {
-      s->var[g] = v;
-      set_blocks(g);
-      int n = 0;
-      for (Req* r : reqs)
-        if (r->group == g) {
-          r->tiles = tiles_of(r->q, v);
-          for (int t = 0; t < r->tiles; ++t) s->h_items[(size_t)g * s->max_items + n++] = make_int2(r->slot, t);
-        }
-      for (int h = 0; h < NGROUPS; ++h) s->h_nitems[h] = h == g ? n : 0;
-      cudaMemcpyAsync(s->d_items[g], s->h_items + (size_t)g * s->max_items, sizeof(int2) * n, cudaMemcpyHostToDevice,
-                      s->stream);
-      cudaMemcpyAsync(s->d_nitems, s->h_nitems, sizeof(int) * NGROUPS, cudaMemcpyHostToDevice, s->stream);
-      for (int k = 0; k < 3; ++k) launch_group(s, g, phase++ % 6, s->stream);  // warm-up
-      for (int round = 0; round < 3; ++round) {
-        cudaEventRecord(e0, s->stream);
-        for (int k = 0; k < 6; ++k) launch_group(s, g, phase++ % 6, s->stream);
-        cudaEventRecord(e1, s->stream);
-        if (cudaEventSynchronize(e1) != cudaSuccess) {
-          ok = false;
-          break;
-        }
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best) {
-          best = ms;
-          best_v = v;
-        }
+      const float ms = set_shape(g, v) ? fastest_round() : -1.0f;
+      if (ms < 0.0f) {
+        ok = false;
+        break;
+      }
+      if (ms < 0.98f * best) {
+        best = ms;
+        best_v = v;
       }
     }
-    s->var[g] = best_v;
-    set_blocks(g);
+    ok = ok && set_shape(g, best_v);
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
