@@ -620,8 +620,8 @@ cudaError_t curv_metrics(const double* nodes, int n0, int n1, const bool periodi
 
 cudaError_t prepare_curv() {
   cudaError_t e = cudaSuccess;
-  const cudaError_t r[17] = {prepare_one<PREC_F64, 0, 1, false, 0, false, false, true>(),
-                            prepare_one<PREC_F32, 0, 1, false, 0, false, false, true>(),
+  const cudaError_t r[17] = {prepare_one<PREC_F64, 2, 1, false, 0, false, false, true>(),
+                            prepare_one<PREC_F32, 2, 1, false, 0, false, false, true>(),
                             prepare_one<PREC_F64, 3, 1, false, 0, false, false, true>(),
                             prepare_one<PREC_F32, 3, 1, false, 0, false, false, true>(),
                             prepare_fused<PREC_F64, 0>(),   prepare_fused<PREC_F64, 1>(),
@@ -673,14 +673,16 @@ namespace {
 template <int PREC>
 void residual_prec(const StepArgs& A, const CurvGeom& G, const SteadyArgs& SA, cudaStream_t s) {
   // 32 x 15 tiles on grids of two or more waves of them, 16 x 11 tiles (one wave of four CTAs per SM
-  // covers 107k cells) on the smaller grids; first-order residuals (coarse multigrid levels) on 8 x 6 tiles
-  // while those make up no more than two waves of eight CTAs per SM (about 100k cells)
+  // covers 107k cells) on the smaller grids.  First-order residuals (coarse multigrid levels) on 8 x 6 tiles
+  // while those make up no more than two waves of eight CTAs per SM (about 100k cells), above on 16 x 11: 96k cells
+  // 15.1 us against 15.8 (FP64 394 and 336), 103k 17.1 against 16.2 (420 and 398), 301k 35.7 against 34.0 (1153 and
+  // 965), and on 32 x 15 tiles 20.2, 22.1 and 41.5 (450, 449 and 1077).
   const bool big = A.g.ncell >= 300000;
   if (SA.first_order) {
     if (A.g.ncell < 100000)
       launch_fused<PREC, 3, 1, false, 0, false, false, true>(A, G, s, SA);
     else
-      launch_fused<PREC, 0, 1, false, 0, false, false, true>(A, G, s, SA);
+      launch_fused<PREC, 2, 1, false, 0, false, false, true>(A, G, s, SA);
   } else if (SA.multid) {
     big ? launch_fused<PREC, 0, 1, true>(A, G, s, SA) : launch_fused<PREC, 2, 1, true>(A, G, s, SA);
   } else {
