@@ -457,7 +457,7 @@ gks_status sticky_status(gks_handle* h) {
 // over the shapes, each trial timed with CUDA events; the shape with the fastest trial is kept for
 // the handle and for later handles of the same grid.  A trial is one launch, or on a grid of up to 2^18 cells four
 // launches one after another, as steps are: a launch of 10 to 30 us alone is mostly latency that the next one hides,
-// and picked the second-best shape of a 528 x 136 body-fitted grid (1450 for 1270 us per 96 steps) in one process of six.
+// and picked the second-best shape of a 528 x 136 body-fitted grid (1450 for 1270 us per 97 steps) in one process of six.
 // The key is everything that decides which shapes are candidates, and the grid: arithmetic, expansion, reconstruction
 // and kind of grid (0 rectilinear, 1 body-fitted, 2 with fused transport).  A shape found under it is a candidate.
 using TuneKey = std::array<int, 8>;  // D, n0, n1, n2, arithmetic, multid, recon, kind

@@ -205,7 +205,7 @@ struct CurvTileGeom {
 
 // Limiter of two variables' differences (van Leer on the paired instructions) into s[0], s[1].  The step issues
 // instructions most of its time, and the slopes of a face are 8 to 16 limiters: two at a time, out of states whose
-// values lie together (CellData; alone within 1 us), 96 steps at 528 x 136 took 1349 us before and 1273 after,
+// values lie together (CellData; alone within 1 us), 97 steps at 528 x 136 took 1349 us before and 1273 after,
 // 1056 x 272 3513 and 3354.
 __device__ __forceinline__ void limiter_pair(int lim, F2 a, F2 b, float* s) {
   if (lim == LIM_VANLEER) {

@@ -14,7 +14,7 @@
 // operations per 2D multi-dimensional face and 1193 in 3D (moment tables: 1674 and 2767).  The kernels are bound
 // by their instruction count, in single precision (issue and FP32 pipe about 58% busy) and in double (FP64 pipe 88%
 // busy), so the step times followed: 1024^2 with the double state 122 -> 98 us, 512^2 in FP64 1.88 -> 1.33 ms, 160^3
-// 1.59 -> 1.11 ms (85 us, 1.13 ms and 0.88 ms with the changes noted where they stand).
+// 1.59 -> 1.11 ms (84 us, 1.18 ms and 0.88 ms with the changes noted where they stand).
 #pragma once
 #ifndef GKS_HOST_COUNT
 #include <cuda_runtime.h>
@@ -85,10 +85,9 @@ template <> GKS_FN double g_fma_rn<double>(double a, double b, double c) { retur
 // Quotient and reciprocal: IEEE in double precision (the FP64 path matches the oracle to 1e-12);
 // in single precision the hardware reciprocal (about 1 ulp), which avoids the multi-instruction
 // IEEE sequence and its slow-path branch.  The FP32 form's tolerances are far above this error.  The
-// flush-to-zero instruction: the plain one is wrapped in a range test and two scalings for subnormal divisors,
-// four instructions per quotient where the 1024^2 step executes twenty a face (1024^2 with the double state 91 -> 87.5
-// us per step, WENO-5 at 603 x 501 50 -> 45.8).
-// g_div_full keeps them, for divisors that are a caller's data (epsilon, omega).
+// flush-to-zero form of it needs a normal divisor and is shorter (1024^2 with the double state 91 -> 87.5 us per
+// step, WENO-5 at 603 x 501 50 -> 45.8).  g_div_full takes any divisor, for those that are a caller's data (epsilon, omega,
+// the distances of gks_face_flux).
 template <class T> GKS_FN T g_div(T a, T b) { return a / b; }
 template <class T> GKS_FN T g_rcp(T x) { return T(1) / x; }
 template <class T> GKS_FN T g_div_full(T a, T b) { return a / b; }
@@ -113,8 +112,9 @@ template <> GKS_FN float g_exp<float>(float x) { return __expf(x); }
 // sums of them): the hardware's approximation and one third-order step, r (1 + e + e^2) with e = 1 - x r, and
 // y (1 + h/2 + 3 h^2/8) with h = 1 - x y^2 (the binomial series; Householder's iterations).  Three and five
 // double operations, with no slow path: the FP64 pipe (one warp instruction per 64 clocks and sub-partition) is
-// what the FP64 kernels wait for.  Relative errors at most 1.11e-16 and 1.38e-16 over a
-// million arguments (2^-57 to 2^57).  Quotients that may see zero or infinity keep the IEEE form (g_div).
+// what the FP64 kernels wait for.  The reciprocal is within 0.505 units in the last place (a division within 0.5), the
+// reciprocal square root closer than 1 / sqrt(x) by two IEEE operations, over a million arguments (2^-60 to 2^60).
+// Quotients that may see zero or infinity keep the IEEE form (g_div).
 template <> GKS_FN double g_rcp<double>(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -177,9 +177,11 @@ template <class T> GKS_FN void g_gauss(T x, T& c, T& e) {
 // both ends, is a polynomial of degree 24 in t = (a - 3)/(a + 3) to 1.2e-17: its Chebyshev series on [-1, 1], computed
 // in 60 digits (the mapping of Schonfelder and of Shepherd and Laframboise for this function), its leading coefficient
 // in two parts.  The roundings of a^2, of the polynomial's last step and of the quotient are carried to first order into
-// the last operation, so that of the error little more than the exponential's is left.  With it, the reciprocals above and
-// the inverse widths in the update, the FP64 step takes 1.13 ms instead of 1.34 at 512^2 (k-epsilon, multi-dimensional) and
-// 29.7 us instead of 39.0 on the 400-cell shock tube.
+// the last operation, so that of the error little more than the exponential's is left: relative error of erfc at most
+// 4.0e-16 where it is normal (CUDA's 4.7e-16), 8.1e-17 in the root mean square (9.6e-17).  One exponential, the reciprocals
+// above and the inverse widths in the update took the FP64 step from 1.34 to 1.13 ms at 512^2 (k-epsilon,
+// multi-dimensional) and from 39.0 to 29.7 us on the 400-cell shock tube; of that the corrected quotients took back
+// 23 and 0.6 us, these corrections 17 and 0.4.
 template <> GKS_FN void g_gauss<double>(double x, double& c, double& e) {
   const double m0 = 1.130814990365315, m0l = 1.0122955773236472e-16;
   const double m[24] = {-0.15730767105387838, -0.0142078862510333066, 0.0978158787627484546, -0.0975498893780881991,

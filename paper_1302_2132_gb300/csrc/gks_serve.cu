@@ -320,9 +320,9 @@ void launch_group(gks_server* s, int g, int phase, cudaStream_t st) {
     launch_batch_d2(s->prec, s->var[g], g == GROUP_2D_MULTID, B, s->blocks[g], st);
 }
 
-// Steps of all groups (a multiple of six: the phases start over): the groups share no solve and each counts its own steps, so their launches are
-// branches of the graph that run side by side (a small group's launch leaves most of the chip idle, and an
-// empty one costs its launch latency).  A burst of
+// Steps of all groups (a multiple of six: the phases start over).  The groups share no solve and each counts its own
+// steps, so their launches are branches of the graph that run side by side (a small group's launch leaves most of the
+// chip idle, and an empty one costs its launch latency).  A burst of
 // 16 solves (8 in 1D, 8 in 2D up to 256^2, 40 to 120 steps) 5.66 -> 4.56 ms against one stream for all.
 bool capture_steps(gks_server* s, int steps, cudaGraphExec_t* exec) {
   cudaEvent_t ev[NGROUPS] = {nullptr, nullptr, nullptr};

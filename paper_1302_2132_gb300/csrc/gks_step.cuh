@@ -32,7 +32,7 @@ enum { RECON_MUSCL2 = 0, RECON_MUSCL3 = 1, RECON_WENO5 = 2 };
 __host__ __device__ constexpr int halo_of(int recon) { return recon == RECON_WENO5 ? 3 : 2; }
 constexpr int kMaxWarps = 16;   // largest CTA of any tile variant: 512 threads
 
-// Tile of cells owned by one CTA (variant 0 is the default; 2D has four more, chosen by the
+// Tile of cells owned by one CTA (variant 0 is the default; 1D and 3D have three more, 2D nine, chosen by the
 // autotuner).  Each 2D shape makes the face count of a tile fill whole rounds of its threads:
 // 32x15: 1007 faces / 256 threads, 64x7: 967 / 256, 32x31: 2047 / 512.
 template <int D, int V = 0> struct Tile;
@@ -206,8 +206,8 @@ struct KOmegaArgs {
 template <int PREC> struct PrecT;
 
 // Cell slopes are precomputed in shared memory in 1D, 2D and for the small 3D tiles (variants 1, 2:
-// 256 cells); the 15 slopes per ring cell of the 512-cell 3D tile would hold it to one CTA per SM,
-// so its faces recompute them (two CTAs per SM in FP32).
+// 256 cells, one of which the autotuner picks as a rule); the 15 slopes per ring cell of the 512-cell 3D tile would hold
+// it to one CTA per SM, so its faces recompute them (two CTAs per SM in FP32).
 template <int D, int PREC, int V = 0> __host__ __device__ constexpr bool pre_slopes() { return D < 3 || V > 0; }
 
 // Axis order of the face frame of a face normal to axis ax: the normal first, then the tangential
@@ -437,7 +437,7 @@ __device__ __forceinline__ long field_cell(const DevGrid& g, int D, int i, int j
 // Shared-memory layout of a tile's states, slopes and fluxes: in 2D single precision the four values of a cell or
 // face together, so that one 16-byte access moves them (the step is bound by its instruction count, and its faces and
 // ring cells read whole states); otherwise one plane per variable, also for WENO-5 (H = 3), whose six cells per
-// face then hold too many registers at once (603 x 501: 2131 us per 48 steps in planes, 2271 together).  48 steps in
+// face then hold too many registers at once (603 x 501: 2131 us per 49 steps in planes, 2271 together).  49 steps in
 // double-state form, 1024^2: 4328 us in planes, 4164 together; 1024 x 384: 1959 and 1891.
 template <int D, class R, int H, int N> struct CellData {
   static constexpr bool AOS = D == 2 && sizeof(R) == sizeof(float) && H == 2;
@@ -640,8 +640,9 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 
 // CFL rate of one cell, sum_d (|U_d| + c) / dx_d, c = sqrt(gamma p / rho), from the inverse cell widths, with one
 // reciprocal of the density and one square root.  The step kernel (for its successor) and the rate kernel
-// (for a state that was copied in) take it, every operation rounded as written, so that a run restarted
-// from a copied-out state takes the same time steps to the last bit.
+// (for a state that was copied in) take it, every operation rounded as written, so that an FP64 or float-pair run
+// restarted from a copied-out state takes the same time steps to the last bit.  (With the double state the step
+// adds its increment to the state in float, and the rate kernel rounds the stored sum: the last bit of dt may differ.)
 template <int D, class R>
 __device__ __forceinline__ R cell_rate_inv(const R* w, R gamma, const R* ih) {
   const R ir = g_rcp(w[0]);
@@ -857,7 +858,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
   R* iwx = igz + HZ;  // 1 / width, per axis
   R* iwy = iwx + HX;
   R* iwz = iwy + HY;
-  R* Fs = Ws + G::template fs_offset<R>();  // [nv][NF], 8-byte aligned
+  R* Fs = Ws + G::template fs_offset<R>();  // [nv][NF], 16-byte aligned
   R* Ss = Fs + (size_t)nv * G::NF;          // PRE: [D][nv][NR] limited slopes of the ring cells along each axis
   R* Fl = Ss + (PRE ? (size_t)D * nv * G::NR : 0);  // [2][NR] turbulence fields of the ring cells
   float* Lo = (float*)(Fl + 2 * G::NR);             // PREC_F32: [nv][NC] low words of the tile's cells
@@ -1381,7 +1382,7 @@ __device__ __forceinline__ void step_tile(const StepArgs& A, const int b) {
           R F[nv], tau;
           if constexpr (std::is_same<R, float>::value) {
             // single precision: the two sides of the face on the paired FP32 instructions (in 3D they take
-            // the 128 registers of two CTAs per SM with 8 bytes spilled; 160^3 with the double state
+            // the 128 registers of two CTAs per SM, without spills; 160^3 with the double state
             // 1.08 -> 0.98 ms per step against the scalar sides)
             face_flux_ps_inv<D, MULTID, RAR>(in.wl, in.wr, in.cl, in.cr, in.sl, in.sr, in.tl, in.tr, in.idxl, in.idxr,
                                              in.tau_t, dt, gas, g.abar_t0, F, &tau);
