@@ -272,7 +272,9 @@ GKS_FN Maxw<D, T> maxwellian(const T* w, T ibK) {
     g.U[i] = w[1 + i] * g.ir;
     q += g.U[i] * g.U[i];
   }
-  g.th = (T(2) * w[D + 1] - w[0] * q) * g.ir * ibK;
+  // (2 rho E as a sum, exactly: the two-lane type would round one of two products before their difference)
+  const T e2 = w[D + 1] + w[D + 1];
+  g.th = (e2 - w[0] * q) * g.ir * ibK;
   g.it = g_rcp(g.th);
   return g;
 }
@@ -890,9 +892,9 @@ GKS_FN void face_flux_ps(const float* wl, const float* wr, const In& in, float i
   // Eqs. relaxation time and taua; the artificial part only with C_a > 0
   T tau = gas.mu * g0.it * g0.ir + tau_t;
   if (gas.C_a != T(0)) {
-    const F2 plr = F2(gs.rho * gs.th);
-    const T pl = plr.v.x, pr = plr.v.y;
-    tau += g_div(gas.C_a * g_abs(pr - pl), pr + pl) * dt;
+    // p_r - p_l and p_r + p_l with p_r unrounded
+    const T rr = gs.rho.v.y, tr = gs.th.v.y, pl = gs.rho.v.x * gs.th.v.x;
+    tau += g_div(gas.C_a * g_abs(g_fma_rn(rr, tr, -pl)), g_fma_rn(rr, tr, pl)) * dt;
   }
   *tau_out = tau;
   TimeCoef<T> c;
